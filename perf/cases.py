@@ -575,7 +575,8 @@ def prepare(case, seed):
             P.blob.copy_(poses)  # the step's poses and velocities, handed over in one packed copy
             pl.substeps(case["sub"], 1.0, SUB_DT, form="fused")
 
-        out = _views(pl, False)
+        # what the host code takes back: forces, poses and velocities
+        out = {key: t for key, t in _views(pl, False).items() if key != "n"}
         out.update({key: P.t[key] for key in ("x", "y", "z", "qw", "qx", "qy", "qz", "vx", "vy", "vz", "wx", "wy", "wz")})
         return {"call": _captured(call, True), "out": out, "keep": (pl, poses)}
 
@@ -914,7 +915,7 @@ def _exact_substeps(case, seed):
         mom = inertia(o, parts["w"], ipar, iperp) + dt * t
         parts["q"] = _rotate(parts["q"], dt * inertia(o, mom, 1 / ipar, 1 / iperp))
         parts["w"] = inertia(_axis(parts["q"]), mom, 1 / ipar, 1 / iperp)
-    out = {"force": f.T.contiguous(), "torque": t.T.contiguous(), "pair_i": None, "pair_j": None, "n": n.T.contiguous()}
+    out = {"force": f.T.contiguous(), "torque": t.T.contiguous(), "pair_i": None, "pair_j": None}
     for keys, key in ((("x", "y", "z"), "pos"), (("qw", "qx", "qy", "qz"), "q"), (("vx", "vy", "vz"), "v"),
                       (("wx", "wy", "wz"), "w")):
         out.update({k: parts[key][:, c].contiguous() for c, k in enumerate(keys)})
