@@ -31,13 +31,6 @@
 namespace {
 
 
-__device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
-
-__device__ __forceinline__ float gelu_d_f(float x)
-{
-    return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * expf(-0.5f * x * x) * 0.3989422804014327f;
-}
-
 __device__ __forceinline__ float wrap_pi_f(float x)
 {
     const float tp = 6.283185307179586f;
@@ -56,130 +49,305 @@ __global__ void k_mlp_features(PView P, DView D, const int32_t *__restrict__ pi,
 }
 
 // ---------------------------------------------------------------------------
-// training (FP32)
+// training (FP32): one fused forward/backward kernel, one reduction
 // ---------------------------------------------------------------------------
-constexpr int TS = 32;  // tile edge of the small GEMMs
-
-// Y[m][n] = sum_k X[m][k] W[n][k] + b[n]; Z = Y; H = gelu(Y) if act
-__global__ void k_linear_fwd(const float *__restrict__ X, const float *__restrict__ W, const float *__restrict__ b,
-                             int M, int K, int N, float *__restrict__ Z, float *__restrict__ H, int act)
+// GELU (erf form) and its derivative, from one erf and one exponential
+__device__ __forceinline__ float2 gelu_both(float x)
 {
-    __shared__ float xs[TS][TS + 1], ws[TS][TS + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-    const int m0 = blockIdx.y * TS, n0 = blockIdx.x * TS;
-    float acc[4] = {0, 0, 0, 0};
-    for (int k0 = 0; k0 < K; k0 += TS) {
-        for (int r = ty; r < TS; r += 8) {
-            const int m = m0 + r, k = k0 + tx, n = n0 + r;
-            xs[r][tx] = (m < M && k < K) ? X[(size_t)m * K + k] : 0.f;
-            ws[r][tx] = (n < N && k < K) ? W[(size_t)n * K + k] : 0.f;
-        }
-        __syncthreads();
-        for (int kk = 0; kk < TS; ++kk) {
-            const float wv = ws[tx][kk];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] += xs[ty + 8 * q][kk] * wv;
-        }
-        __syncthreads();
-    }
-    const int n = n0 + tx;
-    if (n >= N) return;
-    for (int q = 0; q < 4; ++q) {
-        const int m = m0 + ty + 8 * q;
-        if (m >= M) continue;
-        const float v = acc[q] + b[n];
-        Z[(size_t)m * N + n] = v;
-        if (act) H[(size_t)m * N + n] = gelu_f(v);
-    }
+    const float c = 0.5f * (1.0f + erff(x * 0.70710678118654752f));
+    return make_float2(x * c, c + x * 0.3989422804014327f * expf(-0.5f * x * x));
 }
 
-// dX[m][k] = sum_n dZ[m][n] W[n][k]   (optionally times gelu'(Zprev[m][k]))
-__global__ void k_linear_bwd_x(const float *__restrict__ dZ, const float *__restrict__ W, int M, int K, int N,
-                               const float *__restrict__ Zprev, float *__restrict__ dX)
+// A block of 256 threads takes tiles of 8 RW rows (samples); the weights, the
+// tile's activations and the derivatives of its GELUs stay in shared memory,
+// and the weight gradients of all its tiles in registers, so a step reads its
+// batch once and writes one partial gradient per block (k_mlp_train_reduce
+// adds them in block order).  Warp w owns rows [RW w, RW w + RW): every product
+// along the rows (z1, z2, y, d2, d1) needs only its own rows, so the warps run
+// without block barriers until the weight gradients, which read all of them.
+// Bound: the FP32 pipe (3.4 MFMA per 64 rows, about 13 us for 64 rows on one
+// SM) and the shared-memory loads that feed it.  In the products with W2 a
+// lane holds RW rows x 4 columns: per four steps of the sum RW broadcast
+// loads and four 16-byte loads for 16 RW multiply-adds.  W2 serves the
+// forward product along its rows (lane's columns lane + 32 j) and the backward
+// one along its columns (4 lane ..): the row stride of 132 floats keeps both,
+// and the activations' rows, free of bank conflicts.  Measured: forward,
+// backward and Adam on 8,192 samples in 44 us, against 1,559 us for one launch
+// per layer and direction (32 x 32 tiles, each weight gradient summed over
+// the whole batch by a single block per tile).
+constexpr int TLD = 132;  // row stride of W2 and the activations (floats)
+
+template <int RW>
+struct TrainSmem {
+    float W2[NH * TLD];
+    float h1[8 * RW * TLD], g1[8 * RW * TLD];  // GELU(z1) and its derivative; g1 becomes d1 = dL/dz1
+    float h2[8 * RW * TLD], d2[8 * RW * TLD];  // GELU(z2); its derivative, then d2 = dL/dz2
+    float W1t[NI * NH];                        // [k][n]
+    float W3[NO * NH];
+    float x[8 * RW * NI];
+    float dy[8 * RW * NO];
+    float b1[NH], b2[NH], b3[NO];
+};
+
+template <int RW>
+__global__ void __launch_bounds__(256, 1) k_mlp_train(const float *__restrict__ params, const float *__restrict__ x,
+                                                      const float *__restrict__ tgt, const float *__restrict__ wgt,
+                                                      int M, float *__restrict__ part, float *__restrict__ lrow)
 {
-    __shared__ float ds[TS][TS + 1], ws[TS][TS + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int m0 = blockIdx.y * TS, k0 = blockIdx.x * TS;
-    float acc[4] = {0, 0, 0, 0};
-    for (int n0 = 0; n0 < N; n0 += TS) {
-        for (int r = ty; r < TS; r += 8) {
-            const int m = m0 + r, n = n0 + tx;
-            ds[r][tx] = (m < M && n < N) ? dZ[(size_t)m * N + n] : 0.f;
-            const int nn = n0 + r, k = k0 + tx;
-            ws[r][tx] = (nn < N && k < K) ? W[(size_t)nn * K + k] : 0.f;
-        }
-        __syncthreads();
-        for (int nn = 0; nn < TS; ++nn) {
-            const float wv = ws[nn][tx];
+    extern __shared__ __align__(16) unsigned char train_raw[];
+    TrainSmem<RW> &S = *reinterpret_cast<TrainSmem<RW> *>(train_raw);
+    constexpr int R = 8 * RW;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int r0 = w * RW;  // this warp's first row of the tile
+    const float *W1 = params, *b1 = W1 + NH * NI, *W2 = b1 + NH, *b2 = W2 + NH * NH, *W3 = b2 + NH, *b3 = W3 + NO * NH;
+    pdl_wait();
+    pdl_trigger();
+    for (int e = tid; e < NH * NH; e += 256) S.W2[(e >> 7) * TLD + (e & 127)] = W2[e];
+    for (int e = tid; e < NH * NI; e += 256) S.W1t[(e % NI) * NH + e / NI] = W1[e];
+    for (int e = tid; e < NO * NH; e += 256) S.W3[e] = W3[e];
+    if (tid < NH) {
+        S.b1[tid] = b1[tid];
+        S.b2[tid] = b2[tid];
+    }
+    if (tid < NO) S.b3[tid] = b3[tid];
+    // this thread's share of the weight gradients, over all the block's tiles:
+    // dW2 rows {4 tn + a, 64 + 4 tn + a} x columns {4 tk + b, 64 + 4 tk + b};
+    // dW3 rows 2 hf, 2 hf + 1 and dW1 columns 6 hf .. of row (column) cn
+    const int tn = tid >> 4, tk = tid & 15, cn = tid & 127, hf = tid >> 7;
+    float g2a[8][8], g3a[2] = {0.f, 0.f}, g1a[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, gba = 0.f, gb3 = 0.f;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] += ds[ty + 8 * q][nn] * wv;
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 8; ++b) g2a[a][b] = 0.f;
+    const float inv_m = 1.0f / (float)M;
+    for (int base = blockIdx.x * R; base < M; base += gridDim.x * R) {
+        __syncthreads();  // the weights are staged; the tile before is used up
+        for (int e = tid; e < R * NI; e += 256) {
+            const int64_t at = (int64_t)base * NI + e;
+            S.x[e] = at < (int64_t)M * NI ? x[at] : 0.f;
         }
         __syncthreads();
+        // layer 1: z1 = x W1^T + b1, columns lane + 32 j
+        {
+            float acc[RW][4];
+#pragma unroll
+            for (int q = 0; q < RW; ++q)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[q][j] = S.b1[lane + 32 * j];
+#pragma unroll
+            for (int k = 0; k < NI; ++k) {
+                float wv[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) wv[j] = S.W1t[k * NH + lane + 32 * j];
+#pragma unroll
+                for (int q = 0; q < RW; ++q) {
+                    const float xv = S.x[(r0 + q) * NI + k];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[q][j] = fmaf(xv, wv[j], acc[q][j]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < RW; ++q)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 g = gelu_both(acc[q][j]);
+                    S.h1[(r0 + q) * TLD + lane + 32 * j] = g.x;
+                    S.g1[(r0 + q) * TLD + lane + 32 * j] = g.y;
+                }
+        }
+        __syncwarp();
+        // layer 2: z2 = h1 W2^T + b2, columns lane + 32 j
+        {
+            float acc[RW][4];
+#pragma unroll
+            for (int q = 0; q < RW; ++q)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[q][j] = S.b2[lane + 32 * j];
+#pragma unroll 2
+            for (int k = 0; k < NH; k += 4) {
+                float4 wv[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    wv[j] = *reinterpret_cast<const float4 *>(&S.W2[(lane + 32 * j) * TLD + k]);
+#pragma unroll
+                for (int q = 0; q < RW; ++q) {
+                    const float4 a = *reinterpret_cast<const float4 *>(&S.h1[(r0 + q) * TLD + k]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        acc[q][j] = fmaf(a.x, wv[j].x, acc[q][j]);
+                        acc[q][j] = fmaf(a.y, wv[j].y, acc[q][j]);
+                        acc[q][j] = fmaf(a.z, wv[j].z, acc[q][j]);
+                        acc[q][j] = fmaf(a.w, wv[j].w, acc[q][j]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < RW; ++q)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 g = gelu_both(acc[q][j]);
+                    S.h2[(r0 + q) * TLD + lane + 32 * j] = g.x;
+                    S.d2[(r0 + q) * TLD + lane + 32 * j] = g.y;
+                }
+        }
+        __syncwarp();
+        // layer 3, the loss, and d2 = (dy W3) gelu'(z2): lane's columns 4 lane ..
+        {
+            float4 w3[NO];
+#pragma unroll
+            for (int o = 0; o < NO; ++o) w3[o] = *reinterpret_cast<const float4 *>(&S.W3[o * NH + 4 * lane]);
+#pragma unroll 1
+            for (int q = 0; q < RW; ++q) {
+                const int m = base + r0 + q;
+                const float4 hv = *reinterpret_cast<const float4 *>(&S.h2[(r0 + q) * TLD + 4 * lane]);
+                float y[NO];
+#pragma unroll
+                for (int o = 0; o < NO; ++o)
+                    y[o] = fmaf(hv.x, w3[o].x, fmaf(hv.y, w3[o].y, fmaf(hv.z, w3[o].z, hv.w * w3[o].w)));
+#pragma unroll
+                for (int s = 16; s; s >>= 1)
+#pragma unroll
+                    for (int o = 0; o < NO; ++o) y[o] += __shfl_xor_sync(0xffffffffu, y[o], s);
+                float dyv[NO] = {0.f, 0.f, 0.f, 0.f};
+                if (m < M) {
+                    float l = 0.f;
+#pragma unroll
+                    for (int o = 0; o < NO; ++o) {
+                        float r = y[o] + S.b3[o] - tgt[(size_t)m * NO + o];
+                        if (o & 1) r = wrap_pi_f(r);
+                        const float wg = wgt ? wgt[(size_t)m * NO + o] : 1.f;
+                        l += 0.5f * wg * r * r;
+                        dyv[o] = wg * r * inv_m;
+                    }
+                    if (lane == 0) lrow[m] = l;
+                }
+                if (lane == 0)
+                    *reinterpret_cast<float4 *>(&S.dy[(r0 + q) * NO]) = make_float4(dyv[0], dyv[1], dyv[2], dyv[3]);
+                float4 *dp = reinterpret_cast<float4 *>(&S.d2[(r0 + q) * TLD + 4 * lane]);
+                float4 g = *dp;
+                g.x *= fmaf(dyv[0], w3[0].x, fmaf(dyv[1], w3[1].x, fmaf(dyv[2], w3[2].x, dyv[3] * w3[3].x)));
+                g.y *= fmaf(dyv[0], w3[0].y, fmaf(dyv[1], w3[1].y, fmaf(dyv[2], w3[2].y, dyv[3] * w3[3].y)));
+                g.z *= fmaf(dyv[0], w3[0].z, fmaf(dyv[1], w3[1].z, fmaf(dyv[2], w3[2].z, dyv[3] * w3[3].z)));
+                g.w *= fmaf(dyv[0], w3[0].w, fmaf(dyv[1], w3[1].w, fmaf(dyv[2], w3[2].w, dyv[3] * w3[3].w)));
+                *dp = g;
+            }
+        }
+        __syncwarp();
+        // d1 = (d2 W2) gelu'(z1): lane's columns 4 lane .., in place of g1
+        {
+            float4 acc[RW];
+#pragma unroll
+            for (int q = 0; q < RW; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+            for (int n = 0; n < NH; n += 4) {
+                float4 wv[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    wv[j] = *reinterpret_cast<const float4 *>(&S.W2[(n + j) * TLD + 4 * lane]);
+#pragma unroll
+                for (int q = 0; q < RW; ++q) {
+                    const float4 a = *reinterpret_cast<const float4 *>(&S.d2[(r0 + q) * TLD + n]);
+                    const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        acc[q].x = fmaf(av[j], wv[j].x, acc[q].x);
+                        acc[q].y = fmaf(av[j], wv[j].y, acc[q].y);
+                        acc[q].z = fmaf(av[j], wv[j].z, acc[q].z);
+                        acc[q].w = fmaf(av[j], wv[j].w, acc[q].w);
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < RW; ++q) {
+                float4 *gp = reinterpret_cast<float4 *>(&S.g1[(r0 + q) * TLD + 4 * lane]);
+                float4 g = *gp;
+                g.x *= acc[q].x;
+                g.y *= acc[q].y;
+                g.z *= acc[q].z;
+                g.w *= acc[q].w;
+                *gp = g;
+            }
+        }
+        __syncthreads();
+        // weight gradients: sums over the tile's rows (rows past the batch have dy = 0)
+#pragma unroll 2
+        for (int m = 0; m < R; ++m) {
+            const float4 p0 = *reinterpret_cast<const float4 *>(&S.d2[m * TLD + 4 * tn]);
+            const float4 p1 = *reinterpret_cast<const float4 *>(&S.d2[m * TLD + 64 + 4 * tn]);
+            const float4 q0 = *reinterpret_cast<const float4 *>(&S.h1[m * TLD + 4 * tk]);
+            const float4 q1 = *reinterpret_cast<const float4 *>(&S.h1[m * TLD + 64 + 4 * tk]);
+            const float pv[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+            const float qv[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+#pragma unroll
+            for (int a = 0; a < 8; ++a)
+#pragma unroll
+                for (int b = 0; b < 8; ++b) g2a[a][b] = fmaf(pv[a], qv[b], g2a[a][b]);
+        }
+#pragma unroll 4
+        for (int m = 0; m < R; ++m) {
+            const float hv = S.h2[m * TLD + cn], dv = S.g1[m * TLD + cn];
+            const float2 d3 = *reinterpret_cast<const float2 *>(&S.dy[m * NO + 2 * hf]);
+            g3a[0] = fmaf(d3.x, hv, g3a[0]);
+            g3a[1] = fmaf(d3.y, hv, g3a[1]);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const float2 xv = *reinterpret_cast<const float2 *>(&S.x[m * NI + 6 * hf + 2 * a]);
+                g1a[2 * a] = fmaf(dv, xv.x, g1a[2 * a]);
+                g1a[2 * a + 1] = fmaf(dv, xv.y, g1a[2 * a + 1]);
+            }
+            gba += hf ? S.d2[m * TLD + cn] : dv;  // db1 (first half of the block), db2
+        }
+        if (tid < NO)
+            for (int m = 0; m < R; ++m) gb3 += S.dy[m * NO + tid];
     }
-    const int k = k0 + tx;
-    if (k >= K) return;
-    for (int q = 0; q < 4; ++q) {
-        const int m = m0 + ty + 8 * q;
-        if (m >= M) continue;
-        float v = acc[q];
-        if (Zprev) v *= gelu_d_f(Zprev[(size_t)m * K + k]);
-        dX[(size_t)m * K + k] = v;
-    }
+    // the block's partial gradient
+    float *out = part + (size_t)blockIdx.x * (NH * NI + NH + NH * NH + NH + NO * NH + NO);
+    float *oW1 = out, *ob1 = oW1 + NH * NI, *oW2 = ob1 + NH, *ob2 = oW2 + NH * NH, *oW3 = ob2 + NH, *ob3 = oW3 + NO * NH;
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 8; ++b)
+            oW2[(4 * tn + (a & 3) + 64 * (a >> 2)) * NH + 4 * tk + (b & 3) + 64 * (b >> 2)] = g2a[a][b];
+    oW3[(2 * hf) * NH + cn] = g3a[0];
+    oW3[(2 * hf + 1) * NH + cn] = g3a[1];
+#pragma unroll
+    for (int a = 0; a < 6; ++a) oW1[cn * NI + 6 * hf + a] = g1a[a];
+    (hf ? ob2 : ob1)[cn] = gba;
+    if (tid < NO) ob3[tid] = gb3;
 }
 
-// dW[n][k] = sum_m dZ[m][n] X[m][k];  db[n] = sum_m dZ[m][n]
-__global__ void k_linear_bwd_w(const float *__restrict__ dZ, const float *__restrict__ X, int M, int K, int N,
-                               float *__restrict__ dW, float *__restrict__ db)
+// grads[e] = the sum of the blocks' partial gradients, in block order: eight
+// threads per parameter group, each an eighth of the blocks, then their sums
+// in order (the same result on every run)
+__global__ void __launch_bounds__(256) k_mlp_train_reduce(const float *__restrict__ part, int nblk, int n,
+                                                          float *__restrict__ grads)
 {
-    __shared__ float ds[TS][TS + 1], xs[TS][TS + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int n0 = blockIdx.y * TS, k0 = blockIdx.x * TS;
-    float acc[4] = {0, 0, 0, 0};
-    float bacc = 0.f;
-    for (int m0 = 0; m0 < M; m0 += TS) {
-        for (int r = ty; r < TS; r += 8) {
-            const int m = m0 + r;
-            ds[r][tx] = (m < M && n0 + tx < N) ? dZ[(size_t)m * N + n0 + tx] : 0.f;
-            xs[r][tx] = (m < M && k0 + tx < K) ? X[(size_t)m * K + k0 + tx] : 0.f;
-        }
-        __syncthreads();
-        for (int mm = 0; mm < TS; ++mm) {
-            const float xv = xs[mm][tx];
+    pdl_wait();
+    pdl_trigger();
+    __shared__ float s[8][32];
+    const int c = threadIdx.x & 31, r = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + c;
+    const int per = (nblk + 7) >> 3, b0 = r * per, b1 = b0 + per < nblk ? b0 + per : nblk;
+    float a = 0.f;
+    if (e < n) {
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) a += part[(size_t)b * n + e];
+    }
+    s[r][c] = a;
+    __syncthreads();
+    if (r == 0 && e < n) {
+        float t = s[0][c];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] += ds[mm][ty + 8 * q] * xv;
-        }
-        if (blockIdx.x == 0 && ty == 0)
-            for (int mm = 0; mm < TS; ++mm) bacc += ds[mm][tx];
-        __syncthreads();
-    }
-    const int k = k0 + tx;
-    for (int q = 0; q < 4; ++q) {
-        const int n = n0 + ty + 8 * q;
-        if (n < N && k < K) dW[(size_t)n * K + k] = acc[q];
-    }
-    if (blockIdx.x == 0 && ty == 0 && n0 + tx < N) db[n0 + tx] = bacc;
-}
-
-// weighted loss terms and dY = w r / M (azimuth errors wrapped); per-row losses to lrow
-__global__ void k_mlp_loss(const float *__restrict__ Y, const float *__restrict__ T, const float *__restrict__ Wt,
-                           int M, float *__restrict__ dY, float *__restrict__ lrow)
-{
-    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
-        float l = 0.f;
-        for (int o = 0; o < NO; ++o) {
-            float r = Y[(size_t)m * NO + o] - T[(size_t)m * NO + o];
-            if (o & 1) r = wrap_pi_f(r);
-            const float wgt = Wt ? Wt[(size_t)m * NO + o] : 1.f;
-            l += 0.5f * wgt * r * r;
-            dY[(size_t)m * NO + o] = wgt * r / (float)M;
-        }
-        lrow[m] = l;
+        for (int q = 1; q < 8; ++q) t += s[q][c];
+        grads[e] = t;
     }
 }
 
 __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v,
                        int n, float lr, float b1, float b2, float eps, float c1, float c2)
 {
+    pdl_wait();
+    pdl_trigger();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const float gk = g[k];
         const float mk = b1 * m[k] + (1.f - b1) * gk;
@@ -555,39 +723,57 @@ int launch_mlp_features(lub_ctx *ctx, const PView &P, const DView &D, const int3
     return lub_check_cuda(ctx, cudaGetLastError(), "k_mlp_features launch");
 }
 
+template <int RW>
+static int launch_train(lub_ctx *ctx, int nblk, const float *params, const float *x, const float *tgt,
+                        const float *wgt, int M, float *part, float *loss_rows, cudaStream_t st)
+{
+    int rc = lub_check_cuda(ctx,
+                            cudaFuncSetAttribute(k_mlp_train<RW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)sizeof(TrainSmem<RW>)),
+                            "shared memory attribute");
+    if (rc) return rc;
+    return lub_check_cuda(ctx,
+                          launch_pdl(k_mlp_train<RW>, nblk, 256, sizeof(TrainSmem<RW>), st, params, x, tgt, wgt, M,
+                                     part, loss_rows),
+                          "mlp forward/backward launch");
+}
+
 int launch_mlp_forward_backward(lub_ctx *ctx, const float *params, const float *x, const float *tgt,
                                 const float *wgt, int M, float *grads, float *work, float *loss_rows, cudaStream_t st)
 {
-    const float *W1 = params, *b1 = W1 + NH * NI, *W2 = b1 + NH, *b2 = W2 + NH * NH, *W3 = b2 + NH, *b3 = W3 + NO * NH;
-    float *gW1 = grads, *gb1 = gW1 + NH * NI, *gW2 = gb1 + NH, *gb2 = gW2 + NH * NH, *gW3 = gb2 + NH,
-          *gb3 = gW3 + NO * NH;
-    // work: z1 h1 z2 h2 [M x 128] each, y dy [M x 4], d2 d1 [M x 128]
-    float *z1 = work, *h1 = z1 + (size_t)M * NH, *z2 = h1 + (size_t)M * NH, *h2 = z2 + (size_t)M * NH;
-    float *y = h2 + (size_t)M * NH, *dy = y + (size_t)M * NO, *d2 = dy + (size_t)M * NO, *d1 = d2 + (size_t)M * NH;
-    const dim3 blk(32, 8);
-    auto grid = [&](int cols, int rows) { return dim3((cols + TS - 1) / TS, (rows + TS - 1) / TS); };
-    k_linear_fwd<<<grid(NH, M), blk, 0, st>>>(x, W1, b1, M, NI, NH, z1, h1, 1);
-    k_linear_fwd<<<grid(NH, M), blk, 0, st>>>(h1, W2, b2, M, NH, NH, z2, h2, 1);
-    k_linear_fwd<<<grid(NO, M), blk, 0, st>>>(h2, W3, b3, M, NH, NO, y, nullptr, 0);
-    k_mlp_loss<<<grid_for(M, 256, ctx ? ctx->num_sms : 152, 8), 256, 0, st>>>(y, tgt, wgt, M, dy, loss_rows);
-    // layer 3
-    k_linear_bwd_w<<<grid(NH, NO), blk, 0, st>>>(dy, h2, M, NH, NO, gW3, gb3);
-    k_linear_bwd_x<<<grid(NH, M), blk, 0, st>>>(dy, W3, M, NH, NO, z2, d2);
-    // layer 2
-    k_linear_bwd_w<<<grid(NH, NH), blk, 0, st>>>(d2, h1, M, NH, NH, gW2, gb2);
-    k_linear_bwd_x<<<grid(NH, M), blk, 0, st>>>(d2, W2, M, NH, NH, z1, d1);
-    // layer 1
-    k_linear_bwd_w<<<grid(NI, NH), blk, 0, st>>>(d1, x, M, NI, NH, gW1, gb1);
-    return lub_check_cuda(ctx, cudaGetLastError(), "mlp forward/backward launch");
+    // rows per block: the fewest (in eights) that cover the batch in one wave
+    // of one block per SM, and whose partial gradients fit the caller's
+    // scratch; larger batches take tiles of 64 rows in turns
+    const int sms = ctx ? ctx->num_sms : 152;
+    const int64_t room = (int64_t)M * LUB_MLP_WORK_PER_SAMPLE / LUB_MLP_PARAMS;
+    const int most = (int)(room < 1 ? 1 : (room < sms ? room : sms));
+    auto fits = [&](int rw) { return ((int64_t)M + 8 * rw - 1) / (8 * rw) <= most; };
+    const int rw = fits(1) ? 1 : fits(2) ? 2 : fits(4) ? 4 : fits(6) ? 6 : fits(7) ? 7 : 8;
+    int64_t nblk = ((int64_t)M + 8 * rw - 1) / (8 * rw);
+    if (nblk > most) nblk = most;
+    // one block writes the gradient itself
+    float *part = nblk > 1 ? work : grads;
+    int rc = rw == 1 ? launch_train<1>(ctx, (int)nblk, params, x, tgt, wgt, M, part, loss_rows, st)
+           : rw == 2 ? launch_train<2>(ctx, (int)nblk, params, x, tgt, wgt, M, part, loss_rows, st)
+           : rw == 4 ? launch_train<4>(ctx, (int)nblk, params, x, tgt, wgt, M, part, loss_rows, st)
+           : rw == 6 ? launch_train<6>(ctx, (int)nblk, params, x, tgt, wgt, M, part, loss_rows, st)
+           : rw == 7 ? launch_train<7>(ctx, (int)nblk, params, x, tgt, wgt, M, part, loss_rows, st)
+                     : launch_train<8>(ctx, (int)nblk, params, x, tgt, wgt, M, part, loss_rows, st);
+    if (rc || nblk == 1) return rc;
+    return lub_check_cuda(ctx,
+                          launch_pdl(k_mlp_train_reduce, (LUB_MLP_PARAMS + 31) / 32, 256, 0, st, (const float *)work,
+                                     (int)nblk, (int)LUB_MLP_PARAMS, grads),
+                          "mlp gradient sum launch");
 }
 
 int launch_mlp_adam(lub_ctx *ctx, float *params, const float *grads, float *m, float *v, int n, int t, float lr,
                     float b1, float b2, float eps, cudaStream_t st)
 {
     const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
-    k_adam<<<grid_for(n, 256, ctx ? ctx->num_sms : 152, 4), 256, 0, st>>>(params, grads, m, v, n, lr, b1, b2, eps, c1,
-                                                                          c2);
-    return lub_check_cuda(ctx, cudaGetLastError(), "mlp adam launch");
+    return lub_check_cuda(ctx,
+                          launch_pdl(k_adam, grid_for(n, 256, ctx ? ctx->num_sms : 152, 4), 256, 0, st, params, grads,
+                                     m, v, n, lr, b1, b2, eps, c1, c2),
+                          "mlp adam launch");
 }
 
 // pack FP32 parameters into the BF16 inference layout owned by the context
