@@ -14,128 +14,194 @@
 // act at the two intersection points, torques about the centres; walls give
 // nothing.
 //
-// One warp per pair; the lanes take the sites of the box where i's extent
-// meets j's extent widened by 2 on every axis (a link, or two, moves a site by
-// at most 2 per axis).  Sites are integer offsets from each centre's integer
-// part, so membership is decided in FP32 from (float) offset - fraction
-// (exact to about 1e-7) with a margin, and again in FP64 inside the margin:
-// every decision is the FP64 one without an FP64 operation per test; the
-// links that qualify are measured in FP64.
+// A warp takes 16 pairs at a time.  What bounds the work is the FP64 pipe (two
+// lanes per clock and SM: one warp instruction costs as much as some 70 on
+// the other pipes), so every FP64 operation runs with all lanes busy, and
+// what need not be FP64 is not:
+//   set-up    the 32 bodies of the 16 pairs, one per lane, into shared memory;
+//   sites     the integer points of the box where i's extent meets j's extent
+//             widened by 2 on every axis (a link, or two, moves a site by at
+//             most 2 per axis), one per lane, as integer offsets from each
+//             centre's integer part: membership is decided in FP32 from
+//             (float) offset - fraction (exact to about 1e-7) with a margin,
+//             and again in FP64 inside the margin, so every decision is the
+//             FP64 one; sites too deep in i or too far from j for any link
+//             are dropped by the norms sqrt(quad) (a step of length s changes
+//             one by at most s / R_min), the rest are gathered;
+//   links     the (site, direction) pairs of the gathered sites, one per lane;
+//             the links that qualify queue up, over all 16 pairs;
+//   measure   32 queued links at a time, one per lane, in FP64, and their
+//             sums per pair, nine components x three thirds of the links, one
+//             per lane, in a fixed order.
+// Measuring across pairs fills the lanes (a pair has some 35 links, so one
+// batch of 32 per pair would be followed by a nearly empty one), and the
+// set-up of one body per lane replaces one by all lanes for every pair.
 #include "lub_internal.cuh"
 
 namespace {
 
 constexpr float kMargin = 1e-4f;  // relative margin of the FP32 membership test
+constexpr int LB = 16;            // pairs per warp and batch (two bodies each: one per lane)
+constexpr int LQ = 64;            // queued links and gathered sites per warp: at most 31 waiting plus 32 new
 
+// A particle at its (image) centre r: what the tests and the measure need.
 struct Body {
     double r[3], o[3];
-    double ia2, ic2;    // 1 / R_perp^2, 1 / R_par^2
-    double Rpar, Rperp;
+    double ia2, dc;     // 1 / R_perp^2, 1 / R_par^2 - 1 / R_perp^2
+    double c2, kk;      // R_par^2, (R_perp^2 - R_par^2) / R_par^2 (curvature)
+    double rr, rq;      // R_par R_perp, R_par / R_perp
+    double v[3], w[3];
     int nint[3];        // floor of the centre (the anchor of the site offsets)
     float f[3];         // centre - floor, in float
-    float of[3], ia2f, dcf;  // axis, 1 / R_perp^2 and 1 / R_par^2 - 1 / R_perp^2 in float
+    float of[3], ia2f, dcf;  // axis, 1 / R_perp^2 and dc in float
+    float half[3];      // half extents along the axes
+    float irmin;        // 1 / the smaller semi-axis
 };
 
-__device__ __forceinline__ Body body_at(const PView &P, int k, const double r[3])
+// one queued link: the site of i (offset from i's anchor) and direction |
+// (links from j's site: 1 or 2) << 8 | pair of the batch << 16
+struct LinkEntry {
+    int m[3];
+    int tag;
+};
+
+struct LinkWarp {
+    Body body[2 * LB];        // pair q: i at 2 q, j at 2 q + 1
+    double res[9][33];        // the measured links' force on i and torques on i and j (rows padded)
+    double acc[3][9][LB];     // their sums per pair, by thirds of the batches
+    LinkEntry queue[LQ];
+    int site[LQ][3];
+    int nl[LB];
+};
+
+__device__ __forceinline__ void body_at(Body &b, const PView &P, int k, const V3<double> &r)
 {
-    Body b;
     const V3<double> o = quat_axis<double>(__ldg(P.qw + k), __ldg(P.qx + k), __ldg(P.qy + k), __ldg(P.qz + k));
-    b.o[0] = o.x;
-    b.o[1] = o.y;
-    b.o[2] = o.z;
-    b.Rpar = __ldg(P.rpar + k);
-    b.Rperp = __ldg(P.rperp + k);
-    b.ia2 = 1.0 / (b.Rperp * b.Rperp);
-    b.ic2 = 1.0 / (b.Rpar * b.Rpar);
+    const float rpar = __ldg(P.rpar + k), rperp = __ldg(P.rperp + k);
+    const double Rpar = rpar, Rperp = rperp;
+    const double ia2 = 1.0 / (Rperp * Rperp), ic2 = 1.0 / (Rpar * Rpar);
+    const double rv[3] = {r.x, r.y, r.z}, ov[3] = {o.x, o.y, o.z};
+    b.ia2 = ia2;
+    b.dc = ic2 - ia2;
+    b.c2 = Rpar * Rpar;
+    b.kk = (Rperp * Rperp - Rpar * Rpar) * ic2;
+    b.rr = Rpar * Rperp;
+    b.rq = Rpar * rcp64(Rperp);
+    const float a2 = rperp * rperp, e = rpar * rpar - a2;
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-        b.r[a] = r[a];
-        const double fl = floor(r[a]);
+        const double fl = floor(rv[a]);
+        const float of = (float)ov[a];
+        b.r[a] = rv[a];
+        b.o[a] = ov[a];
         b.nint[a] = (int)fl;
-        b.f[a] = (float)(r[a] - fl);
-        b.of[a] = (float)b.o[a];
+        b.f[a] = (float)(rv[a] - fl);
+        b.of[a] = of;
+        b.half[a] = sqrtf(fmaxf(a2 + e * of * of, 0.f));
     }
-    b.ia2f = (float)b.ia2;
-    b.dcf = (float)(b.ic2 - b.ia2);
-    return b;
+    b.ia2f = (float)ia2;
+    b.dcf = (float)(ic2 - ia2);
+    b.irmin = 1.0f / fminf(rpar, rperp);
+    b.v[0] = __ldg(P.vx + k);
+    b.v[1] = __ldg(P.vy + k);
+    b.v[2] = __ldg(P.vz + k);
+    b.w[0] = __ldg(P.wx + k);
+    b.w[1] = __ldg(P.wy + k);
+    b.w[2] = __ldg(P.wz + k);
 }
 
 // (x - r)^T M^-1 (x - r) for the site x = floor(r) + m (m: integer offset
 // from the body's anchor), in FP32 from (float) m - frac r, and in FP64
-__device__ __forceinline__ float quad_f(const Body &b, const int m[3])
+__device__ __forceinline__ float quad_f(const Body &b, int m0, int m1, int m2)
 {
-    float u[3];
-    for (int a = 0; a < 3; ++a) u[a] = (float)m[a] - b.f[a];
-    const float ou = b.of[0] * u[0] + b.of[1] * u[1] + b.of[2] * u[2];
-    return (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * b.ia2f + ou * ou * b.dcf;
+    const float u0 = (float)m0 - b.f[0], u1 = (float)m1 - b.f[1], u2 = (float)m2 - b.f[2];
+    const float ou = b.of[0] * u0 + b.of[1] * u1 + b.of[2] * u2;
+    return (u0 * u0 + u1 * u1 + u2 * u2) * b.ia2f + ou * ou * b.dcf;
 }
 
-__device__ __forceinline__ double quad_d(const Body &b, const int m[3])
+__device__ __noinline__ bool inside_d(const Body &b, int m0, int m1, int m2)
 {
+    const int m[3] = {m0, m1, m2};
     double u[3];
     for (int a = 0; a < 3; ++a) u[a] = (double)(b.nint[a] + m[a]) - b.r[a];
     const double ou = b.o[0] * u[0] + b.o[1] * u[1] + b.o[2] * u[2];
-    return (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * b.ia2 + ou * ou * (b.ic2 - b.ia2);
+    return (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * b.ia2 + ou * ou * b.dc <= 1.0;
 }
 
-__device__ __forceinline__ bool inside(const Body &b, const int m[3])
+// membership from the FP32 value q, decided in FP64 inside the margin
+__device__ __forceinline__ bool decide(const Body &b, float q, int m0, int m1, int m2)
 {
-    const float q = quad_f(b, m);
     if (q < 1.0f - kMargin) return true;
     if (q > 1.0f + kMargin) return false;
-    return quad_d(b, m) <= 1.0;
+    return inside_d(b, m0, m1, m2);
 }
 
-// the line x0 + t e (|e| = 1) meets the surface at t_lo <= t_hi (false: misses)
-__device__ __forceinline__ bool line_surface(const Body &b, const double x0[3], const double e[3], double &t_lo,
-                                             double &t_hi)
+__device__ __forceinline__ bool inside(const Body &b, int m0, int m1, int m2)
 {
-    const double u[3] = {x0[0] - b.r[0], x0[1] - b.r[1], x0[2] - b.r[2]};
-    const double ou = b.o[0] * u[0] + b.o[1] * u[1] + b.o[2] * u[2];
-    const double oe = b.o[0] * e[0] + b.o[1] * e[1] + b.o[2] * e[2];
-    const double dc = b.ic2 - b.ia2;
-    const double A = b.ia2 + oe * oe * dc;  // |e| = 1
-    const double B = 2.0 * ((u[0] * e[0] + u[1] * e[1] + u[2] * e[2]) * b.ia2 + ou * oe * dc);
-    const double C = (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * b.ia2 + ou * ou * dc - 1.0;
-    const double disc = B * B - 4.0 * A * C;
+    return decide(b, quad_f(b, m0, m1, m2), m0, m1, m2);
+}
+
+// the 18 nonzero D3Q19 lattice vectors, two bits per component and vector
+// (component + 1): (+-1,0,0), (0,+-1,0), (0,0,+-1), then the face diagonals
+// (+-1,+-1,0), (+-1,0,+-1), (0,+-1,+-1)
+constexpr int kD3Q19[18][3] = {{1, 0, 0},  {-1, 0, 0}, {0, 1, 0},  {0, -1, 0},  {0, 0, 1},  {0, 0, -1},
+                               {1, 1, 0},  {-1, -1, 0}, {1, -1, 0}, {-1, 1, 0},  {1, 0, 1},  {-1, 0, -1},
+                               {1, 0, -1}, {-1, 0, 1},  {0, 1, 1},  {0, -1, -1}, {0, 1, -1}, {0, -1, 1}};
+constexpr unsigned long long d3q19_bits(int a)
+{
+    unsigned long long v = 0;
+    for (int r = 0; r < 18; ++r) v |= (unsigned long long)(kD3Q19[r][a] + 1) << (2 * r);
+    return v;
+}
+__device__ __forceinline__ int d3q19(int r, int a)
+{
+    constexpr unsigned long long bits[3] = {d3q19_bits(0), d3q19_bits(1), d3q19_bits(2)};
+    return (int)((a == 0 ? bits[0] : a == 1 ? bits[1] : bits[2]) >> (2 * r) & 3) - 1;
+}
+
+// c x for c = -1, 0 or 1 on the integer pipe
+__device__ __forceinline__ double times_sign(int c, double x)
+{
+    const int hi = __double2hiint(x) ^ (c & 0x80000000), lo = __double2loint(x);
+    return c ? __hiloint2double(hi, lo) : 0.0;
+}
+
+// The line x0 + t c (c: a lattice vector, |c|^2 = cc) and body b: t of the
+// smaller or larger crossing of its surface, from x0 - r = u; false where it
+// misses.  uxc: u x c.  H: twice the mean curvature at the crossing (radii of
+// curvature of Eq. lub:curvature-radii): with z the crossing's height along
+// the axis and sin^2 p = z^2 / R_par^2, cos^2 p = 1 - sin^2 p on the surface,
+// s1^2 = R_perp^2 sin^2 p + R_par^2 cos^2 p, 1/S1 = R_par R_perp / s1^3 and
+// 1/S2 = R_par / (R_perp s1).
+template <bool LARGER>
+__device__ __forceinline__ bool cross_surface(const Body &b, const double u[3], const int c[3], double &t, double &H,
+                                              double uxc[3])
+{
+    const double o0 = b.o[0], o1 = b.o[1], o2 = b.o[2];
+    const double ou = o0 * u[0] + o1 * u[1] + o2 * u[2];
+    const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    const double oc = times_sign(c[0], o0) + times_sign(c[1], o1) + times_sign(c[2], o2);
+    const double uc = times_sign(c[0], u[0]) + times_sign(c[1], u[1]) + times_sign(c[2], u[2]);
+    const int diag = (c[0] != 0) + (c[1] != 0) + (c[2] != 0) == 2;
+    const double ia2 = b.ia2, dc = b.dc;
+    // |c|^2 / R_perp^2 by the exponent
+    const double ccia2 = __hiloint2double(__double2hiint(ia2) + (diag << 20), __double2loint(ia2));
+    const double dou = dc * ou;
+    const double A = fma(oc * oc, dc, ccia2);
+    const double B = fma(dou, oc, uc * ia2);  // half the linear coefficient
+    const double C = fma(dou, ou, fma(uu, ia2, -1.0));
+    const double disc = fma(B, B, -A * C);
     if (!(disc >= 0.0)) return false;
     const double sq = disc > 0.0 ? disc * rsqrt64(disc) : 0.0;
-    const double i2a = rcp64(2.0 * A);
-    t_lo = (-B - sq) * i2a;
-    t_hi = (-B + sq) * i2a;
+    t = ((LARGER ? sq : -sq) - B) * rcp64(A);
+    const double z = fma(t, oc, ou);
+    const double is1 = rsqrt64(fma(b.kk * z, z, b.c2));
+    H = is1 * fma(b.rr * is1, is1, b.rq);
+    uxc[0] = times_sign(c[2], u[1]) - times_sign(c[1], u[2]);
+    uxc[1] = times_sign(c[0], u[2]) - times_sign(c[2], u[0]);
+    uxc[2] = times_sign(c[1], u[0]) - times_sign(c[0], u[1]);
     return true;
 }
-
-// mean curvature (1/S1 + 1/S2) / 2 at the surface point y (radii of
-// curvature of Eq. lub:curvature-radii, in the body coordinates of y)
-__device__ __forceinline__ double mean_curvature(const Body &b, const double y[3])
-{
-    // with sin p ~ z_b / R_par and cos p ~ rho / R_perp (normalised),
-    // s1^2 = R_perp^2 sin^2 p + R_par^2 cos^2 p; 1/S1 = R_par R_perp / s1^3,
-    // 1/S2 = R_par / (R_perp s1)
-    const double u[3] = {y[0] - b.r[0], y[1] - b.r[1], y[2] - b.r[2]};
-    const double zb = b.o[0] * u[0] + b.o[1] * u[1] + b.o[2] * u[2];
-    const double rho2 = fmax(u[0] * u[0] + u[1] * u[1] + u[2] * u[2] - zb * zb, 0.0);
-    const double sp2 = zb * zb * b.ic2, cp2 = rho2 * b.ia2;
-    const double s1sq = (b.Rperp * b.Rperp * sp2 + b.Rpar * b.Rpar * cp2) * rcp64(sp2 + cp2);
-    const double is1 = rsqrt64(s1sq);
-    return 0.5 * (b.Rpar * b.Rperp * is1 * is1 * is1 + b.Rpar * rcp64(b.Rperp) * is1);
-}
-
-// the 18 nonzero D3Q19 lattice vectors: (+-1,0,0), (0,+-1,0), (0,0,+-1), then
-// the face diagonals (+-1,+-1,0), (+-1,0,+-1), (0,+-1,+-1)
-__constant__ int8_t kD3Q19[18][3] = {{1, 0, 0},  {-1, 0, 0}, {0, 1, 0},  {0, -1, 0},  {0, 0, 1},  {0, 0, -1},
-                                     {1, 1, 0},  {-1, -1, 0}, {1, -1, 0}, {-1, 1, 0},  {1, 0, 1},  {-1, 0, -1},
-                                     {1, 0, -1}, {-1, 0, 1},  {0, 1, 1},  {0, -1, -1}, {0, 1, -1}, {0, -1, 1}};
-
-__device__ __forceinline__ int d3q19(int r, int a) { return kD3Q19[r][a]; }
-
-// a qualifying link: the site of i (offset from i's anchor), the direction,
-// one link (1) or two through a fluid site (2)
-struct LinkEntry {
-    int m[3];
-    int r, kind;
-};
-constexpr int kQueue = 64;  // entries per warp: at most 31 waiting plus 32 new
 
 template <bool ENS>
 __global__ void __launch_bounds__(128) k_links(PView P, const __grid_constant__ DView D0, Ens E,
@@ -146,157 +212,238 @@ __global__ void __launch_bounds__(128) k_links(PView P, const __grid_constant__ 
 {
     pdl_wait();
     pdl_trigger();
-    __shared__ LinkEntry link_queue[4 * kQueue];
+    extern __shared__ __align__(16) unsigned char links_raw[];
+    LinkWarp &W = reinterpret_cast<LinkWarp *>(links_raw)[threadIdx.x >> 5];
     const int count = pair_count(d_count, cap);
     const size_t C = (size_t)cap;
     const int lane = threadIdx.x & 31;
+    const unsigned FULL = 0xffffffffu, below = (1u << lane) - 1u;
     const int nwarp = (gridDim.x * blockDim.x) >> 5;
-    for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < count; k += nwarp) {
-        const int i = __ldg(pi + k), j = __ldg(pj + k);
-        double F[3] = {0, 0, 0}, Ti[3] = {0, 0, 0}, Tj[3] = {0, 0, 0};
-        int nl = 0;
-        bool alien = false;
-        const DView &D = pair_domain<ENS>(D0, E, i, j, &alien);
-        const bool ok = !alien && i >= 0 && i < P.n && j >= 0 && j < P.n && i != j &&
-                        shape_ok(__ldg(P.rpar + i), __ldg(P.rperp + i)) &&
-                        shape_ok(__ldg(P.rpar + j), __ldg(P.rperp + j));
-        if (ok) {
-            const V3<double> ri = load_pos(P, i);
-            const V3<double> d = min_image(D, sub(load_pos(P, j), ri));
-            const double rir[3] = {ri.x, ri.y, ri.z}, rjr[3] = {ri.x + d.x, ri.y + d.y, ri.z + d.z};
-            const Body bi = body_at(P, i, rir), bj = body_at(P, j, rjr);
-            const double vi[3] = {__ldg(P.vx + i), __ldg(P.vy + i), __ldg(P.vz + i)};
-            const double wi[3] = {__ldg(P.wx + i), __ldg(P.wy + i), __ldg(P.wz + i)};
-            const double vj[3] = {__ldg(P.vx + j), __ldg(P.vy + j), __ldg(P.vz + j)};
-            const double wj[3] = {__ldg(P.wx + j), __ldg(P.wy + j), __ldg(P.wz + j)};
-            // sites of i's box within 2 (per axis) of j's box, as offsets m from
-            // i's anchor (the same site is m + dij from j's)
-            int lo[3], n[3], dij[3];
-            int nsites = 1;
-            for (int a = 0; a < 3; ++a) {
-                const double wa = sqrt(bi.Rperp * bi.Rperp + (bi.Rpar * bi.Rpar - bi.Rperp * bi.Rperp) * bi.o[a] * bi.o[a]);
-                const double wb = sqrt(bj.Rperp * bj.Rperp + (bj.Rpar * bj.Rpar - bj.Rperp * bj.Rperp) * bj.o[a] * bj.o[a]);
-                const double l = fmax(ceil(rir[a] - wa), ceil(rjr[a] - wb - 2.0 - 1e-9));
-                const double h = fmin(floor(rir[a] + wa), floor(rjr[a] + wb + 2.0 + 1e-9));
-                lo[a] = (int)l - bi.nint[a];
-                n[a] = h >= l ? (int)(h - l) + 1 : 0;
-                nsites *= n[a];
-                dij[a] = bi.nint[a] - bj.nint[a];
+    const double pre = -3.0 * qbar * mu;
+    for (int64_t k0 = (int64_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * LB; k0 < count;
+         k0 += (int64_t)nwarp * LB) {
+        const int np = (int)(count - k0 < LB ? count - k0 : LB);
+        // the bodies: lane 2 q takes i of pair q, lane 2 q + 1 takes j
+        unsigned valid;
+        {
+            const int q = lane >> 1;
+            bool ok = false;
+            if (q < np) {
+                const int i = __ldg(pi + k0 + q), j = __ldg(pj + k0 + q);
+                bool alien = false;
+                const DView &D = pair_domain<ENS>(D0, E, i, j, &alien);
+                ok = !alien && i >= 0 && i < P.n && j >= 0 && j < P.n && i != j &&
+                     shape_ok(__ldg(P.rpar + i), __ldg(P.rperp + i)) && shape_ok(__ldg(P.rpar + j), __ldg(P.rperp + j));
+                if (ok) {
+                    V3<double> r = load_pos(P, i);
+                    if (lane & 1) r = add(r, min_image(D, sub(load_pos(P, j), r)));
+                    body_at(W.body[lane], P, lane & 1 ? j : i, r);
+                }
             }
-            // Qualifying links go to a per-warp queue and are measured 32 at a
-            // time, one per lane: they cluster on a few sites, and measuring
-            // them where they are found would run the FP64 code with most
-            // lanes idle.
-            auto measure = [&](const LinkEntry &en) {
-                const int c0 = d3q19(en.r, 0), c1 = d3q19(en.r, 1), c2 = d3q19(en.r, 2);
-                const double cr = en.r < 6 ? 1.0 : 1.4142135623730951, icr = en.r < 6 ? 1.0 : 0.7071067811865476;
-                const double e[3] = {c0 * icr, c1 * icr, c2 * icr};
-                const double x0[3] = {(double)(bi.nint[0] + en.m[0] - en.kind * c0),
-                                      (double)(bi.nint[1] + en.m[1] - en.kind * c1),
-                                      (double)(bi.nint[2] + en.m[2] - en.kind * c2)};
-                double tjl, tjh, til, tih;
-                if (!line_surface(bj, x0, e, tjl, tjh) || !line_surface(bi, x0, e, til, tih)) return;
-                const double hs = til - tjh;
-                if (!(hs > 0.0 && hs < cr)) return;
-                double pI[3], pJ[3], aI[3], aJ[3];
+            valid = __ballot_sync(FULL, ok);
+            for (int e = lane; e < 3 * 9 * LB; e += 32) (&W.acc[0][0][0])[e] = 0.0;
+            if (lane < LB) W.nl[lane] = 0;
+        }
+        __syncwarp();
+        int queued = 0;  // links waiting (warp-uniform)
+        // measures the first min(32, queued) entries of the queue and moves the rest to the front
+        auto measure = [&]() {
+            __syncwarp();
+            const int n = queued < 32 ? queued : 32;
+            const LinkEntry en = W.queue[lane];
+            const LinkEntry nx = W.queue[32 + lane];
+            __syncwarp();
+            if (lane < queued - 32) W.queue[lane] = nx;
+            double F[3] = {0, 0, 0}, Ti[3] = {0, 0, 0}, Tj[3] = {0, 0, 0};
+            const int pr = lane < n ? en.tag >> 16 : 0;
+            if (lane < n) {
+                const Body &bi = W.body[2 * pr], &bj = W.body[2 * pr + 1];
+                const int r = en.tag & 255, kind = (en.tag >> 8) & 255;
+                const int c[3] = {d3q19(r, 0), d3q19(r, 1), d3q19(r, 2)};
+                double ui[3], uj[3];
+#pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    pI[a] = x0[a] + til * e[a];
-                    pJ[a] = x0[a] + tjh * e[a];
-                    aI[a] = pI[a] - rir[a];
-                    aJ[a] = pJ[a] - rjr[a];
+                    const double x0 = (double)(bi.nint[a] + en.m[a] - kind * c[a]);
+                    ui[a] = x0 - bi.r[a];
+                    uj[a] = x0 - bj.r[a];
                 }
-                double dv[3];
-                dv[0] = (vi[0] + wi[1] * aI[2] - wi[2] * aI[1]) - (vj[0] + wj[1] * aJ[2] - wj[2] * aJ[1]);
-                dv[1] = (vi[1] + wi[2] * aI[0] - wi[0] * aI[2]) - (vj[1] + wj[2] * aJ[0] - wj[0] * aJ[2]);
-                dv[2] = (vi[2] + wi[0] * aI[1] - wi[1] * aI[0]) - (vj[2] + wj[0] * aJ[1] - wj[1] * aJ[0]);
-                const double lam = 0.5 * (mean_curvature(bi, pI) + mean_curvature(bj, pJ));
-                const double icr2 = en.r < 6 ? 1.0 : 0.5;
-                const double coef = -1.5 * qbar * mu * icr2 * rcp64(lam) * (rcp64(hs * hs) - icr2) *
-                                    (e[0] * dv[0] + e[1] * dv[1] + e[2] * dv[2]);
-                const double df[3] = {coef * e[0], coef * e[1], coef * e[2]};
-                F[0] += df[0];
-                F[1] += df[1];
-                F[2] += df[2];
-                Ti[0] += aI[1] * df[2] - aI[2] * df[1];
-                Ti[1] += aI[2] * df[0] - aI[0] * df[2];
-                Ti[2] += aI[0] * df[1] - aI[1] * df[0];
-                Tj[0] -= aJ[1] * df[2] - aJ[2] * df[1];
-                Tj[1] -= aJ[2] * df[0] - aJ[0] * df[2];
-                Tj[2] -= aJ[0] * df[1] - aJ[1] * df[0];
-                ++nl;
-            };
-            LinkEntry *queue = link_queue + (threadIdx.x >> 5) * kQueue;
-            int queued = 0;  // warp-uniform
-            auto drain = [&]() {  // measure the first 32 entries, move the rest to the front
-                __syncwarp();
-                const LinkEntry en = queue[lane];
-                __syncwarp();
-                if (lane < queued - 32) queue[lane] = queue[32 + lane];
-                __syncwarp();
-                measure(en);
-                queued -= 32;
-            };
-            for (int q0 = 0; q0 < nsites; q0 += 32) {
-                const int q = q0 + lane;
-                int mi[3] = {0, 0, 0};
-                bool site = false;
-                if (q < nsites) {
-                    mi[0] = lo[0] + q % n[0];
-                    mi[1] = lo[1] + (q / n[0]) % n[1];
-                    mi[2] = lo[2] + q / (n[0] * n[1]);
-                    site = inside(bi, mi);
+                double ti, tj, Hi, Hj, xi[3], xj[3];
+                const bool mi = cross_surface<false>(bi, ui, c, ti, Hi, xi);
+                const bool mj = cross_surface<true>(bj, uj, c, tj, Hj, xj);
+                const double tau = ti - tj;  // h* / c_r
+                if (mi && mj && tau > 0.0 && tau < 1.0) {
+                    // c.(v_i + w_i x a_i - v_j - w_j x a_j), with c.(w x a) = w.(a x c) = w.(u x c)
+                    const double cv = times_sign(c[0], bi.v[0] - bj.v[0]) + times_sign(c[1], bi.v[1] - bj.v[1]) +
+                                      times_sign(c[2], bi.v[2] - bj.v[2]) + bi.w[0] * xi[0] + bi.w[1] * xi[1] +
+                                      bi.w[2] * xi[2] - bj.w[0] * xj[0] - bj.w[1] * xj[1] - bj.w[2] * xj[2];
+                    // df = -3 qbar mu / (2 c_r^2 lambda) (c/c_r) (c/c_r . dv) (1/h*^2 - 1/c_r^2),
+                    // lambda = (H_i + H_j) / 4, h* = tau c_r
+                    const double t2 = tau * tau;
+                    double s = 2.0 * pre * cv * (1.0 - t2) * rcp64((Hi + Hj) * t2);
+                    if (r >= 6) s *= 0.125;  // c_r^6 = 8
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        F[a] = times_sign(c[a], s);
+                        Ti[a] = s * xi[a];
+                        Tj[a] = -s * xj[a];
+                    }
+                    atomicAdd(&W.nl[pr], 1);
                 }
-                for (int r = 0; r < 18; ++r) {
-                    int kind = 0;
-                    if (site) {
+            }
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                W.res[a][lane] = F[a];
+                W.res[3 + a][lane] = Ti[a];
+                W.res[6 + a][lane] = Tj[a];
+            }
+            __syncwarp();
+            const int part = lane / 9, comp = lane - 9 * part;
+            const int e0 = part * 11, e1 = part < 2 ? e0 + 11 : 32;
+            int cur = -1;
+            double run = 0.0;
+            for (int e = 0; e < 11; ++e) {
+                const int at = e0 + e < e1 ? e0 + e : 31;
+                const int p = __shfl_sync(FULL, pr, at);
+                if (part < 3 && e0 + e < e1 && e0 + e < n) {
+                    if (p != cur) {
+                        if (cur >= 0) W.acc[part][comp][cur] += run;
+                        cur = p;
+                        run = 0.0;
+                    }
+                    run += W.res[comp][at];
+                }
+            }
+            if (cur >= 0) W.acc[part][comp][cur] += run;
+            __syncwarp();
+            queued -= n;
+        };
+        for (int q = 0; q < np; ++q) {
+            if (!((valid >> (2 * q)) & 1u)) continue;
+            const Body &bi = W.body[2 * q], &bj = W.body[2 * q + 1];
+            // the box of sites as offsets m from i's anchor (the same site is
+            // m + dij from j's); 1e-3 outward for the FP32 half extents
+            int lo[3], nn[3], dij[3];
+            int nsites = 1;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                dij[a] = bi.nint[a] - bj.nint[a];
+                const int l = max((int)ceilf(bi.f[a] - bi.half[a] - 1e-3f),
+                                  (int)ceilf(bj.f[a] - bj.half[a] - 2.001f) - dij[a]);
+                const int h = min((int)floorf(bi.f[a] + bi.half[a] + 1e-3f),
+                                  (int)floorf(bj.f[a] + bj.half[a] + 2.001f) - dij[a]);
+                lo[a] = l;
+                nn[a] = max(h - l + 1, 0);
+                nsites *= nn[a];
+            }
+            if (nsites <= 0) continue;
+            // a site that ends a link is in i within sqrt(2) of a site outside
+            // i, and within 2 sqrt(2) of a site of j
+            const float deep = fmaxf(1.0f - 1.4143f * bi.irmin, 0.f), far = 1.0f + 2.8286f * bj.irmin;
+            const float qi_min = deep * deep * (1.0f - kMargin) - kMargin, qj_max = far * far * (1.0f + kMargin) + kMargin;
+            const int n0 = nn[0], n01 = nn[0] * nn[1];
+            const float in0 = 1.0f / (float)n0, in01 = 1.0f / (float)n01;
+            int ns = 0;  // gathered sites (warp-uniform)
+            // the links of the first min(32, ns) gathered sites
+            auto links_of = [&]() {
+                __syncwarp();
+                const int n = ns < 32 ? ns : 32;
+                const int total = 18 * n;
+                for (int e0 = 0; e0 < total; e0 += 32) {
+                    const int e = e0 + lane;
+                    int kind = 0, m0 = 0, m1 = 0, m2 = 0, r = 0;
+                    if (e < total) {
+                        const int sidx = (e * 3641) >> 16;  // e / 18 for e < 576
+                        r = e - 18 * sidx;
+                        m0 = W.site[sidx][0];
+                        m1 = W.site[sidx][1];
+                        m2 = W.site[sidx][2];
                         const int c0 = d3q19(r, 0), c1 = d3q19(r, 1), c2 = d3q19(r, 2);
-                        const int y1[3] = {mi[0] - c0, mi[1] - c1, mi[2] - c2};
-                        const int y1b[3] = {y1[0] + dij[0], y1[1] + dij[1], y1[2] + dij[2]};
-                        const bool y1i = inside(bi, y1), y1j = inside(bj, y1b);
-                        if (y1j && !y1i) {
-                            kind = 1;
-                        } else if (!y1j && !y1i) {
-                            const int y2[3] = {mi[0] - 2 * c0, mi[1] - 2 * c1, mi[2] - 2 * c2};
-                            const int y2b[3] = {y2[0] + dij[0], y2[1] + dij[1], y2[2] + dij[2]};
-                            if (inside(bj, y2b) && !inside(bi, y2)) kind = 2;
+                        const int a0 = m0 - c0, a1 = m1 - c1, a2 = m2 - c2;
+                        if (!inside(bi, a0, a1, a2)) {
+                            if (inside(bj, a0 + dij[0], a1 + dij[1], a2 + dij[2])) {
+                                kind = 1;
+                            } else {
+                                const int b0 = a0 - c0, b1 = a1 - c1, b2 = a2 - c2;
+                                if (inside(bj, b0 + dij[0], b1 + dij[1], b2 + dij[2]) && !inside(bi, b0, b1, b2))
+                                    kind = 2;
+                            }
                         }
                     }
-                    const unsigned hit = __ballot_sync(0xffffffffu, kind != 0);
+                    const unsigned hit = __ballot_sync(FULL, kind != 0);
                     if (!hit) continue;
                     if (kind) {
-                        LinkEntry &en = queue[queued + __popc(hit & ((1u << lane) - 1u))];
-                        en.m[0] = mi[0];
-                        en.m[1] = mi[1];
-                        en.m[2] = mi[2];
-                        en.r = r;
-                        en.kind = kind;
+                        LinkEntry &en = W.queue[queued + __popc(hit & below)];
+                        en.m[0] = m0;
+                        en.m[1] = m1;
+                        en.m[2] = m2;
+                        en.tag = r | kind << 8 | q << 16;
                     }
                     queued += __popc(hit);
-                    if (queued >= 32) drain();
+                    if (queued >= 32) measure();
                 }
+                // the rest to the front
+                __syncwarp();
+                int s0 = 0, s1 = 0, s2 = 0;
+                const bool mv = lane < ns - 32;
+                if (mv) {
+                    s0 = W.site[32 + lane][0];
+                    s1 = W.site[32 + lane][1];
+                    s2 = W.site[32 + lane][2];
+                }
+                __syncwarp();
+                if (mv) {
+                    W.site[lane][0] = s0;
+                    W.site[lane][1] = s1;
+                    W.site[lane][2] = s2;
+                }
+                ns -= n;
+            };
+            for (int q0 = 0; q0 < nsites; q0 += 32) {
+                const int e = q0 + lane;
+                int m0 = 0, m1 = 0, m2 = 0;
+                bool site = false;
+                if (e < nsites) {
+                    // e = (z n1 + y) n0 + x by FP32 quotients, corrected to the exact ones
+                    int z = (int)((float)e * in01);
+                    int rem = e - z * n01;
+                    if (rem < 0) { --z; rem += n01; }
+                    if (rem >= n01) { ++z; rem -= n01; }
+                    int y = (int)((float)rem * in0);
+                    int x = rem - y * n0;
+                    if (x < 0) { --y; x += n0; }
+                    if (x >= n0) { ++y; x -= n0; }
+                    m0 = lo[0] + x;
+                    m1 = lo[1] + y;
+                    m2 = lo[2] + z;
+                    const float qi = quad_f(bi, m0, m1, m2);
+                    site = qi >= qi_min && qi <= 1.0f + kMargin &&
+                           quad_f(bj, m0 + dij[0], m1 + dij[1], m2 + dij[2]) <= qj_max && decide(bi, qi, m0, m1, m2);
+                }
+                const unsigned hit = __ballot_sync(FULL, site);
+                if (site) {
+                    int *s = W.site[ns + __popc(hit & below)];
+                    s[0] = m0;
+                    s[1] = m1;
+                    s[2] = m2;
+                }
+                ns += __popc(hit);
+                if (ns >= 32) links_of();
             }
-            // the rest: one per lane
-            __syncwarp();
-            if (lane < queued) measure(queue[lane]);
-            __syncwarp();
+            if (ns > 0) links_of();
         }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            for (int a = 0; a < 3; ++a) {
-                F[a] += __shfl_xor_sync(0xffffffffu, F[a], o);
-                Ti[a] += __shfl_xor_sync(0xffffffffu, Ti[a], o);
-                Tj[a] += __shfl_xor_sync(0xffffffffu, Tj[a], o);
+        while (queued > 0) measure();
+        __syncwarp();
+        // rows of consecutive pairs: lane = pair (half warps take alternate rows)
+        const int q = lane & (LB - 1), row0 = lane / LB;
+        if (q < np) {
+            for (int row = row0; row < 9; row += 32 / LB) {
+                const double v = W.acc[0][row][q] + W.acc[1][row][q] + W.acc[2][row][q];
+                double *dst = row < 3 ? force + row * C : torque + (row - 3) * C;
+                dst[k0 + q] = v;
             }
-            nl += __shfl_xor_sync(0xffffffffu, nl, o);
+            if (nlinks && row0 == 0) nlinks[k0 + q] = W.nl[q];
         }
-        if (lane == 0) {
-            for (int a = 0; a < 3; ++a) {
-                force[a * C + k] = F[a];
-                torque[a * C + k] = Ti[a];
-                torque[(3 + a) * C + k] = Tj[a];
-            }
-            if (nlinks) nlinks[k] = nl;
-        }
+        __syncwarp();  // the batch's shared memory is reused
     }
 }
 
@@ -308,15 +455,22 @@ int launch_links(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E, con
 {
     if (cap == 0) return LUB_OK;
     const int block = 128;
-    const int64_t warps = cap;
-    int64_t grid = (warps * 32 + block - 1) / block;
+    const size_t smem = (block / 32) * sizeof(LinkWarp);
+    static_assert(4 * sizeof(LinkWarp) <= 113 * 1024, "two blocks fit an SM");
+    const int warps = block / 32;
+    int64_t grid = ((int64_t)cap + LB * warps - 1) / (LB * warps);
     if (grid > 64 * (int64_t)ctx->num_sms) grid = 64 * (int64_t)ctx->num_sms;
+    int rc = lub_check_cuda(ctx,
+                            cudaFuncSetAttribute(E.nb ? k_links<true> : k_links<false>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                            "shared memory attribute");
+    if (rc) return rc;
     cudaError_t e;
     if (E.nb)
-        e = launch_pdl(k_links<true>, (int)grid, block, 0, st, P, D, E, pi, pj, d_count, cap, mu, qbar, force, torque,
+        e = launch_pdl(k_links<true>, (int)grid, block, smem, st, P, D, E, pi, pj, d_count, cap, mu, qbar, force, torque,
                        nlinks);
     else
-        e = launch_pdl(k_links<false>, (int)grid, block, 0, st, P, D, E, pi, pj, d_count, cap, mu, qbar, force,
+        e = launch_pdl(k_links<false>, (int)grid, block, smem, st, P, D, E, pi, pj, d_count, cap, mu, qbar, force,
                        torque, nlinks);
     return lub_check_cuda(ctx, e, "k_links launch");
 }
