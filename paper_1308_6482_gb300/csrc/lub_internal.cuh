@@ -220,28 +220,52 @@ __device__ __forceinline__ V3<T> axpy(T s, const V3<T> &a, const V3<T> &b)  // s
     return mk<T>(s * a.x + b.x, s * a.y + b.y, s * a.z + b.z);
 }
 
-// Double-precision reciprocal and reciprocal square root by Newton-Raphson
-// from an FP32 seed (x_{k+1} = x_k (2 - a x_k) and y_{k+1} = y_k (3 - a y_k^2)/2;
-// two steps take the seed's ~2^-22 relative error below double rounding).
-// GB300's FP64 pipe is about 60 times slower than FP32, and these use a
-// handful of FP64 multiply-adds where a full-precision division or square
-// root takes several times more.  Inputs are positive, normal and within the
-// float range here (squared lengths, shape factors, determinants).
+// Conversions between double and float on the integer pipe.  GB300 issues one
+// FP64 warp instruction per 19 clocks and SM, and the conversions use that
+// pipe too (17 clocks), so one costs as much as some seventy integer
+// instructions.
+// The double of a float, exactly (float subnormals give zero).
+__device__ __forceinline__ double widen_bits(float f)
+{
+    const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+    unsigned hi = (m >> 3) + (m < 0x7f800000u ? 0x38000000u : 0x70000000u);
+    unsigned lo = b << 29;
+    if (m < 0x00800000u) hi = lo = 0u;
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo);
+}
+
+// Double-precision reciprocal and reciprocal square root: an FP32 seed from
+// the argument's mantissa (its exponent handled by integer operations, so the
+// whole double range is covered and nothing is converted) and one third-order
+// step.  With the residual e = 1 - a x (1 - a y^2), of order 2^-22 (the seed
+// and its truncated argument), 1/(1 - e) = 1 + e + e^2 + ... and (1 - e)^(-1/2)
+// = 1 + e/2 + 3 e^2/8 + ... leave an error of order e^3 = 2^-66, below double
+// rounding, in 3 and 5 FP64 operations (two Newton-Raphson steps with
+// converted seeds took 6 and 9).  A zero argument gives infinity or a huge
+// value, a negative square root NaN.
 __device__ __forceinline__ double rcp64(double a)
 {
-    double x = (double)__frcp_rn((float)a);
-    x = x * fma(-a, x, 2.0);
-    x = x * fma(-a, x, 2.0);
-    return x;
+    const int hi = __double2hiint(a), k = (hi >> 20 & 0x7ff) - 1023;
+    // m = |a| 2^-k in [1, 2) as a float
+    const float m = __uint_as_float(((unsigned)(hi & 0xfffff) << 3) | 0x3f800000u | ((unsigned)__double2loint(a) >> 29));
+    const unsigned f = __float_as_uint(__frcp_rn(m));
+    const double x = __hiloint2double((int)((f >> 3) + 0x38000000u - ((unsigned)k << 20)) | (hi & (int)0x80000000u),
+                                      (int)(f << 29));
+    const double e = fma(-a, x, 1.0);
+    return fma(x, fma(e, e, e), x);
 }
 
 __device__ __forceinline__ double rsqrt64(double a)
 {
-    double y = (double)rsqrtf((float)a);
-    const double h = 0.5 * a;
-    y = y * fma(-h * y, y, 1.5);
-    y = y * fma(-h * y, y, 1.5);
-    return y;
+    const int hi = __double2hiint(a), k = ((hi >> 20) - 1023) >> 1;
+    // m = a 4^-k in [1, 4) as a float
+    const unsigned mh = (unsigned)hi - ((unsigned)k << 21) - 0x38000000u;
+    const float m = __uint_as_float((mh << 3) | ((unsigned)__double2loint(a) >> 29));
+    const unsigned f = __float_as_uint(rsqrtf(m));
+    const int yh = (int)((f >> 3) + 0x38000000u - ((unsigned)k << 20));
+    const double y = __hiloint2double(hi < 0 ? 0x7ff80000 : yh, (int)(f << 29));
+    const double e = fma(-(a * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // Reciprocal and square root of the FP32 resistance path: the hardware
