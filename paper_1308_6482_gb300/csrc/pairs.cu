@@ -115,6 +115,7 @@ struct BuildView {
     float rmax_bound;
     int32_t cap;
     int64_t ncell_total;  // cells of all grids (the cell counts hold one more entry)
+    int32_t sweep_tiles, sweep_rows;  // the sweep's blocks per pass over the slots, and rows per block (see there)
     int2 *und;            // candidates left to the FP64 test (in the cell index storage, free after the fill)
     int32_t und_cap;
 };
@@ -388,6 +389,9 @@ constexpr int SC = 32;        // candidates a group stages per round
 constexpr float kFar = 1e18f;  // x of an unused staging entry: fails every test
 constexpr int kNone = 1 << 30;
 
+// up to this many particles the sweep takes one row per block
+constexpr int64_t kSweepSplitMax = 200000;
+
 template <bool B>
 struct BoolTag {
     static constexpr bool value = B;
@@ -521,6 +525,13 @@ static_assert(sizeof(SweepWarp) % 16 == 0, "warp blocks stay 16-byte aligned");
 // the FP64 test's registers in the sweep's loop, where they cost spills
 // (the sweep ran 10 % faster without it).
 
+//
+// Rows: a block takes V.rows of the five rows of its slots (blocks [b tiles,
+// (b + 1) tiles) rows [b rows, (b + 1) rows)).  Large inputs take all five in
+// one block: the group's set-up is then paid once, and the blocks fill the
+// GPU anyway.  Small ones take one row per block: the rows are a chain of
+// dependent loads (cell starts, records, staged tests), and with a few
+// hundred blocks in all nothing else hides their latency.
 template <bool ENS>
 __device__ __forceinline__ void sweep_groups(const BuildView &V)
 {
@@ -548,7 +559,9 @@ __device__ __forceinline__ void sweep_groups(const BuildView &V)
     // this warp's part of the block's dynamic shared memory
     extern __shared__ float4 sweep_smem[];
     SweepWarp &W = reinterpret_cast<SweepWarp *>(sweep_smem)[wq];
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const int part = blockIdx.x / V.sweep_tiles;
+    const int s = (blockIdx.x - part * V.sweep_tiles) * blockDim.x + threadIdx.x;
+    const int row_first = part * V.sweep_rows;
     const int s0w = s - lane;
     const bool valid = s < N;
     // the full test and the store of queue entry e (the candidate's record
@@ -582,32 +595,34 @@ __device__ __forceinline__ void sweep_groups(const BuildView &V)
         cc = own.y;
         const int cy = (cc >> 10) & 1023, cz = cc >> 20;
         colkey = cell_base<ENS>(EG, b) + (cz * G.nc[1] + cy) * G.nc[0];  // first cell of the column
-        // plane walls: the gap dir (z - z_w) - sigma(e_z) in FP32 from the
+        pidx = own.x;
+        // (the blocks of the first rows) plane walls: the gap dir (z - z_w) - sigma(e_z) in FP32 from the
         // records (z - z_w in float-float), decided in FP64 only within the
         // margin (the exact test costs some 60 FP64 operations)
-        const int i = own.x;
-        pidx = i;
-        const float rm2 = a0.w * a0.w;
-        const float sz = sqrt_fast(fmaxf((a1.w > 0.f ? rm2 - a1.w : rm2) + a1.w * a1.z * a1.z, 0.f));
-        int wf = 0, bits = 0;
-        // z - z_w in float-float from the bits of both (no FP64 pipe)
-        const ff zf = ff_split_bits_nan(P.z[i]);
-        for (int ww = 0; ww < D.n_walls; ++ww) {
-            const ff dzw = ff_sub(zf, ff_split_bits_nan(D.wall_z[ww]));
-            const float hw = (float)D.wall_dir[ww] * (dzw.hi + dzw.lo) - sz;
-            bool in = hw < G.cutoff - G.margin;
-            if (!in && hw <= G.cutoff + G.margin) {
-                const Shape<double> si = load_shape<double>(P, i);
-                in = (double)D.wall_dir[ww] * (P.z[i] - D.wall_z[ww]) - support(si, mk<double>(0.0, 0.0, 1.0)) <
-                     cutoff_d;
+        if (row_first == 0) {
+            const int i = own.x;
+            const float rm2 = a0.w * a0.w;
+            const float sz = sqrt_fast(fmaxf((a1.w > 0.f ? rm2 - a1.w : rm2) + a1.w * a1.z * a1.z, 0.f));
+            int wf = 0, bits = 0;
+            // z - z_w in float-float from the bits of both (no FP64 pipe)
+            const ff zf = ff_split_bits_nan(P.z[i]);
+            for (int ww = 0; ww < D.n_walls; ++ww) {
+                const ff dzw = ff_sub(zf, ff_split_bits_nan(D.wall_z[ww]));
+                const float hw = (float)D.wall_dir[ww] * (dzw.hi + dzw.lo) - sz;
+                bool in = hw < G.cutoff - G.margin;
+                if (!in && hw <= G.cutoff + G.margin) {
+                    const Shape<double> si = load_shape<double>(P, i);
+                    in = (double)D.wall_dir[ww] * (P.z[i] - D.wall_z[ww]) - support(si, mk<double>(0.0, 0.0, 1.0)) <
+                         cutoff_d;
+                }
+                if (in) {
+                    bits |= 1 << ww;
+                    ++wf;
+                }
             }
-            if (in) {
-                bits |= 1 << ww;
-                ++wf;
-            }
+            cnt[N + i] = wf;
+            wbits[i] = (uint8_t)bits;
         }
-        cnt[N + i] = wf;
-        wbits[i] = (uint8_t)bits;
     }
     const int cx = cc & 1023;
     float4 *const cg = &W.cand[g * (SC + 1)];
@@ -648,7 +663,7 @@ __device__ __forceinline__ void sweep_groups(const BuildView &V)
             W.ownw[lane] = make_float2(a0.w, marg);
             W.own_i[lane] = pidx;
         }
-        for (int row = 0; row < SWEEP_ROWS; ++row) {
+        for (int row = row_first; row < row_first + V.sweep_rows; ++row) {
             int dy, dz;
             row_offsets(row, dy, dz);
             int yc = lcy + dy, zc = lcz + dz;
@@ -1166,7 +1181,9 @@ int build_core(lub_ctx *ctx, int num_sms, void *scratch, const Grid &G, const PV
     if ((rc = lub_check_cuda(ctx, e, "cells fill launch"))) return rc;
     // one slot per thread (no grid-stride loop)
     Shape2 sw = tuned_shape(ctx, LUB_TUNE_SWEEP, N);
-    sw.grid = (int)((N + sw.block - 1) / sw.block);
+    V.sweep_tiles = (int)((N + sw.block - 1) / sw.block);
+    V.sweep_rows = N <= kSweepSplitMax ? 1 : SWEEP_ROWS;
+    sw.grid = V.sweep_tiles * (SWEEP_ROWS / V.sweep_rows);
     lub_trace_mark(ctx, LUB_TRACE_SWEEP, st);
     e = launch_pdl(k_pairs_sweep<ENS>, sw.grid, sw.block, (size_t)(sw.block / 32) * sizeof(SweepWarp), st, V);
     lub_trace_mark(ctx, LUB_TRACE_SWEEP, st);
