@@ -14,11 +14,11 @@
 // act at the two intersection points, torques about the centres; walls give
 // nothing.
 //
-// A warp takes 16 pairs at a time.  What bounds the work is the FP64 pipe (two
+// A warp takes 8 pairs at a time.  What bounds the work is the FP64 pipe (two
 // lanes per clock and SM: one warp instruction costs as much as some 70 on
 // the other pipes), so every FP64 operation runs with all lanes busy, and
 // what need not be FP64 is not:
-//   set-up    the 32 bodies of the 16 pairs, one per lane, into shared memory;
+//   set-up    the 16 bodies of the 8 pairs, one per lane, into shared memory;
 //   sites     the integer points of the box where i's extent meets j's extent
 //             widened by 2 on every axis (a link, or two, moves a site by at
 //             most 2 per axis), one per lane, as integer offsets from each
@@ -29,7 +29,7 @@
 //             are dropped by the norms sqrt(quad) (a step of length s changes
 //             one by at most s / R_min), the rest are gathered;
 //   links     the (site, direction) pairs of the gathered sites, one per lane;
-//             the links that qualify queue up, over all 16 pairs;
+//             the links that qualify queue up, over all 8 pairs;
 //   measure   32 queued links at a time, one per lane, in FP64, and their
 //             sums per pair, nine components x three thirds of the links, one
 //             per lane, in a fixed order.
@@ -40,8 +40,7 @@
 
 namespace {
 
-constexpr float kMargin = 1e-4f;  // relative margin of the FP32 membership test
-constexpr int LB = 16;            // pairs per warp and batch (two bodies each: one per lane)
+constexpr int LB = 8;             // pairs per warp and batch (two bodies each: one per lane)
 constexpr int LQ = 64;            // queued links and gathered sites per warp: at most 31 waiting plus 32 new
 
 // A particle at its (image) centre r: what the tests and the measure need.
@@ -56,6 +55,7 @@ struct Body {
     float of[3], ia2f, dcf;  // axis, 1 / R_perp^2 and dc in float
     float half[3];      // half extents along the axes
     float irmin;        // 1 / the smaller semi-axis
+    float margin;       // of the FP32 membership test (decide)
 };
 
 // one queued link: the site of i (offset from i's anchor) and direction |
@@ -78,7 +78,7 @@ __device__ __forceinline__ void body_at(Body &b, const PView &P, int k, const V3
 {
     const V3<double> o = quat_axis<double>(__ldg(P.qw + k), __ldg(P.qx + k), __ldg(P.qy + k), __ldg(P.qz + k));
     const float rpar = __ldg(P.rpar + k), rperp = __ldg(P.rperp + k);
-    const double Rpar = rpar, Rperp = rperp;
+    const double Rpar = widen_bits(rpar), Rperp = widen_bits(rperp);
     const double ia2 = 1.0 / (Rperp * Rperp), ic2 = 1.0 / (Rpar * Rpar);
     const double rv[3] = {r.x, r.y, r.z}, ov[3] = {o.x, o.y, o.z};
     b.ia2 = ia2;
@@ -102,12 +102,14 @@ __device__ __forceinline__ void body_at(Body &b, const PView &P, int k, const V3
     b.ia2f = (float)ia2;
     b.dcf = (float)(ic2 - ia2);
     b.irmin = 1.0f / fminf(rpar, rperp);
-    b.v[0] = __ldg(P.vx + k);
-    b.v[1] = __ldg(P.vy + k);
-    b.v[2] = __ldg(P.vz + k);
-    b.w[0] = __ldg(P.wx + k);
-    b.w[1] = __ldg(P.wy + k);
-    b.w[2] = __ldg(P.wz + k);
+    const float ratio = fmaxf(rpar, rperp) * b.irmin;
+    b.margin = 8e-6f * (1.0f + ratio * ratio) + 1e-6f * ratio * b.irmin;
+    b.v[0] = widen_bits(__ldg(P.vx + k));
+    b.v[1] = widen_bits(__ldg(P.vy + k));
+    b.v[2] = widen_bits(__ldg(P.vz + k));
+    b.w[0] = widen_bits(__ldg(P.wx + k));
+    b.w[1] = widen_bits(__ldg(P.wy + k));
+    b.w[2] = widen_bits(__ldg(P.wz + k));
 }
 
 // (x - r)^T M^-1 (x - r) for the site x = floor(r) + m (m: integer offset
@@ -128,11 +130,15 @@ __device__ __noinline__ bool inside_d(const Body &b, int m0, int m1, int m2)
     return (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * b.ia2 + ou * ou * b.dc <= 1.0;
 }
 
-// membership from the FP32 value q, decided in FP64 inside the margin
+// membership from the FP32 value q, decided in FP64 inside the margin: the
+// terms of quad_f are of order ratio^2 (|u|^2 / R_perp^2 against a negative
+// (o.u)^2 dc for a prolate), each within a few 2^-24 of its value, so q is
+// within some 20 2^-24 (1 + ratio^2) of the exact one, and the fraction's
+// rounding adds 2^-23 ratio / R_min; the margin is six to eight times that
 __device__ __forceinline__ bool decide(const Body &b, float q, int m0, int m1, int m2)
 {
-    if (q < 1.0f - kMargin) return true;
-    if (q > 1.0f + kMargin) return false;
+    if (q < 1.0f - b.margin) return true;
+    if (q > 1.0f + b.margin) return false;
     return inside_d(b, m0, m1, m2);
 }
 
@@ -157,6 +163,12 @@ __device__ __forceinline__ int d3q19(int r, int a)
 {
     constexpr unsigned long long bits[3] = {d3q19_bits(0), d3q19_bits(1), d3q19_bits(2)};
     return (int)((a == 0 ? bits[0] : a == 1 ? bits[1] : bits[2]) >> (2 * r) & 3) - 1;
+}
+
+// the double of an integer below 2^24 in magnitude, off the FP64 pipe
+__device__ __forceinline__ double small_int(int m)
+{
+    return abs(m) < (1 << 24) ? widen_bits((float)m) : (double)m;
 }
 
 // c x for c = -1, 0 or 1 on the integer pipe
@@ -204,7 +216,7 @@ __device__ __forceinline__ bool cross_surface(const Body &b, const double u[3], 
 }
 
 template <bool ENS>
-__global__ void __launch_bounds__(128) k_links(PView P, const __grid_constant__ DView D0, Ens E,
+__global__ void __launch_bounds__(128, 4) k_links(PView P, const __grid_constant__ DView D0, Ens E,
                                                const int32_t *__restrict__ pi, const int32_t *__restrict__ pj,
                                                const int32_t *__restrict__ d_count, int32_t cap, double mu,
                                                double qbar, double *__restrict__ force, double *__restrict__ torque,
@@ -263,7 +275,7 @@ __global__ void __launch_bounds__(128) k_links(PView P, const __grid_constant__ 
                 double ui[3], uj[3];
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    const double x0 = (double)(bi.nint[a] + en.m[a] - kind * c[a]);
+                    const double x0 = small_int(bi.nint[a] + en.m[a] - kind * c[a]);
                     ui[a] = x0 - bi.r[a];
                     uj[a] = x0 - bj.r[a];
                 }
@@ -339,7 +351,7 @@ __global__ void __launch_bounds__(128) k_links(PView P, const __grid_constant__ 
             // a site that ends a link is in i within sqrt(2) of a site outside
             // i, and within 2 sqrt(2) of a site of j
             const float deep = fmaxf(1.0f - 1.4143f * bi.irmin, 0.f), far = 1.0f + 2.8286f * bj.irmin;
-            const float qi_min = deep * deep * (1.0f - kMargin) - kMargin, qj_max = far * far * (1.0f + kMargin) + kMargin;
+            const float qi_min = deep * deep - 2.0f * bi.margin, qj_max = far * far * (1.0f + 2.0f * bj.margin);
             const int n0 = nn[0], n01 = nn[0] * nn[1];
             const float in0 = 1.0f / (float)n0, in01 = 1.0f / (float)n01;
             int ns = 0;  // gathered sites (warp-uniform)
@@ -416,7 +428,7 @@ __global__ void __launch_bounds__(128) k_links(PView P, const __grid_constant__ 
                     m1 = lo[1] + y;
                     m2 = lo[2] + z;
                     const float qi = quad_f(bi, m0, m1, m2);
-                    site = qi >= qi_min && qi <= 1.0f + kMargin &&
+                    site = qi >= qi_min && qi <= 1.0f + bi.margin &&
                            quad_f(bj, m0 + dij[0], m1 + dij[1], m2 + dij[2]) <= qj_max && decide(bi, qi, m0, m1, m2);
                 }
                 const unsigned hit = __ballot_sync(FULL, site);
