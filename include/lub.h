@@ -403,15 +403,17 @@ int lub_resistance_apply(lub_ctx *ctx, const lub_particles *p, const lub_domain 
  *     calls up to rounding (the same arithmetic, which the compiler may
  *     contract into multiply-adds differently inside the one kernel; the
  *     particle sums also add in another order).
- *   - LUB_MIXED: the kernels of lub_closest_points followed by those of
- *     lub_resistance_apply, on one set of per-call particle records (built
- *     once instead of once per call); the results are those of the two calls,
- *     the particle sums up to the order of the atomic additions.
+ *   - LUB_MIXED: on one set of per-call particle records (built once instead
+ *     of once per call), for capacities up to 1.6 million pairs and without
+ *     the network one pass as in LUB_FP64, else the kernels of
+ *     lub_closest_points followed by those of lub_resistance_apply; the
+ *     results are those of the two calls up to rounding, the particle sums up
+ *     to the order of the atomic additions.
  * n [3][cap] is required: it holds the start normals of a warm start
  * (LUB_WARM_PREVIOUS, LUB_WARM_MLP_ALL, LUB_WARM_MLP) and receives the
  * normals.  gap, status, iters, FT and lever are written where given and
- * skipped where NULL (in LUB_MIXED the context scratch holds gap and status
- * between the kernels when they are NULL).  force and torque [3][n] (float in
+ * skipped where NULL (in the two-kernel form of LUB_MIXED the context scratch
+ * holds them between the kernels).  force and torque [3][n] (float in
  * LUB_MIXED, double in LUB_FP64) are zeroed first unless accumulate is set.
  * Ensemble mode as for the separate calls.
  */
@@ -510,11 +512,11 @@ int lub_random_motion(lub_ctx *ctx, const lub_particles *p, uint64_t seed, int64
  * are persistent grid-stride loops; their shape is (threads per block, blocks
  * per SM), the grid being min(work / block, blocks_per_sm x SMs).
  * ------------------------------------------------------------------------- */
-#define LUB_TUNE_CLOSEST_MIXED 0   /* lub_closest_points, LUB_MIXED, FP32 stage */
+#define LUB_TUNE_CLOSEST_MIXED 0   /* lub_closest_points, LUB_MIXED, FP32 stage; lub_correct's one pass */
 #define LUB_TUNE_CLOSEST_REFINE 1  /* lub_closest_points, LUB_MIXED, work list of FP64 solves */
 #define LUB_TUNE_CLOSEST_FP64 2    /* lub_closest_points, LUB_FP64 */
 #define LUB_TUNE_RESISTANCE 3      /* lub_resistance, lub_resistance_apply (and so
-                                      lub_correct in LUB_MIXED) */
+                                      lub_correct's two-kernel form) */
 #define LUB_TUNE_APPLY 4           /* lub_apply, atomic form */
 #define LUB_TUNE_SWEEP 5           /* lub_pairs_build, the cell sweep (one thread per
                                       particle slot: only the block counts, the grid
@@ -545,7 +547,8 @@ int lub_set_launch_shape(lub_ctx *ctx, int32_t kernel, int32_t block, int32_t bl
  * support for per-kernel rooflines.
  * ------------------------------------------------------------------------- */
 #define LUB_TRACE_SWEEP      0  /* lub_pairs_build: the cell sweep (k_pairs_sweep) */
-#define LUB_TRACE_CLOSEST    1  /* lub_closest_points: the solve (FP32 stage, FP64 or learned kernel) */
+#define LUB_TRACE_CLOSEST    1  /* lub_closest_points: the solve (FP32 stage, FP64 or learned kernel);
+                                    lub_correct's one pass in LUB_MIXED */
 #define LUB_TRACE_RESISTANCE 2  /* lub_resistance / lub_resistance_apply: the pair-force kernel */
 #define LUB_TRACE_APPLY      3  /* lub_apply: the scatter kernel */
 #define LUB_TRACE_COUNT      4

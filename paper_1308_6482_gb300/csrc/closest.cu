@@ -174,6 +174,17 @@ __device__ __forceinline__ double wall_gap(const PView &P, const DView &D, int i
 // per-pair solves, shared by the separate kernels and the fused pass
 // ---------------------------------------------------------------------------
 constexpr int kNoEntry = 0x7fffffff;
+// Largest capacity of a pair list that lub_correct takes in one pass
+// (k_fused_mixed) in mixed precision.  One pass saves two launches, the
+// records' second read and the normals' and gaps' way through memory, some
+// 15 us in all; two kernels of 64 and 72 registers keep more warps in flight
+// than one of 96, which is worth 13 us per million pairs.  Measured: 60.4 ->
+// 55.8 us (step, 65k pairs), 238 -> 231 us (0.6M pairs, ensemble), 828 -> 893
+// us (4.4M pairs): level near 1.2 million pairs, and capacities are usually a
+// third above the count.
+constexpr int kFusedMax = 1600000;
+// blocks of 128 threads per SM that the one-pass kernel's registers allow for
+constexpr int kFusedBlocks = 5;
 
 // The FP32 stage's finish for a particle pair, in float-float on the FP32
 // pipe (GB300 runs FP64 at 1/74 of the FP32 rate): the gap at the FP32 Newton
@@ -835,6 +846,91 @@ __global__ void __launch_bounds__(128) k_fused_fp64(PView P, const __grid_consta
     }
 }
 
+// One pass of the mixed mode (lub_correct, without the network): each pair's
+// closest points and gap, resistance and scatter by the same thread, the
+// normal and gap staying in registers in float-float.  The pairs of a block
+// whose FP32 Newton did not converge are gathered in shared memory and solved
+// in FP64 by its first lanes before the block goes on, so that a few such
+// pairs cost one FP64 solve per block and not one per warp.
+template <bool ENS>
+__global__ void __launch_bounds__(128, kFusedBlocks) k_fused_mixed(
+    PView P, const __grid_constant__ DView D0, Ens E, const __grid_constant__ RParams R,
+    const int32_t *__restrict__ pi, const int32_t *__restrict__ pj, const int32_t *__restrict__ d_count, int32_t cap,
+    double *__restrict__ nout, double *__restrict__ gap, uint8_t *__restrict__ status, uint8_t *__restrict__ iters,
+    float *__restrict__ FT, float *__restrict__ lever, int maxit, float tol32, int warm, float *__restrict__ force,
+    float *__restrict__ torque, const float2 *__restrict__ pff)
+{
+    pdl_wait();
+    pdl_trigger();
+    __shared__ int redo[128], nredo;
+    const int count = pair_count(d_count, cap);
+    const size_t C = (size_t)cap;
+    if (threadIdx.x == 0) nredo = 0;
+    __syncthreads();
+    // block-uniform loop bound: the warps take part in the scatter, the block in the second solve
+    for (int base = blockIdx.x * blockDim.x; base < count; base += gridDim.x * blockDim.x) {
+        const int k = base + threadIdx.x;
+        int i = -1, j = -1, st = LUB_ST_DEGENERATE;
+        float ci[6] = {0, 0, 0, 0, 0, 0}, cj[6] = {0, 0, 0, 0, 0, 0};
+        bool again = false;
+        if (k < count) {
+            i = __ldg(pi + k);
+            j = __ldg(pj + k);
+            V3<double> n64;
+            double h;
+            ff nf[3], hf;
+            int nit;
+            again = closest_mixed_one<ENS>(P, D0, E, pff, i, j, k, nout, C, warm, maxit, tol32, n64, h, nf, hf, st,
+                                           nit) != kNoEntry;
+            if (again) {
+                redo[atomicAdd(&nredo, 1)] = k;
+                i = j = -1;
+            } else {
+                // (the normal and gap before the force: fewer live values)
+                nout[k] = n64.x;
+                nout[C + k] = n64.y;
+                nout[2 * C + k] = n64.z;
+                if (gap) gap[k] = h;
+                if (iters) iters[k] = (uint8_t)(nit > 255 ? 255 : nit);
+                float out[12];
+                pair_force_ff(R, i, j, nf, hf, st, out, pff);
+                store_force(FT, lever, C, k, out);
+                if (status) status[k] = (uint8_t)st;
+                side_contrib(out, 0, ci);
+                if (j >= 0) side_contrib(out, 1, cj);
+            }
+        }
+        const bool ok = !again && !(st & LUB_ST_DEGENERATE);
+        scatter_warp<float>(ok ? i : -1, ok ? j : -1, (size_t)P.n, ci, cj, force, torque);
+        if (__syncthreads_or(again)) {
+            const int m = nredo;
+            for (int q0 = 0; q0 < m; q0 += blockDim.x) {
+                const int q = q0 + threadIdx.x;
+                i = j = -1;
+                if (q < m) {
+                    const int kk = redo[q];
+                    i = __ldg(pi + kk);
+                    j = __ldg(pj + kk);
+                    V3<double> n64;
+                    double h;
+                    int nit;
+                    refine_one<ENS>(P, D0, E, i, j, maxit, n64, h, st, nit);
+                    float out[12];
+                    pair_force<float>(P, R, i, j, n64, h, st, out, pff);
+                    store_force(FT, lever, C, kk, out);
+                    store_pair(nout, gap, status, iters, C, kk, n64, h, st, nit);
+                    side_contrib(out, 0, ci);
+                    side_contrib(out, 1, cj);
+                }
+                scatter_warp<float>(i, j, (size_t)P.n, ci, cj, force, torque);
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) nredo = 0;
+            __syncthreads();
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
@@ -991,6 +1087,23 @@ int launch_correct_t(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E,
         // the kernels of lub_closest_points, then those of lub_resistance_apply
         // on the same per-call particle records (built once; their kernel also
         // clears the sums unless accumulate is set)
+        if (prm.warm_start != LUB_WARM_MLP && prm.warm_start != LUB_WARM_MLP_ALL && cap <= kFusedMax) {
+            // small lists: the records, then one pass over the pairs
+            if ((rc = lub_ensure_scratch(ctx, particles_ff_bytes(P.n)))) return rc;
+            float2 *pff = (float2 *)ctx->scratch;
+            if ((rc = launch_particles_ff(ctx, P, pff, st, nullptr, accumulate ? nullptr : (float *)force,
+                                          accumulate ? nullptr : (float *)torque)))
+                return rc;
+            const RParams R = make_rparams(prm);
+            const Shape2 sh = tuned_shape(ctx, LUB_TUNE_CLOSEST_MIXED, cap);
+            lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
+            (void)launch_pdl(k_fused_mixed<ENS>, sh.grid, sh.block, 0, st, P, D, E, R, pi, pj, d_count, cap, n, gap,
+                             status, iters, (float *)FT, (float *)lever, prm.max_newton, (float)prm.newton_tol,
+                             (int)(prm.warm_start == LUB_WARM_PREVIOUS), (float *)force, (float *)torque,
+                             (const float2 *)pff);
+            lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
+            return lub_check_cuda(ctx, cudaGetLastError(), "one-pass launch");
+        }
         ClosestKeep keep;
         if ((rc = launch_closest_t<ENS>(ctx, P, D, E, prm, pi, pj, d_count, cap, n, gap, status, iters, st, &keep,
                                         accumulate ? nullptr : (float *)force,
