@@ -29,7 +29,8 @@
 //   * pairs whose FP32 Newton did not converge are appended to a compacted
 //     work list (one atomic per warp) and solved again in FP64 by a second
 //     kernel, so only full warps of such pairs use the slow FP64 pipe.
-// LUB_FP64: the whole solve and gap in double.
+// LUB_FP64: the iterations in FP32 and float-float, the gap and the last step
+// in double (solve_ff, finish_fp64).
 #include "ff.cuh"
 #include "lub_mlp.cuh"
 #include "mlp_infer.cuh"
@@ -408,7 +409,252 @@ __device__ __forceinline__ void refine_one(const PView &P, const DView &D0, cons
     if (h <= 0.0) st |= LUB_ST_OVERLAP;
 }
 
-// LUB_FP64: the whole solve and gap of pair k in double
+// ---------------------------------------------------------------------------
+// LUB_FP64: the Newton iterations on the FP32 pipe, the result in FP64
+// ---------------------------------------------------------------------------
+// One FP64 warp instruction costs as much as some seventy FP32 ones here, and
+// Newton's early iterations need no FP64: the FP64 iteration's own steps are
+// reproduced well enough by FP32 ones (while a step is long) and by
+// float-float ones (near the end), and one FP64 evaluation of the gap and its
+// gradient at the float-float normal (good to ~1e-12 rad) gives a last step
+// that leaves ~1e-16 rad, and the FP64 gap.  About 100 FP64 instructions a
+// pair, set-up included, instead of some 110 an iteration.
+//
+// The iteration count stays that of the FP64 iteration (which stops after
+// the first step below kTolFp64), without running it: its steps are followed
+// to a relative 1e-6 or so (the Hessian is FP32) once the iterate is held in
+// float-float, so the count can differ only where a step lies within that of
+// kTolFp64.  Such pairs, and any solve that does not go straight down
+// (halved steps, an indefinite Hessian, more than max_newton iterations), are
+// solved again by the FP64 iteration itself (newton_sphere<double>).
+
+// One Newton step from the float normal n (|n| = 1 to FP32) with the gradient
+// in float-float, as in polish_gap_ff but for steps of any length: m the
+// stepped unit normal in float-float, s2 the step's squared length.  False
+// where the Hessian is not positive definite.
+__device__ __forceinline__ bool newton_step_ff(const ff d[3], const ff oi[3], const ff oj[3], float api, float cpi,
+                                               float apj, float cpj, const V3<float> n, ff m[3], float &s2)
+{
+    const ff a2i = two_prod(api, api), ei = ff_sub(two_prod(cpi, cpi), a2i);
+    const ff a2j = two_prod(apj, apj), ej = ff_sub(two_prod(cpj, cpj), a2j);
+    const float nv[3] = {n.x, n.y, n.z};
+    const ff nn = ff_dot3_exact(nv, nv);
+    const ff ci = ff_dot3f_c(oi, nv), cj = ff_dot3f_c(oj, nv);
+    const ff ri = ff_rsqrt(ff_add(ff_mul(a2i, nn), ff_mul(ei, ff_mul(ci, ci))));
+    const ff rj = ff_rsqrt(ff_add(ff_mul(a2j, nn), ff_mul(ej, ff_mul(cj, cj))));
+    const ff bi = ff_mul(ff_mul(ei, ci), ri), bj = ff_mul(ff_mul(ej, cj), rj);
+    ff Rp[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) Rp[a] = ff_sub(ff_sub(d[a], ff_mul(bi, oi[a])), ff_mul(bj, oj[a]));
+    const ff nRp = ff_dot3f_c(Rp, nv);
+    // R_t = R' - (n.R' / |n|^2) n, exactly normal to n, rounded once formed
+    const ff in = ff_rsqrt(nn);
+    const ff lam = ff_mul(nRp, ff_mul(in, in));
+    float Rt[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const ff t = ff_sub(Rp[a], ff_mulf(lam, nv[a]));
+        Rt[a] = __fadd_rn(t.hi, t.lo);
+    }
+    const V3<float> t1 = perp_unit(n), t2 = cross(n, t1);
+    const float G1 = t1.x * Rt[0] + t1.y * Rt[1] + t1.z * Rt[2];
+    const float G2 = t2.x * Rt[0] + t2.y * Rt[1] + t2.z * Rt[2];
+    const V3<float> ofi = mk<float>(oi[0].hi, oi[1].hi, oi[2].hi), ofj = mk<float>(oj[0].hi, oj[1].hi, oj[2].hi);
+    const float u1i = dot(ofi, t1), u2i = dot(ofi, t2), u1j = dot(ofj, t1), u2j = dot(ofj, t2);
+    const float Ai = a2i.hi * ri.hi, Aj = a2j.hi * rj.hi;
+    const float gf = nRp.hi - Ai - Aj;
+    const float Ei = ei.hi * ri.hi * ri.hi, Ej = ej.hi * rj.hi * rj.hi;
+    const float P11 = Ai * (1.f + Ei * u1i * u1i) + Aj * (1.f + Ej * u1j * u1j) + gf;
+    const float P22 = Ai * (1.f + Ei * u2i * u2i) + Aj * (1.f + Ej * u2j * u2j) + gf;
+    const float P12 = Ai * Ei * u1i * u2i + Aj * Ej * u1j * u2j;
+    const float det = P11 * P22 - P12 * P12;
+    if (!(P11 > 0.f && det > 0.f)) return false;
+    const float idet = rcp_fast(det);
+    float s1 = (P22 * G1 - P12 * G2) * idet, sb = (P11 * G2 - P12 * G1) * idet;
+    s2 = s1 * s1 + sb * sb;
+    if (s2 > 0.25f) {
+        const float f = 0.5f * rsqrtf(s2);
+        s1 *= f;
+        sb *= f;
+    }
+    const float tv1[3] = {t1.x, t1.y, t1.z}, tv2[3] = {t2.x, t2.y, t2.z};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) m[a] = two_sum(nv[a], __fmaf_rn(s1, tv1[a], __fmul_rn(sb, tv2[a])));
+    const ff im = ff_rsqrt(ff_dot3(m, m));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) m[a] = ff_mul(m[a], im);
+    return isfinite(s2);
+}
+
+// The solve from the start n0 (any length): nf the normal in float-float, good
+// to ~1e-12 rad, and the FP64 iteration's count; false: solve in FP64.
+__device__ __forceinline__ bool solve_ff(const ff d[3], const ff oi[3], const ff oj[3], float api, float cpi,
+                                         float apj, float cpj, const ff n0[3], int maxit, ff nf[3], int &iters)
+{
+    constexpr float kLast = 5e-4f;  // the step below which FP32 hands over
+    const Shape<float> si = shape_ff(oi, cpi, api), sj = shape_ff(oj, cpj, apj);
+    const V3<float> df = mk<float>(d[0].hi, d[1].hi, d[2].hi);
+    const ff i0 = ff_rsqrt(ff_dot3(n0, n0));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) nf[a] = ff_mul(n0[a], i0);
+    V3<float> n = mk<float>(nf[0].hi, nf[1].hi, nf[2].hi);
+    const float noise = 4e-7f * (sqrtf(dot(df, df)) + fmaxf(api, cpi) + fmaxf(apj, cpj));
+    V3<float> before = n, t1 = perp_unit(n);
+    float g_last = 0.f, s_last = 0.f;
+    int it = 0;
+    // FP32 iterations (as newton_sphere) up to the first step below kLast, which is not taken
+    for (;;) {
+        if (it >= maxit) return false;
+        const V3<float> t2 = cross(n, t1);
+        const float ci = dot(si.o, n), u1i = dot(si.o, t1), u2i = dot(si.o, t2);
+        const float cj = dot(sj.o, n), u1j = dot(sj.o, t1), u2j = dot(sj.o, t2);
+        const float qi = si.a2 + si.e * ci * ci, qj = sj.a2 + sj.e * cj * cj;
+        const float ri = rsqrtf(qi), rj = rsqrtf(qj);
+        const float g = dot(n, df) - qi * ri - qj * rj;
+        const float ki = si.e * ci * ri, kj = sj.e * cj * rj;
+        const float g1 = dot(t1, df) - ki * u1i - kj * u1j, g2 = dot(t2, df) - ki * u2i - kj * u2j;
+        const float Ai = si.a2 * ri, Aj = sj.a2 * rj, Ei = si.e * ri * ri, Ej = sj.e * rj * rj;
+        const float P11 = Ai * (1.f + Ei * u1i * u1i) + Aj * (1.f + Ej * u1j * u1j) + g;
+        const float P22 = Ai * (1.f + Ei * u2i * u2i) + Aj * (1.f + Ej * u2j * u2j) + g;
+        const float P12 = Ai * Ei * u1i * u2i + Aj * Ej * u1j * u2j;
+        const float det = P11 * P22 - P12 * P12;
+        if (!(P11 > 0.f && det > 0.f)) return false;
+        const float idet = rcp_fast(det);
+        float s1 = (P22 * g1 - P12 * g2) * idet, s2 = (P11 * g2 - P12 * g1) * idet;
+        const float sn2 = s1 * s1 + s2 * s2;
+        if (!(sn2 >= kLast * kLast)) {
+            if (!isfinite(sn2)) return false;
+            break;
+        }
+        // a long step that did not raise g beyond FP32's noise: the FP64
+        // iteration may halve it (a short one, with the Hessian positive
+        // definite, raises g by more than its noise)
+        if (s_last > 0.03f && !(g > g_last + noise)) return false;
+        g_last = g;
+        if (sn2 > 0.25f) {
+            const float f = 0.5f * rsqrtf(sn2);
+            s1 *= f;
+            s2 *= f;
+        }
+        before = n;
+        s_last = sqrtf(sn2);
+        n = normalized(axpy(s1, t1, axpy(s2, t2, n)));
+        t1 = normalized(axpy(-dot(t1, n), n, t1));
+        ++it;
+    }
+    // Float-float steps from here.  dev: how far the iterate may be off the
+    // FP64 iteration's.  With no FP32 step the iterate is the start (nf holds
+    // it); after some, FP32 has left it off by some 3e-7, so that a step
+    // near or below that is not the FP64 iteration's: then the step is taken
+    // again from the iterate before, where it was long.
+    float dev = 1e-11f, sq;
+    if (it > 0) {
+        if (!newton_step_ff(d, oi, oj, api, cpi, apj, cpj, n, nf, sq)) return false;
+        if (sq >= 9e-12f) {
+            ++it;
+            s_last = sqrtf(sq);
+        } else if (!newton_step_ff(d, oi, oj, api, cpi, apj, cpj, before, nf, sq)) {
+            return false;
+        }
+        dev = 4e-6f * fminf(s_last, 0.5f);
+    }
+    for (int q = 0; q < 6; ++q) {
+        if (it >= maxit) return false;
+        const V3<float> nx = mk<float>(nf[0].hi, nf[1].hi, nf[2].hi);
+        ff m[3];
+        if (!newton_step_ff(d, oi, oj, api, cpi, apj, cpj, nx, m, sq)) return false;
+        // the step from the float-float iterate, not from its float part
+        float v[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            v[a] = __fadd_rn(__fsub_rn(m[a].hi, nf[a].hi), __fsub_rn(m[a].lo, nf[a].lo));
+            nf[a] = m[a];
+        }
+        const float s = sqrtf(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+        ++it;
+        if (fabsf(s - (float)kTolFp64) <= dev + 1e-11f) return false;
+        if (s < (float)kTolFp64) {
+            iters = it;
+            return isfinite(s);
+        }
+        dev = 1e-6f * s;
+    }
+    return false;
+}
+
+// The gap at the float-float normal nf and one Newton step from it, in FP64
+// (the Hessian in FP32): n64 the unit normal, h the gap.  False where the
+// step is not small, or the normal does not point from i to j.
+__device__ __forceinline__ bool finish_fp64(const V3<double> &d, const Shape<double> &si, const Shape<double> &sj,
+                                            const ff nf[3], V3<double> &n64, double &h)
+{
+    const V3<double> n = mk<double>(widen_bits(nf[0].hi) + widen_bits(nf[0].lo),
+                                    widen_bits(nf[1].hi) + widen_bits(nf[1].lo),
+                                    widen_bits(nf[2].hi) + widen_bits(nf[2].lo));
+    const double nn = dot(n, n);  // 1 to ~1e-13
+    const double ci = dot(si.o, n), cj = dot(sj.o, n);
+    const double ti = si.e * ci, tj = sj.e * cj;
+    const double ri = rsqrt64(fma(ti, ci, si.a2 * nn)), rj = rsqrt64(fma(tj, cj, sj.a2 * nn));
+    const double ki = ti * ri, kj = tj * rj, al = fma(si.a2, ri, sj.a2 * rj);
+    const V3<double> R = axpy(-ki, si.o, axpy(-kj, sj.o, d));  // grad g + al n
+    const double nR = dot(n, R);
+    const double g = fma(-al, nn, nR);
+    const double sc = fma(-0.5, nn, 1.5);  // 1 / |n|
+    h = g * sc;
+    // the part of R normal to n (n.R / |n|^2 = n.R (2 - |n|^2) to 1e-26)
+    const V3<double> Rt = axpy(-nR * (2.0 - nn), n, R);
+    const V3<float> nv = mk<float>(nf[0].hi, nf[1].hi, nf[2].hi);
+    const V3<float> rt = mk<float>(narrow_bits(Rt.x), narrow_bits(Rt.y), narrow_bits(Rt.z));
+    const V3<float> t1 = perp_unit(nv), t2 = cross(nv, t1);
+    const float G1 = dot(t1, rt), G2 = dot(t2, rt);
+    const V3<float> oi = mk<float>(narrow_bits(si.o.x), narrow_bits(si.o.y), narrow_bits(si.o.z));
+    const V3<float> oj = mk<float>(narrow_bits(sj.o.x), narrow_bits(sj.o.y), narrow_bits(sj.o.z));
+    const float u1i = dot(oi, t1), u2i = dot(oi, t2), u1j = dot(oj, t1), u2j = dot(oj, t2);
+    const float rif = narrow_bits(ri), rjf = narrow_bits(rj), gf = narrow_bits(g);
+    const float a2i = narrow_bits(si.a2), a2j = narrow_bits(sj.a2), ei = narrow_bits(si.e), ej = narrow_bits(sj.e);
+    const float Ai = a2i * rif, Aj = a2j * rjf, Ei = ei * rif * rif, Ej = ej * rjf * rjf;
+    const float P11 = Ai * (1.f + Ei * u1i * u1i) + Aj * (1.f + Ej * u1j * u1j) + gf;
+    const float P22 = Ai * (1.f + Ei * u2i * u2i) + Aj * (1.f + Ej * u2j * u2j) + gf;
+    const float P12 = Ai * Ei * u1i * u2i + Aj * Ej * u1j * u2j;
+    const float idet = rcp_fast(P11 * P22 - P12 * P12);
+    const float s1 = (P22 * G1 - P12 * G2) * idet, s2 = (P11 * G2 - P12 * G1) * idet;
+    const V3<float> st = axpy(s1, t1, scl(s2, t2));
+    n64 = mk<double>(n.x + widen_bits(st.x), n.y + widen_bits(st.y), n.z + widen_bits(st.z));
+    n64 = scl(sc, n64);  // (the step is normal to n: |n64| = |n| to 1e-22)
+    const V3<float> df = mk<float>(narrow_bits(d.x), narrow_bits(d.y), narrow_bits(d.z));
+    return s1 * s1 + s2 * s2 < 1e-18f && dot(nv, df) > 1e-3f * sqrtf(dot(df, df)) && isfinite(narrow_bits(h));
+}
+
+// the FP64 iteration itself, for the pairs that solve_ff leaves (out of line:
+// its registers are not the kernels')
+struct Fp64Solve {
+    V3<double> n;
+    double h;
+    int iters, noconv;
+};
+__device__ __noinline__ Fp64Solve solve_fp64(V3<double> d, Shape<double> si, Shape<double> sj, V3<double> n0,
+                                             double scale, int maxit)
+{
+    Fp64Solve r;
+    const NewtonOut o = newton_sphere<double>(si, sj, d, n0, maxit, kTolFp64, 1e-14 * scale);
+    r.iters = o.iters;
+    r.n = normalized(n0);
+    r.h = dot(r.n, d) - support(si, r.n) - support(sj, r.n);
+    r.noconv = !o.converged || !(dot(r.n, d) > 0.0) || !isfinite(r.h);
+    return r;
+}
+
+// minimum image of r_j - r_i, skipping the FP64 image shift of an axis where
+// the separation is clearly within half a box (the shift is then zero)
+__device__ __forceinline__ V3<double> min_image_near(const DView &D, V3<double> d)
+{
+    const float u = fabsf(narrow_bits(d.x)) * D.invLf[0], v = fabsf(narrow_bits(d.y)) * D.invLf[1],
+                w = fabsf(narrow_bits(d.z)) * D.invLf[2];
+    if ((!D.periodic[0] || u < 0.499f) && (!D.periodic[1] || v < 0.499f) && (!D.periodic[2] || w < 0.499f)) return d;
+    return min_image(D, d);
+}
+
+// LUB_FP64: the solve and gap of pair k
 template <bool ENS>
 __device__ __forceinline__ void closest_fp64_one(const PView &P, const DView &D0, const Ens &E, int i, int j, int k,
                                                  const double *__restrict__ nin, size_t C, int warm, int maxit,
@@ -425,31 +671,44 @@ __device__ __forceinline__ void closest_fp64_one(const PView &P, const DView &D0
     } else if (j < 0) {
         h = wall_gap(P, D, i, -1 - j, n64);
     } else {
-        const V3<double> d = min_image(D, sub(load_pos(P, j), load_pos(P, i)));
-        const double dl = sqrt(dot(d, d));
-        if (!(dl > 0.0) || !isfinite(dl)) {
+        const V3<double> d = min_image_near(D, sub(load_pos(P, j), load_pos(P, i)));
+        const double dd = dot(d, d);
+        const double idl = rsqrt64(dd), dl = dd * idl;
+        if (!(dd > 0.0) || !isfinite(dd)) {
             st = LUB_ST_DEGENERATE;
         } else {
             const float rpi = __ldg(P.rpar + i), rqi = __ldg(P.rperp + i);
             const float rpj = __ldg(P.rpar + j), rqj = __ldg(P.rperp + j);
             if (rpi == rqi && rpj == rqj) {
-                n64 = scl(1.0 / dl, d);
-                h = dl - (double)rpi - (double)rpj;
+                n64 = scl(idl, d);
+                h = dl - widen_bits(rpi) - widen_bits(rpj);
             } else {
                 const Shape<double> si = load_shape<double>(P, i), sj = load_shape<double>(P, j);
-                V3<double> nn = scl(1.0 / dl, d);
+                V3<double> nn = scl(idl, d);
                 if (warm) {
                     const V3<double> w0 = mk<double>(nin[k], nin[C + k], nin[2 * C + k]);
-                    const double wl2 = dot(w0, w0);
+                    const V3<float> wf = mk<float>(narrow_bits(w0.x), narrow_bits(w0.y), narrow_bits(w0.z));
+                    const float wl2 = dot(wf, wf);
                     // a start on the far hemisphere falls back to the line of centres
-                    if (wl2 > 0.25 && wl2 < 4.0 && isfinite(wl2) && dot(w0, d) > 0.0) nn = w0;
+                    if (wl2 > 0.25f && wl2 < 4.0f && isfinite(wl2) && dot(w0, d) > 0.0) {
+                        nn = w0;
+                    }
                 }
-                const double scale = dl + (double)fmaxf(rpi, rqi) + (double)fmaxf(rpj, rqj);
-                const NewtonOut o = newton_sphere<double>(si, sj, d, nn, maxit, kTolFp64, 1e-14 * scale);
-                nit = o.iters;
-                n64 = normalized(nn);
-                h = dot(n64, d) - support(si, n64) - support(sj, n64);
-                if (!o.converged || !(dot(n64, d) > 0.0) || !isfinite(h)) st |= LUB_ST_NOCONV;
+                const ff df[3] = {ff_split_bits(d.x), ff_split_bits(d.y), ff_split_bits(d.z)};
+                const ff oi[3] = {ff_split_bits(si.o.x), ff_split_bits(si.o.y), ff_split_bits(si.o.z)};
+                const ff oj[3] = {ff_split_bits(sj.o.x), ff_split_bits(sj.o.y), ff_split_bits(sj.o.z)};
+                const ff n0[3] = {ff_split_bits(nn.x), ff_split_bits(nn.y), ff_split_bits(nn.z)};
+                ff nf[3];
+                bool done = solve_ff(df, oi, oj, rqi, rpi, rqj, rpj, n0, maxit, nf, nit);
+                if (done) done = finish_fp64(d, si, sj, nf, n64, h);
+                if (!done) {
+                    const double scale = dl + (double)fmaxf(rpi, rqi) + (double)fmaxf(rpj, rqj);
+                    const Fp64Solve r = solve_fp64(d, si, sj, nn, scale, maxit);
+                    n64 = r.n;
+                    h = r.h;
+                    nit = r.iters;
+                    if (r.noconv) st |= LUB_ST_NOCONV;
+                }
             }
         }
     }

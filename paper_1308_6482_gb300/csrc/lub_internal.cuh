@@ -234,6 +234,18 @@ __device__ __forceinline__ double widen_bits(float f)
     return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo);
 }
 
+// A double truncated to a float's 24 bits; below the float range 0, above it
+// (and for infinities and NaN) infinity.
+__device__ __forceinline__ float narrow_bits(double d)
+{
+    const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
+    const int e = (int)((hw >> 20) & 0x7ffu) - (1023 - 127);
+    unsigned m = ((unsigned)e << 23) | ((hw & 0xfffffu) << 3) | (lw >> 29);
+    if (e <= 0) m = 0u;
+    if (e >= 255) m = 0x7f800000u;
+    return __uint_as_float(m | (hw & 0x80000000u));
+}
+
 // Double-precision reciprocal and reciprocal square root: an FP32 seed from
 // the argument's mantissa (its exponent handled by integer operations, so the
 // whole double range is covered and nothing is converted) and one third-order
@@ -310,12 +322,16 @@ __device__ __forceinline__ V3<T> cvt(const V3<S> &a)
 // ---------------------------------------------------------------------------
 // particle shape
 // ---------------------------------------------------------------------------
+// (conversions to double on the integer pipe)
+__device__ __forceinline__ float widen_to(float v, float) { return v; }
+__device__ __forceinline__ double widen_to(float v, double) { return widen_bits(v); }
+
 // Axis of rotational symmetry (body z) in the lab frame: third column of the
 // rotation matrix of q/|q|, q scalar first.
 template <typename T>
 __device__ __forceinline__ V3<T> quat_axis(float qw, float qx, float qy, float qz)
 {
-    T w = qw, x = qx, y = qy, z = qz;
+    T w = widen_to(qw, T(0)), x = widen_to(qx, T(0)), y = widen_to(qy, T(0)), z = widen_to(qz, T(0));
     T s = T(2) * rcp_t(w * w + x * x + y * y + z * z);
     return mk<T>(s * (x * z + w * y), s * (y * z - w * x), T(1) - s * (x * x + y * y));
 }
@@ -335,8 +351,8 @@ __device__ __forceinline__ Shape<T> load_shape(const PView &P, int k)
 {
     Shape<T> s;
     s.o = quat_axis<T>(__ldg(P.qw + k), __ldg(P.qx + k), __ldg(P.qy + k), __ldg(P.qz + k));
-    s.rpar = (T)__ldg(P.rpar + k);
-    s.rperp = (T)__ldg(P.rperp + k);
+    s.rpar = widen_to(__ldg(P.rpar + k), T(0));
+    s.rperp = widen_to(__ldg(P.rperp + k), T(0));
     s.a2 = s.rperp * s.rperp;
     s.e = s.rpar * s.rpar - s.a2;
     return s;
