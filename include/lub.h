@@ -306,10 +306,8 @@ int lub_mlp_set(lub_ctx *ctx, const float *params, const float *mean, const floa
  * 32 pairs, activations in registers; LUB_MLP_TCGEN05 with tcgen05.mma, 128
  * pairs per CTA, accumulators in tensor memory, operands staged in shared
  * memory (weights by one bulk copy per CTA).  Same results up to the order
- * of the FP32 accumulation.  With LUB_MLP_MMA_SYNC, lub_closest runs the
- * network inside its own kernel (each warp infers the start normals of its
- * 32 pairs and solves them in the same launch); with LUB_MLP_TCGEN05 the
- * network is a launch of its own before the solve.  A bounded wait of the tcgen05 path that times
+ * of the FP32 accumulation.  Either way the network of a call that starts
+ * every pair from it is a launch of its own before the solve.  A bounded wait of the tcgen05 path that times
  * out sets bit 3 (value 8) of the context's flags and ends the kernel. */
 #define LUB_MLP_MMA_SYNC 0
 #define LUB_MLP_TCGEN05 1
@@ -547,7 +545,7 @@ int lub_set_launch_shape(lub_ctx *ctx, int32_t kernel, int32_t block, int32_t bl
  * support for per-kernel rooflines.
  * ------------------------------------------------------------------------- */
 #define LUB_TRACE_SWEEP      0  /* lub_pairs_build: the cell sweep (k_pairs_sweep) */
-#define LUB_TRACE_CLOSEST    1  /* lub_closest_points: the solve (FP32 stage, FP64 or learned kernel);
+#define LUB_TRACE_CLOSEST    1  /* lub_closest_points: the solve (FP32 stage or FP64);
                                     lub_correct's one pass in LUB_MIXED */
 #define LUB_TRACE_RESISTANCE 2  /* lub_resistance / lub_resistance_apply: the pair-force kernel */
 #define LUB_TRACE_APPLY      3  /* lub_apply: the scatter kernel */

@@ -296,13 +296,42 @@ __device__ __forceinline__ float polish_gap_ff(const ff d[3], const ff oi[3], co
     return (nd > 0.f && isfinite(step2)) ? step2 : INFINITY;
 }
 
+// What the FP32 stage reads of a particle: from its per-call record, or (RAW)
+// from the caller's arrays, forming the same float-float values itself.  The
+// records pay where a particle is in several pairs; for lists shorter than
+// the particles (lub_closest_points on separate pairs) they are an extra pass
+// over all of them: 1M pairs of 2M particles from the network's start 342 us
+// with them, 307 without.
+template <bool RAW>
+__device__ __forceinline__ float4 rec_centre_xy(const PView &P, const float2 *__restrict__ pff, int k)
+{
+    if (!RAW) return rec_ld(pff, k, 0);
+    const ff x = ff_split_bits_nan(__ldg(P.x + k)), y = ff_split_bits_nan(__ldg(P.y + k));
+    return make_float4(x.hi, x.lo, y.hi, y.lo);
+}
+template <bool RAW>
+__device__ __forceinline__ float4 rec_centre_z(const PView &P, const float2 *__restrict__ pff, int k)
+{
+    if (!RAW) return rec_ld(pff, k, 1);
+    const ff z = ff_split_bits_nan(__ldg(P.z + k));
+    return make_float4(z.hi, z.lo, __ldg(P.rpar + k), __ldg(P.rperp + k));
+}
+template <bool RAW>
+__device__ __forceinline__ void rec_axis(const PView &P, const float2 *__restrict__ pff, int k, ff o[3])
+{
+    if (RAW)
+        ff_axis(__ldg(P.qw + k), __ldg(P.qx + k), __ldg(P.qy + k), __ldg(P.qz + k), o);
+    else
+        ff_axis_rec(rec_ld(pff, k, 2), rec_ld(pff, k, 3), o);
+}
+
 // LUB_MIXED, FP32 stage of pair k = (i, j): FP32 Newton, then the
 // float-float gap and Newton step (spheres: the float-float line of centres).
 // The normal and gap in double (n64, h) and in float-float (nf, hf: what the
 // fused pass hands to the force kernel).  Returns the FP64 work-list entry
 // -1-k (a full FP64 solve from the line of centres, for a pair whose FP32
 // Newton did not converge) or kNoEntry.
-template <bool ENS>
+template <bool ENS, bool RAW = false>
 __device__ __forceinline__ int closest_mixed_one(const PView &P, const DView &D0, const Ens &E,
                                                  const float2 *__restrict__ pff, int i, int j, int k,
                                                  const double *__restrict__ nin, size_t C, int warm, int maxit,
@@ -321,10 +350,10 @@ __device__ __forceinline__ int closest_mixed_one(const PView &P, const DView &D0
     bool bad = alien || i < 0 || i >= P.n || j >= P.n || j < -D.n_walls || j == i;
     float4 ri1 = make_float4(0.f, 0.f, 0.f, 0.f), rj1 = ri1;
     if (!bad) {
-        ri1 = rec_ld(pff, i, 1);
+        ri1 = rec_centre_z<RAW>(P, pff, i);
         bad = !shape_ok(ri1.z, ri1.w);
         if (!bad && j >= 0) {
-            rj1 = rec_ld(pff, j, 1);
+            rj1 = rec_centre_z<RAW>(P, pff, j);
             bad = !shape_ok(rj1.z, rj1.w);
         }
     }
@@ -335,7 +364,7 @@ __device__ __forceinline__ int closest_mixed_one(const PView &P, const DView &D0
         nf[2] = ff_make((float)n64.z);  // +-1
         hf = ff_split_bits(h);
     } else {
-        const float4 ri0 = rec_ld(pff, i, 0), rj0 = rec_ld(pff, j, 0);
+        const float4 ri0 = rec_centre_xy<RAW>(P, pff, i), rj0 = rec_centre_xy<RAW>(P, pff, j);
         ff dff[3];
         ff_separation(ri0, ri1, rj0, rj1, D, dff);
         const V3<float> df = mk<float>(dff[0].hi, dff[1].hi, dff[2].hi);
@@ -354,13 +383,13 @@ __device__ __forceinline__ int closest_mixed_one(const PView &P, const DView &D0
             h = ff_to_double(hf);
         } else {
             ff oi[3], oj[3];
-            ff_axis_rec(rec_ld(pff, i, 2), rec_ld(pff, i, 3), oi);
-            ff_axis_rec(rec_ld(pff, j, 2), rec_ld(pff, j, 3), oj);
+            rec_axis<RAW>(P, pff, i, oi);
+            rec_axis<RAW>(P, pff, j, oj);
             const Shape<float> si = shape_ff(oi, rpi, rqi), sj = shape_ff(oj, rpj, rqj);
             const float idl = rsqrtf(dd2), dl = dd2 * idl;  // Newton renormalises its start
             V3<float> n = scl(idl, df);
             if (warm) {
-                const V3<float> w0 = mk<float>((float)nin[k], (float)nin[C + k], (float)nin[2 * C + k]);
+                const V3<float> w0 = mk<float>(round_bits(nin[k]), round_bits(nin[C + k]), round_bits(nin[2 * C + k]));
                 const float wl2 = dot(w0, w0);
                 // a start on the far hemisphere falls back to the line of centres
                 if (wl2 > 0.25f && wl2 < 4.0f && isfinite(wl2) && dot(w0, df) > 0.f) n = scl(rsqrtf(wl2), w0);
@@ -833,8 +862,8 @@ __global__ void __launch_bounds__(256) k_particles_ff(PView P, float4 *__restric
     }
 }
 
-template <bool ENS>
-__global__ void __launch_bounds__(128, 8) k_closest_mixed(PView P, const __grid_constant__ DView D0, Ens E,
+template <bool ENS, bool RAW>
+__global__ void __launch_bounds__(128, RAW ? 7 : 8) k_closest_mixed(PView P, const __grid_constant__ DView D0, Ens E,
                                                        const int32_t *__restrict__ pi, const int32_t *__restrict__ pj,
                                                        const int32_t *__restrict__ d_count, int32_t cap,
                                                        double *__restrict__ nout, double *__restrict__ gap,
@@ -857,7 +886,7 @@ __global__ void __launch_bounds__(128, 8) k_closest_mixed(PView P, const __grid_
             double h;
             ff nf[3], hf;
             int st, nit;
-            entry = closest_mixed_one<ENS>(P, D0, E, pff, i, j, k, nout, C, warm, maxit, tol32, n64, h, nf, hf, st,
+            entry = closest_mixed_one<ENS, RAW>(P, D0, E, pff, i, j, k, nout, C, warm, maxit, tol32, n64, h, nf, hf, st,
                                            nit);
             store_pair(nout, gap, status, iters, C, k, n64, h, st, nit);
             if (nh) store_nh(nh, C, k, nf, hf);
@@ -908,81 +937,6 @@ __global__ void __launch_bounds__(128) k_closest_fp64(PView P, const __grid_cons
         int st, nit;
         closest_fp64_one<ENS>(P, D0, E, __ldg(pi + k), __ldg(pj + k), k, nout, C, warm, maxit, n64, h, st, nit);
         store_pair(nout, gap, status, iters, C, k, n64, h, st, nit);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// the learned warm start inside the closest-point kernels (the mma.sync
-// engine): every warp runs the network for its 32 pairs on the tensor cores,
-// forms Newton's start normals from the outputs, writes them to n (the solve
-// reads them back from there: the same thread, cached) and solves; one launch
-// instead of the network's own, no start normals through HBM in between.
-// ---------------------------------------------------------------------------
-template <bool ENS>
-__global__ void __launch_bounds__(32 * INF_WARPS, 2) k_closest_mixed_learned(
-    PView P, const __grid_constant__ DView D0, Ens E, const int32_t *__restrict__ pi, const int32_t *__restrict__ pj,
-    const int32_t *__restrict__ d_count, int32_t cap, double *__restrict__ nout, double *__restrict__ gap,
-    uint8_t *__restrict__ status, uint8_t *__restrict__ iters, int maxit, float tol32, int32_t *__restrict__ wl_count,
-    int32_t *__restrict__ wl, const float2 *__restrict__ pff, float4 *__restrict__ nh, MlpDevice M)
-{
-    pdl_wait();
-    pdl_trigger();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    InfSmem &S = *reinterpret_cast<InfSmem *>(smem_raw);
-    stage_weights(S, M);
-    __syncthreads();
-    const int count = pair_count(d_count, cap);
-    const size_t C = (size_t)cap;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int base = (blockIdx.x * INF_WARPS + w) * 32; base < count; base += gridDim.x * INF_WARPS * 32) {
-        const int k = base + lane;
-        float f[NI];
-        const PairIn in = pair_inputs<ENS>(P, D0, E, pi, pj, k, count, S.mean, S.istd, f);
-        const float4 y = warp_mlp(S, S.x[w], S.y[w], f, lane);
-        pair_outputs(P, in, y, k, count, C, nout, nullptr);
-        int entry = kNoEntry;
-        if (k < count) {
-            V3<double> n64;
-            double h;
-            ff nf[3], hf;
-            int st, nit;
-            entry = closest_mixed_one<ENS>(P, D0, E, pff, __ldg(pi + k), __ldg(pj + k), k, nout, C, 1, maxit, tol32,
-                                           n64, h, nf, hf, st, nit);
-            store_pair(nout, gap, status, iters, C, k, n64, h, st, nit);
-            if (nh) store_nh(nh, C, k, nf, hf);
-        }
-        worklist_append(entry, wl_count, wl, cap);
-    }
-}
-
-template <bool ENS>
-__global__ void __launch_bounds__(32 * INF_WARPS, 2) k_closest_fp64_learned(
-    PView P, const __grid_constant__ DView D0, Ens E, const int32_t *__restrict__ pi, const int32_t *__restrict__ pj,
-    const int32_t *__restrict__ d_count, int32_t cap, double *__restrict__ nout, double *__restrict__ gap,
-    uint8_t *__restrict__ status, uint8_t *__restrict__ iters, int maxit, MlpDevice M)
-{
-    pdl_wait();
-    pdl_trigger();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    InfSmem &S = *reinterpret_cast<InfSmem *>(smem_raw);
-    stage_weights(S, M);
-    __syncthreads();
-    const int count = pair_count(d_count, cap);
-    const size_t C = (size_t)cap;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int base = (blockIdx.x * INF_WARPS + w) * 32; base < count; base += gridDim.x * INF_WARPS * 32) {
-        const int k = base + lane;
-        float f[NI];
-        const PairIn in = pair_inputs<ENS>(P, D0, E, pi, pj, k, count, S.mean, S.istd, f);
-        const float4 y = warp_mlp(S, S.x[w], S.y[w], f, lane);
-        pair_outputs(P, in, y, k, count, C, nout, nullptr);
-        if (k < count) {
-            V3<double> n64;
-            double h;
-            int st, nit;
-            closest_fp64_one<ENS>(P, D0, E, __ldg(pi + k), __ldg(pj + k), k, nout, C, 1, maxit, n64, h, st, nit);
-            store_pair(nout, gap, status, iters, C, k, n64, h, st, nit);
-        }
     }
 }
 
@@ -1105,7 +1059,7 @@ __global__ void __launch_bounds__(128) k_fused_fp64(PView P, const __grid_consta
     }
 }
 
-// One pass of the mixed mode (lub_correct, without the network): each pair's
+// One pass of the mixed mode (lub_correct, but for LUB_WARM_MLP): each pair's
 // closest points and gap, resistance and scatter by the same thread, the
 // normal and gap staying in registers in float-float.  The pairs of a block
 // whose FP32 Newton did not converge are gathered in shared memory and solved
@@ -1273,34 +1227,29 @@ int launch_closest_t(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E,
                      float *zero_force = nullptr, float *zero_torque = nullptr)
 {
     int warm = 0, rc;
+    // (the network for every pair is a launch of its own before the solve:
+    // inside the solve's kernel its 128 registers and shared-memory weights
+    // left the solve at 16 warps per SM: 131,072 pairs in FP64 195 us, as two
+    // launches 147)
     const bool net_all = net_every_pair(prm);
     const bool net_wl = prm.warm_start == LUB_WARM_MLP && prm.precision == LUB_MIXED;
     if ((net_all || net_wl) && !ctx->mlp_ready)
         return lub_set_error(ctx, LUB_ERR_ARG, "the learned warm start needs lub_mlp_set first");
-    // the learned start of every pair on the mma.sync engine runs inside the solve's kernel
-    const bool fused_mlp = net_all && ctx->mlp_engine == LUB_MLP_MMA_SYNC;
-    if (!fused_mlp && (rc = start_normals(ctx, P, D, E, prm, pi, pj, d_count, cap, n, st, &warm))) return rc;
-    const int learned_grid = 2 * ctx->num_sms;
+    if ((rc = start_normals(ctx, P, D, E, prm, pi, pj, d_count, cap, n, st, &warm))) return rc;
     if (prm.precision == LUB_MIXED) {
         int32_t *wl_count, *wl;
         float2 *pff = nullptr;
         float4 *nh = nullptr;
-        if ((rc = work_list(ctx, cap, st, &wl_count, &wl, keep ? &nh : nullptr, keep ? &status : nullptr, &P, &pff,
-                            zero_force, zero_torque)))
+        const bool raw = !keep && cap <= P.n;  // no more pairs than particles: no records
+        if ((rc = work_list(ctx, cap, st, &wl_count, &wl, keep ? &nh : nullptr, keep ? &status : nullptr,
+                            raw ? nullptr : &P, &pff, zero_force, zero_torque)))
             return rc;
         if (keep) *keep = ClosestKeep{status, pff, nh};
         lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
-        if (fused_mlp) {
-            if ((rc = learned_smem(ctx, k_closest_mixed_learned<ENS>, 16 << ENS))) return rc;
-            (void)launch_pdl(k_closest_mixed_learned<ENS>, learned_grid, 32 * INF_WARPS, sizeof(InfSmem), st, P, D, E,
-                             pi, pj, d_count, cap, n, gap, status, iters, prm.max_newton, (float)prm.newton_tol,
-                             wl_count, wl, (const float2 *)pff, nh, *(const MlpDevice *)ctx->mlp);
-        } else {
-            const Shape2 sh = tuned_shape(ctx, LUB_TUNE_CLOSEST_MIXED, cap);
-            (void)launch_pdl(k_closest_mixed<ENS>, sh.grid, sh.block, 0, st, P, D, E, pi, pj, d_count, cap, n, gap,
-                             status, iters, prm.max_newton, (float)prm.newton_tol, warm, wl_count, wl,
-                             (const float2 *)pff, nh);
-        }
+        const Shape2 sh = tuned_shape(ctx, LUB_TUNE_CLOSEST_MIXED, cap);
+        (void)launch_pdl(raw ? k_closest_mixed<ENS, true> : k_closest_mixed<ENS, false>, sh.grid, sh.block, 0, st, P,
+                         D, E, pi, pj, d_count, cap, n, gap, status, iters, prm.max_newton, (float)prm.newton_tol,
+                         warm, wl_count, wl, (const float2 *)pff, nh);
         lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
         if (net_wl) {
             // the work list's FP64 solves from the network's start (returns at once when it is empty)
@@ -1314,12 +1263,6 @@ int launch_closest_t(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E,
             (void)launch_pdl(k_closest_refine<ENS>, sr.grid, sr.block, 0, st, P, D, E, pi, pj, cap, n, gap, status,
                              iters, prm.max_newton, (const int32_t *)wl_count, (const int32_t *)wl, nh);
         }
-    } else if (fused_mlp) {
-        if ((rc = learned_smem(ctx, k_closest_fp64_learned<ENS>, 64 << ENS))) return rc;
-        lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
-        (void)launch_pdl(k_closest_fp64_learned<ENS>, learned_grid, 32 * INF_WARPS, sizeof(InfSmem), st, P, D, E, pi,
-                         pj, d_count, cap, n, gap, status, iters, prm.max_newton, *(const MlpDevice *)ctx->mlp);
-        lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
     } else {
         const Shape2 sh = tuned_shape(ctx, LUB_TUNE_CLOSEST_FP64, cap);
         lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
@@ -1346,8 +1289,10 @@ int launch_correct_t(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E,
         // the kernels of lub_closest_points, then those of lub_resistance_apply
         // on the same per-call particle records (built once; their kernel also
         // clears the sums unless accumulate is set)
-        if (prm.warm_start != LUB_WARM_MLP && prm.warm_start != LUB_WARM_MLP_ALL && cap <= kFusedMax) {
+        if (prm.warm_start != LUB_WARM_MLP && cap <= kFusedMax) {
             // small lists: the records, then one pass over the pairs
+            int warm = 0;
+            if ((rc = start_normals(ctx, P, D, E, prm, pi, pj, d_count, cap, n, st, &warm))) return rc;
             if ((rc = lub_ensure_scratch(ctx, particles_ff_bytes(P.n)))) return rc;
             float2 *pff = (float2 *)ctx->scratch;
             if ((rc = launch_particles_ff(ctx, P, pff, st, nullptr, accumulate ? nullptr : (float *)force,
@@ -1358,8 +1303,7 @@ int launch_correct_t(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E,
             lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
             (void)launch_pdl(k_fused_mixed<ENS>, sh.grid, sh.block, 0, st, P, D, E, R, pi, pj, d_count, cap, n, gap,
                              status, iters, (float *)FT, (float *)lever, prm.max_newton, (float)prm.newton_tol,
-                             (int)(prm.warm_start == LUB_WARM_PREVIOUS), (float *)force, (float *)torque,
-                             (const float2 *)pff);
+                             warm, (float *)force, (float *)torque, (const float2 *)pff);
             lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
             return lub_check_cuda(ctx, cudaGetLastError(), "one-pass launch");
         }

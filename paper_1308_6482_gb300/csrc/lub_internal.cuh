@@ -234,6 +234,19 @@ __device__ __forceinline__ double widen_bits(float f)
     return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo);
 }
 
+// A double rounded to the nearest float (ties to even), on the integer pipe
+// for results in the normal float range
+__device__ __forceinline__ float round_bits(double d)
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const int e = (int)(hi >> 20 & 0x7ffu) - 1023 + 127;
+    if (e <= 0 || e >= 254) return (float)d;  // zero, subnormal, near overflow, not finite
+    const unsigned m = ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned rest = lo << 3, odd = m & 1u;
+    const unsigned up = rest > 0x80000000u || (rest == 0x80000000u && odd);
+    return __uint_as_float((m + up) | (hi & 0x80000000u));
+}
+
 // A double truncated to a float's 24 bits; below the float range 0, above it
 // (and for infinities and NaN) infinity.
 __device__ __forceinline__ float narrow_bits(double d)

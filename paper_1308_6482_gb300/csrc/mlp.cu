@@ -521,6 +521,8 @@ __global__ void __launch_bounds__(32 * INF_WARPS, 2) k_mlp_start(PView P, const 
                                                                 MlpDevice M, double *__restrict__ n0,
                                                                 float *__restrict__ pq)
 {
+    pdl_wait();
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     InfSmem &S = *reinterpret_cast<InfSmem *>(smem_raw);
     const int count = pair_count(d_count, cap);
@@ -698,9 +700,12 @@ int launch_mlp_start_t(lub_ctx *ctx, const PView &P, const DView &D, const Ens &
         if (rc) return rc;
         ctx->mlp_smem_set |= 1 << ENS;
     }
-    k_mlp_start<ENS><<<ctx->num_sms * 2, 32 * INF_WARPS, smem, st>>>(P, D, E, pi, pj, d_count, cap,
-                                                                     *(const MlpDevice *)ctx->mlp, n0, pq);
-    return lub_check_cuda(ctx, cudaGetLastError(), "k_mlp_start launch");
+    const int64_t tiles = ((int64_t)cap + 32 * INF_WARPS - 1) / (32 * INF_WARPS);
+    const int grid = (int)(tiles < 2 * ctx->num_sms ? tiles : 2 * ctx->num_sms);
+    return lub_check_cuda(ctx,
+                          launch_pdl(k_mlp_start<ENS>, grid, 32 * INF_WARPS, smem, st, P, D, E, pi, pj, d_count, cap,
+                                     *(const MlpDevice *)ctx->mlp, n0, pq),
+                          "k_mlp_start launch");
 }
 
 int launch_mlp_start(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E, const int32_t *pi, const int32_t *pj,

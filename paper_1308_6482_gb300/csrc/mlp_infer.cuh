@@ -1,5 +1,5 @@
 // The learned warm start's inference, shared by the start kernel (mlp.cu)
-// and the closest-point kernels that run it in front of Newton (closest.cu):
+// and the work list's FP64 solves that start from it (closest.cu):
 // the 12 pair features, the warp-level BF16 tensor-core forward pass of the
 // 12 -> 128 -> 128 -> 4 network, and Newton's start normal from its outputs.
 // See mlp.cu for the network and its training.
@@ -7,6 +7,7 @@
 
 #include <cuda_bf16.h>
 
+#include "ff.cuh"
 #include "lub_internal.cuh"
 #include "lub_mlp.cuh"
 
@@ -17,6 +18,25 @@ constexpr int NI = 12, NH = 128, NO = 4;
 // ---------------------------------------------------------------------------
 // features (the same device code for training and inference)
 // ---------------------------------------------------------------------------
+// the separation r_j - r_i at the minimum image, rounded to float (from
+// float-float centres split by integer operations: no FP64 instruction, each
+// of which would cost as much as some seventy others)
+__device__ __forceinline__ V3<float> separation_f(const PView &P, const DView &D, int i, int j)
+{
+    const double *pos[3] = {P.x, P.y, P.z};
+    float r[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        ff d = ff_sub(ff_split_bits_nan(__ldg(pos[a] + j)), ff_split_bits_nan(__ldg(pos[a] + i)));
+        if (D.periodic[a]) {
+            const float k = rintf(d.hi * D.invLf[a]);
+            if (k != 0.f) d = ff_sub(d, ff_mulf(ff{D.Lff[a][0], D.Lff[a][1]}, k));
+        }
+        r[a] = d.hi;
+    }
+    return mk<float>(r[0], r[1], r[2]);
+}
+
 // The 12 features (FP32): in i's body frame turned about its symmetry axis
 // until d lies in the half-plane y = 0, x >= 0: [0] rho / R_perp,i,
 // [1] d_z / R_perp,i, [2..4] j's axis; [5..8] ln of the four semi-axes;
@@ -26,8 +46,7 @@ constexpr int NI = 12, NH = 128, NO = 4;
 __device__ __forceinline__ void pair_features(const PView &P, const DView &D, int i, int j, const float *mean,
                                               const float *istd, float f[NI])
 {
-    const V3<double> dd = min_image(D, sub(load_pos(P, j), load_pos(P, i)));
-    const V3<float> d = cvt<float>(dd);
+    const V3<float> d = separation_f(P, D, i, j);
     float qa[4] = {P.qw[i], P.qx[i], P.qy[i], P.qz[i]};
     const float na = rsqrtf(qa[0] * qa[0] + qa[1] * qa[1] + qa[2] * qa[2] + qa[3] * qa[3]);
     for (int a = 0; a < 4; ++a) qa[a] *= na;
@@ -316,7 +335,7 @@ __device__ __forceinline__ void pair_outputs(const PView &P, const PairIn &in, c
         V3<float> s0 = mk<float>(0, 0, 0);
         if (in.ok) {
             // corrections to the parameters of the line-of-centres start
-            const V3<float> d = cvt<float>(min_image(*in.D, sub(load_pos(P, in.j), load_pos(P, in.i))));
+            const V3<float> d = separation_f(P, *in.D, in.i, in.j);
             const V3<float> e = normalized(d);
             const V3<float> ni = shifted_normal(P, in.i, rot_of(P, in.i), e, y.x, y.y);
             const V3<float> nj = shifted_normal(P, in.j, rot_of(P, in.j), scl(-1.0f, e), y.z, y.w);
@@ -324,9 +343,9 @@ __device__ __forceinline__ void pair_outputs(const PView &P, const PairIn &in, c
             const float l2 = dot(s, s);
             if (l2 > 1e-12f && isfinite(l2)) s0 = scl(rsqrtf(l2), s);
         }
-        n0[k] = s0.x;
-        n0[C + k] = s0.y;
-        n0[2 * C + k] = s0.z;
+        n0[k] = widen_bits(s0.x);
+        n0[C + k] = widen_bits(s0.y);
+        n0[2 * C + k] = widen_bits(s0.z);
     }
 }
 

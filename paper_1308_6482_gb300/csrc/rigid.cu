@@ -23,19 +23,6 @@ namespace {
 // and cosine summed as series of the squared half angle.  32,768 particles:
 // 28 -> 17 us alone (312 -> 150 FP64 instructions a warp).
 
-// a double rounded to the nearest float (ties to even), on the integer pipe
-// for results in the normal float range
-__device__ __forceinline__ float round_bits(double d)
-{
-    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-    const int e = (int)(hi >> 20 & 0x7ffu) - 1023 + 127;
-    if (e <= 0 || e >= 254) return (float)d;  // zero, subnormal, near overflow, not finite
-    const unsigned m = ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-    const unsigned rest = lo << 3, odd = m & 1u;
-    const unsigned up = rest > 0x80000000u || (rest == 0x80000000u && odd);
-    return __uint_as_float((m + up) | (hi & 0x80000000u));
-}
-
 // the symmetry axis of the rotation by q/|q|, from s = 2 / |q|^2
 __device__ __forceinline__ V3<double> axis_of(double s, double w, double x, double y, double z)
 {
