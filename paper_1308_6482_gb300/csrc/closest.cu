@@ -623,11 +623,12 @@ __device__ __forceinline__ bool finish_fp64(const V3<double> &d, const Shape<dou
     const double nn = dot(n, n);  // 1 to ~1e-13
     const double ci = dot(si.o, n), cj = dot(sj.o, n);
     const double ti = si.e * ci, tj = sj.e * cj;
-    const double ri = rsqrt64(fma(ti, ci, si.a2 * nn)), rj = rsqrt64(fma(tj, cj, sj.a2 * nn));
-    const double ki = ti * ri, kj = tj * rj, al = fma(si.a2, ri, sj.a2 * rj);
-    const V3<double> R = axpy(-ki, si.o, axpy(-kj, sj.o, d));  // grad g + al n
+    const double qi = fma(ti, ci, si.a2 * nn), qj = fma(tj, cj, sj.a2 * nn);
+    const double ri = rsqrt64(qi), rj = rsqrt64(qj);
+    const double ki = ti * ri, kj = tj * rj;
+    const V3<double> R = axpy(-ki, si.o, axpy(-kj, sj.o, d));  // grad g but for its part along n
     const double nR = dot(n, R);
-    const double g = fma(-al, nn, nR);
+    const double g = fma(-qj, rj, fma(-qi, ri, dot(n, d)));
     const double sc = fma(-0.5, nn, 1.5);  // 1 / |n|
     h = g * sc;
     // the part of R normal to n (n.R / |n|^2 = n.R (2 - |n|^2) to 1e-26)

@@ -93,7 +93,36 @@ struct Surf {
 };
 
 __device__ __forceinline__ float log1p_t(float x) { return log1pf(x); }
-__device__ __forceinline__ double log1p_t(double x) { return log1p(x); }
+// log(1 + x) for x > -1 in some 22 FP64 instructions (the library's takes
+// several times that, and the FP64 pipe is this mode's bound): 1 + x = 2^k m
+// with m in [sqrt(1/2), sqrt(2)), log m = 2 atanh(s), s = (m - 1)/(m + 1)
+// (Abramowitz & Stegun 4.1.27), |s| < 0.1716, as its Taylor series to s^23
+// (the next term is below 2^-60 of the first).  For k = 0 m - 1 is x itself,
+// so the result keeps its relative accuracy as x goes to 0.
+__device__ __forceinline__ double log1p_t(double x)
+{
+    const double a = 1.0 + x;
+    const int hi = __double2hiint(a);
+    // k: the exponent of a / sqrt(1/2) rounded down
+    const int k = (hi - 0x3fe6a09e) >> 20;
+    const double m = __hiloint2double(hi - (k << 20), __double2loint(a));
+    const double f = k ? m - 1.0 : x;
+    const double s = f * rcp64(2.0 + f), w = s * s;
+    double p = fma(w, 1.0 / 23.0, 1.0 / 21.0);
+    p = fma(w, p, 1.0 / 19.0);
+    p = fma(w, p, 1.0 / 17.0);
+    p = fma(w, p, 1.0 / 15.0);
+    p = fma(w, p, 1.0 / 13.0);
+    p = fma(w, p, 1.0 / 11.0);
+    p = fma(w, p, 1.0 / 9.0);
+    p = fma(w, p, 1.0 / 7.0);
+    p = fma(w, p, 1.0 / 5.0);
+    p = fma(w, p, 1.0 / 3.0);
+    const double s2 = s + s;
+    const double l = fma(w * p, s2, s2);
+    // k is small (|k| < 2^10): its double by the exact float
+    return k ? fma(widen_bits((float)k), 0.693147180559945309417, l) : l;
+}
 
 // Local geometry at surface offset rho = y* - r with outward normal nrm.
 template <typename T>
@@ -104,22 +133,42 @@ __device__ __forceinline__ Surf<T> surface_at(const Shape<T> &s, const V3<T> &rh
     const T zt = dot(rho, s.o);
     const V3<T> rp = axpy(-zt, s.o, rho);  // component normal to the axis
     const T rr2 = dot(rp, rp);
-    const T spr = zt * ipar;                         // sin p, unnormalised
-    const T cpr = sqrt_fast(rr2) * iperp;            // cos p, unnormalised
-    const T hn = rsqrt_t(spr * spr + cpr * cpr);
-    const T sp = spr * hn, cp = cpr * hn;
     V3<T> er;
-    if (rr2 > T(1e-24) * s.a2) {
-        er = scl(rsqrt_t(rr2), rp);
-    } else {  // pole: any direction normal to the axis (umbilic point)
-        V3<T> e = (fabs((double)s.o.x) < 0.6) ? mk<T>(1, 0, 0) : mk<T>(0, 1, 0);
-        er = normalized(axpy(-dot(e, s.o), s.o, e));
+    T sp, cp, is1;
+    if constexpr (sizeof(T) == 4) {
+        const T spr = zt * ipar;               // sin p, unnormalised
+        const T cpr = sqrt_fast(rr2) * iperp;  // cos p, unnormalised
+        const T hn = rsqrt_t(spr * spr + cpr * cpr);
+        sp = spr * hn, cp = cpr * hn;
+        if (rr2 > T(1e-24) * s.a2) {
+            er = scl(rsqrt_t(rr2), rp);
+        } else {  // pole: any direction normal to the axis (umbilic point)
+            V3<T> e = (fabs((double)s.o.x) < 0.6) ? mk<T>(1, 0, 0) : mk<T>(0, 1, 0);
+            er = normalized(axpy(-dot(e, s.o), s.o, e));
+        }
+        // d y~/dp = -R_perp sin p e_r + R_par cos p o
+        V3<T> s1v = axpy(-s.rperp * sp, er, scl(s.rpar * cp, s.o));
+        o.x1 = normalized(axpy(-dot(s1v, nrm), nrm, s1v));
+        is1 = rsqrt_t(s.rperp * s.rperp * sp * sp + s.rpar * s.rpar * cp * cp);
+    } else {
+        // FP64: rho lies on the surface, so sin^2 p + cos^2 p = 1 and
+        // d y~/dp is tangent and of length s1 to rounding; neither is
+        // enforced again (FP32 does: it halves that form's error), one
+        // reciprocal root serves cos p and e_r
+        const T irr = rsqrt_t(rr2);
+        sp = zt * ipar;
+        if (rr2 > T(1e-24) * s.a2) {
+            cp = rr2 * irr * iperp;
+            er = scl(irr, rp);
+        } else {
+            cp = T(0);
+            V3<T> e = (fabs(s.o.x) < 0.6) ? mk<T>(1, 0, 0) : mk<T>(0, 1, 0);
+            er = normalized(axpy(-dot(e, s.o), s.o, e));
+        }
+        const T rsp = s.rperp * sp, rcp_ = s.rpar * cp;
+        is1 = rsqrt_t(rsp * rsp + rcp_ * rcp_);
+        o.x1 = axpy(-rsp * is1, er, scl(rcp_ * is1, s.o));
     }
-    // d y~/dp = -R_perp sin p e_r + R_par cos p o
-    V3<T> s1v = axpy(-s.rperp * sp, er, scl(s.rpar * cp, s.o));
-    o.x1 = normalized(axpy(-dot(s1v, nrm), nrm, s1v));
-    const T s1sq = s.rperp * s.rperp * sp * sp + s.rpar * s.rpar * cp * cp;
-    const T is1 = rsqrt_t(s1sq);
     const T is2 = is1 * is1;
     o.c1 = s.rpar * s.rperp * is1 * is2;            // 1/S1 = R_par R_perp / s1^3
     o.c2 = s.rpar * iperp * is1;                    // 1/S2 = R_par / (R_perp s1)
@@ -274,14 +323,14 @@ __device__ __forceinline__ void pair_force(const PView &P, const RParams &R, int
         PairKin<double> K;
         K.n = n64;
         K.si = load_shape<double>(P, i);
-        K.vi = mk<double>(__ldg(P.vx + i), __ldg(P.vy + i), __ldg(P.vz + i));
-        K.Wi = mk<double>(__ldg(P.wx + i), __ldg(P.wy + i), __ldg(P.wz + i));
+        K.vi = mk<double>(widen_bits(__ldg(P.vx + i)), widen_bits(__ldg(P.vy + i)), widen_bits(__ldg(P.vz + i)));
+        K.Wi = mk<double>(widen_bits(__ldg(P.wx + i)), widen_bits(__ldg(P.wy + i)), widen_bits(__ldg(P.wz + i)));
         K.sj = {};
         K.vj = K.Wj = mk<double>(0.0, 0.0, 0.0);
         if (j >= 0) {
             K.sj = load_shape<double>(P, j);
-            K.vj = mk<double>(__ldg(P.vx + j), __ldg(P.vy + j), __ldg(P.vz + j));
-            K.Wj = mk<double>(__ldg(P.wx + j), __ldg(P.wy + j), __ldg(P.wz + j));
+            K.vj = mk<double>(widen_bits(__ldg(P.vx + j)), widen_bits(__ldg(P.vy + j)), widen_bits(__ldg(P.vz + j)));
+            K.Wj = mk<double>(widen_bits(__ldg(P.wx + j)), widen_bits(__ldg(P.wy + j)), widen_bits(__ldg(P.wz + j)));
         }
         K.u3 = 0.0;
         pair_force_body<double>(R, j, cut, K, out);
@@ -401,7 +450,13 @@ __device__ __forceinline__ void pair_force_body(const RParams &R, int j, const C
         }
         {  // cubic couplings K13, K23, K34, K35 (Gamma_1 = Gamma_3 = 0)
             T beta[4], kap[4];
-            m_rot<T>(cf, sf, G0p, T(0), G2p, T(0), beta);
+            {  // m_rot of (G0p, 0, G2p, 0) by (cf, sf)
+                const T cc = cf * cf, ss = sf * sf, u = G0p * cc, v = G2p * ss, w0 = T(3) * G0p - T(2) * G2p;
+                beta[0] = cf * (u + v);
+                beta[1] = sf * (cc * w0 + v);
+                beta[2] = cf * (ss * w0 + G2p * cc);
+                beta[3] = sf * (G0p * ss + G2p * cc);
+            }
             m_rot<T>(cx, sx, A.G0 + beta[0], beta[1], A.G2 + beta[2], beta[3], kap);
             const T ir1 = rcp_fast(r1), ir2 = rcp_fast(r2);
             kap[0] *= ir1 * ir1 * ir1;
