@@ -479,6 +479,7 @@ __device__ __forceinline__ void defer_candidate(int i, int j, const BuildView &V
 // them, dynamic): the groups' staging (rows padded by one entry, so that the
 // groups' broadcast reads fall in different banks), each lane's particle,
 // and the warp's queue of candidates for the full test (a ring of 64).
+constexpr int kWarpUnd = 15;
 struct SweepWarp {
     float4 cand[NG * (SC + 1)];
     float4 own1[32];  // each lane's symmetry axis and e
@@ -488,6 +489,8 @@ struct SweepWarp {
     int own_i[32];    // each lane's particle index
     int qt[64];       // queued: candidate slot t
     uint8_t qo[64];   // queued: lane of the particle
+    int2 und[kWarpUnd];  // candidates inside the FP32 margin (smaller, larger index)
+    int nund, pad;       // how many there were
 };
 static_assert(sizeof(SweepWarp) % 16 == 0, "warp blocks stay 16-byte aligned");
 
@@ -519,20 +522,23 @@ static_assert(sizeof(SweepWarp) % 16 == 0, "warp blocks stay 16-byte aligned");
 // E 2^-20 to the grid's, so that every decision inside it still goes to the
 // FP64 test.
 //
-// Candidates inside the FP32 margin (about one in 10^4) are left to the
-// next kernel (defer_candidate), which tests them in float-float and, inside
-// that test's far smaller margin, in FP64: deciding them in the drain kept
-// the FP64 test's registers in the sweep's loop, where they cost spills
-// (the sweep ran 10 % faster without it).
+// Candidates inside the FP32 margin (about one in 10^4) are put aside by
+// their warp and tested at its end, in float-float and, inside that test's
+// far smaller margin, in FP64: deciding them in the drain kept the FP64 test's
+// registers in the sweep's loop, where they cost spills (the sweep ran 10 %
+// faster without it).  A warp with more than kWarpUnd of them (inputs built on
+// the filters' edges) leaves the rest to the next kernel (defer_candidate).
+// (All of them in the next kernel was a chain of some 8 us on its own: a few
+// hundred candidates leave the GPU empty while they wait for their loads.)
 
 //
-// Rows: a block takes V.rows of the five rows of its slots (blocks [b tiles,
-// (b + 1) tiles) rows [b rows, (b + 1) rows)).  Large inputs take all five in
+// Rows (ROW1): a block takes one of the five rows of its slots (blocks [b
+// tiles, (b + 1) tiles) row b), or all five.  Large inputs take all five in
 // one block: the group's set-up is then paid once, and the blocks fill the
 // GPU anyway.  Small ones take one row per block: the rows are a chain of
 // dependent loads (cell starts, records, staged tests), and with a few
 // hundred blocks in all nothing else hides their latency.
-template <bool ENS>
+template <bool ENS, bool ROW1>
 __device__ __forceinline__ void sweep_groups(const BuildView &V)
 {
     const PView &P = V.P;
@@ -559,9 +565,9 @@ __device__ __forceinline__ void sweep_groups(const BuildView &V)
     // this warp's part of the block's dynamic shared memory
     extern __shared__ float4 sweep_smem[];
     SweepWarp &W = reinterpret_cast<SweepWarp *>(sweep_smem)[wq];
-    const int part = blockIdx.x / V.sweep_tiles;
+    const int part = ROW1 ? blockIdx.x / V.sweep_tiles : 0;
     const int s = (blockIdx.x - part * V.sweep_tiles) * blockDim.x + threadIdx.x;
-    const int row_first = part * V.sweep_rows;
+    const int row_first = ROW1 ? part : 0;
     const int s0w = s - lane;
     const bool valid = s < N;
     // the full test and the store of queue entry e (the candidate's record
@@ -577,12 +583,19 @@ __device__ __forceinline__ void sweep_groups(const BuildView &V)
         const int bo = ENS ? sbat[s0w + o] : 0;
         const Grid &G = grid_ref<ENS>(G0, EG, bo);
         const int r = pair_decide(G.cutoff, wm.y, wm.x, W.own1[o], d.w, b1, d.x, d.y, d.z);
-        // inside the margin the FP64 test decides, in the next kernel
+        // inside the margin the test in float-float and FP64 decides, at the end
         if (r == kAccept)
             store_candidate(ii, jj, N, cnt, slots, ovf_n, cap, pair_i, pair_j);
-        else if (r == kUndecided)
-            defer_candidate(ii, jj, V);
+        else if (r == kUndecided) {
+            const int u = atomicAdd(&W.nund, 1);
+            if (u < kWarpUnd)
+                W.und[u] = make_int2(min(ii, jj), max(ii, jj));
+            else
+                defer_candidate(ii, jj, V);
+        }
     };
+    if (lane == 0) W.nund = 0;
+    __syncwarp();
     int b = 0, cc = 0, colkey = -1, pidx = -1;
     float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
     if (valid) {
@@ -663,7 +676,7 @@ __device__ __forceinline__ void sweep_groups(const BuildView &V)
             W.ownw[lane] = make_float2(a0.w, marg);
             W.own_i[lane] = pidx;
         }
-        for (int row = row_first; row < row_first + V.sweep_rows; ++row) {
+        for (int row = ROW1 ? row_first : 0; row < (ROW1 ? row_first + 1 : SWEEP_ROWS); ++row) {
             int dy, dz;
             row_offsets(row, dy, dz);
             int yc = lcy + dy, zc = lcz + dz;
@@ -808,16 +821,26 @@ __device__ __forceinline__ void sweep_groups(const BuildView &V)
     }
     __syncwarp();
     if (lane < qn) drain((qh + lane) & 63);
+    // the warp's candidates inside the margin, one per lane
+    __syncwarp();
+    if (lane < min(W.nund, kWarpUnd)) {
+        const int2 e = W.und[lane];
+        const int b = ENS ? batch_of(E, e.x) : 0;
+        const DView &D = dom_ref<ENS>(D0, E, b);
+        const int dec = pair_decide_ff(P, D, e.x, e.y, cutoff_d);
+        if (dec == kAccept || (dec == kUndecided && pair_test_fp64(P, D, e.x, e.y, cutoff_d)))
+            store_candidate(e.x, e.y, N, cnt, slots, ovf_n, cap, pair_i, pair_j);
+    }
 }
 
 // 64 registers: four blocks of 256 or eight of 128 per SM (the shared memory
 // follows the block: blockDim.x / 32 SweepWarp)
-template <bool ENS>
+template <bool ENS, bool ROW1>
 __global__ void __launch_bounds__(256, 4) k_pairs_sweep(const __grid_constant__ BuildView V)
 {
     pdl_wait();
     pdl_trigger();
-    sweep_groups<ENS>(V);
+    sweep_groups<ENS, ROW1>(V);
 }
 
 // The test of the candidates the sweep left inside its FP32 margin, in
@@ -1444,7 +1467,8 @@ int build_core(lub_ctx *ctx, int num_sms, void *scratch, const Grid &G, const PV
     V.sweep_rows = N <= kSweepSplitMax ? 1 : SWEEP_ROWS;
     sw.grid = V.sweep_tiles * (SWEEP_ROWS / V.sweep_rows);
     lub_trace_mark(ctx, LUB_TRACE_SWEEP, st);
-    e = launch_pdl(k_pairs_sweep<ENS>, sw.grid, sw.block, (size_t)(sw.block / 32) * sizeof(SweepWarp), st, V);
+    e = launch_pdl(V.sweep_rows == 1 ? k_pairs_sweep<ENS, true> : k_pairs_sweep<ENS, false>, sw.grid,
+                   sw.block, (size_t)(sw.block / 32) * sizeof(SweepWarp), st, V);
     lub_trace_mark(ctx, LUB_TRACE_SWEEP, st);
     if ((rc = lub_check_cuda(ctx, e, "sweep launch"))) return rc;
     e = launch_pdl(k_pairs_undecided<ENS>, num_sms, 256, 0, st, V);
