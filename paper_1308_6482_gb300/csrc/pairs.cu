@@ -389,8 +389,10 @@ constexpr int SC = 32;        // candidates a group stages per round
 constexpr float kFar = 1e18f;  // x of an unused staging entry: fails every test
 constexpr int kNone = 1 << 30;
 
-// up to this many particles the sweep takes one row per block
-constexpr int64_t kSweepSplitMax = 200000;
+// Up to this many particles the sweep takes one row per block.  Measured, the
+// ensemble step at 262,144 particles 225 us with all rows in a block and 216
+// with one; the build at 500,000 157 and 163.
+constexpr int64_t kSweepSplitMax = 350000;
 
 template <bool B>
 struct BoolTag {
@@ -1028,16 +1030,21 @@ __global__ void __launch_bounds__(256) k_pairs_compact(const __grid_constant__ B
 // Small suspensions: every pair tested, two launches
 // ---------------------------------------------------------------------------
 // Up to kSmallMax particles (one suspension) the cell grid's eight launches
-// cost more than testing all pairs: a warp per particle i tests the j > i, 32
-// at a time, by the same prefilter, tests and margins, and its ballots are
-// the row's accepted pairs in order, one word per 32 candidates (no slots, no
-// counters to clear).  A second kernel writes the list: every block sums the
-// counts itself (a few thousand integers), so no scan is launched either.
-// The tests grow with n^2: measured, the build at 64 particles took 22 us as
-// the grid's eight launches and 5 as these two, at 4,096 33 and 15.
-constexpr int kSmallMax = 4096;
-constexpr int SMALL_WARPS = 8;       // particles per block
-constexpr int SMALL_STAGE = 256;     // candidates staged at a time (one per thread)
+// cost more than testing all pairs.  A block takes 8 rows (particles i, a warp
+// each) and a chunk of 256 candidates j, staged in shared memory: every warp
+// tests its particle against those with j > i, 32 at a time, by the grid
+// sweep's prefilter, tests and margins, and its ballots are the row's accepted
+// pairs in order, one word per 32 candidates (no slots, no counters to clear).
+// A second kernel writes the list: every block sums the counts of the blocks
+// before its rows itself (a few thousand integers), so no scan is launched
+// either.  (One block per 8 rows looping over the chunks waited for each
+// chunk's loads in turn: 31 us at 2,048 particles.)
+// Measured (build alone, in a graph): 6 us at 64 particles, 9 at 256, 13 at
+// 1,024, 22 at 1,500, 30 at 2,048 (the tests grow with n^2); the cell grid
+// takes 31 us at 64 and 25 to 28 from 2,048 on.
+constexpr int kSmallMax = 1536;
+constexpr int SMALL_WARPS = 8;       // rows per block
+constexpr int SMALL_CHUNK = 256;     // candidates per block (one staged per thread)
 
 struct SmallView {
     PView P;
@@ -1046,7 +1053,9 @@ struct SmallView {
     double cutoff_d;
     uint32_t *words;  // [n][nw]: row i's accepted candidates, 32 per word
     int32_t nw;
-    int32_t *cnt;     // [n] accepted pairs per row
+    int32_t nrb, nch; // blocks of rows, chunks of candidates
+    uint16_t *cnt;    // [nch][n] accepted pairs of a row in a chunk
+    int32_t *bsum;    // [nch][nrb] accepted pairs of a block of rows in a chunk
     uint8_t *wbits;   // [n] walls, and bit 7: a semi-axis above the bound
     int32_t *pair_i, *pair_j, *d_count, *flags_out;
     int32_t cap;
@@ -1063,14 +1072,28 @@ __global__ void __launch_bounds__(32 * SMALL_WARPS) k_small_tests(const __grid_c
 {
     pdl_wait();
     pdl_trigger();
-    static_assert(SMALL_STAGE == 32 * SMALL_WARPS, "one staged candidate per thread");
-    __shared__ float4 hi_s[SMALL_STAGE];  // x, y, z and Rmax
-    __shared__ float4 lo_s[SMALL_STAGE];  // the low parts of x, y, z
+    static_assert(SMALL_CHUNK == 32 * SMALL_WARPS, "one staged candidate per thread");
+    __shared__ float4 hi_s[SMALL_CHUNK];  // x, y, z and Rmax
+    __shared__ float4 lo_s[SMALL_CHUNK];  // the low parts of x, y, z, and the coordinates' magnitude
+    __shared__ int count_s[SMALL_WARPS];
     const PView &P = V.P;
     const DView &D = V.D;
     const int n = P.n, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int i = blockIdx.x * SMALL_WARPS + w;
+    const int chunk = blockIdx.x / V.nrb, rb = blockIdx.x - chunk * V.nrb;
+    const int i = rb * SMALL_WARPS + w, j0 = chunk * SMALL_CHUNK;
     const bool live = i < n;
+    // the chunk's candidates, one per thread, fetched before the row's own data is needed
+    {
+        const int j = j0 + threadIdx.x;
+        float4 h = make_float4(NAN, 0.f, 0.f, 0.f), l = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (j < n && j0 + SMALL_CHUNK - 1 > rb * SMALL_WARPS) {
+            const ff a = ff_split_bits_nan(P.x[j]), b = ff_split_bits_nan(P.y[j]), c = ff_split_bits_nan(P.z[j]);
+            h = make_float4(a.hi, b.hi, c.hi, fmaxf(P.rpar[j], P.rperp[j]));
+            l = make_float4(a.lo, b.lo, c.lo, fabsf(a.hi) + fabsf(b.hi) + fabsf(c.hi));
+        }
+        hi_s[threadIdx.x] = h;
+        lo_s[threadIdx.x] = l;
+    }
     const ff x = ff_split_bits_nan(live ? P.x[i] : 0.0), y = ff_split_bits_nan(live ? P.y[i] : 0.0),
              z = ff_split_bits_nan(live ? P.z[i] : 0.0);
     const float rpar = live ? P.rpar[i] : 0.f, rperp = live ? P.rperp[i] : 0.f;
@@ -1081,7 +1104,7 @@ __global__ void __launch_bounds__(32 * SMALL_WARPS) k_small_tests(const __grid_c
         a1.x = o.x;
         a1.y = o.y;
         a1.z = o.z;
-        if (lane == 0) {
+        if (lane == 0 && chunk == 0) {
             // plane walls, as in the sweep
             const float rm2 = rm * rm;
             const float sz = sqrt_fast(fmaxf((a1.w > 0.f ? rm2 - a1.w : rm2) + a1.w * a1.z * a1.z, 0.f));
@@ -1106,25 +1129,9 @@ __global__ void __launch_bounds__(32 * SMALL_WARPS) k_small_tests(const __grid_c
 #pragma unroll
     for (int a = 0; a < 3; ++a) mag += D.periodic[a] ? D.Lff[a][0] : 0.f;
     int count = 0;
-    const int first = (int)(blockIdx.x * SMALL_WARPS) / SMALL_STAGE * SMALL_STAGE;  // no j > i before
+    __syncthreads();
     if (live)
-        for (int q = lane; q < first / 32; q += 32) V.words[(size_t)i * V.nw + q] = 0u;
-    for (int j0 = first; j0 < n; j0 += SMALL_STAGE) {
-        __syncthreads();
-        {
-            const int j = j0 + threadIdx.x;
-            float4 h = make_float4(NAN, 0.f, 0.f, 0.f), l = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (j < n) {
-                const ff a = ff_split_bits_nan(P.x[j]), b = ff_split_bits_nan(P.y[j]), c = ff_split_bits_nan(P.z[j]);
-                h = make_float4(a.hi, b.hi, c.hi, fmaxf(P.rpar[j], P.rperp[j]));
-                l = make_float4(a.lo, b.lo, c.lo, fabsf(a.hi) + fabsf(b.hi) + fabsf(c.hi));
-            }
-            hi_s[threadIdx.x] = h;
-            lo_s[threadIdx.x] = l;
-        }
-        __syncthreads();
-        if (!live) continue;
-        for (int c0 = 0; c0 < SMALL_STAGE && j0 + c0 < n; c0 += 32) {
+        for (int c0 = 0; c0 < SMALL_CHUNK && j0 + c0 < n; c0 += 32) {
             const int j = j0 + c0 + lane;
             bool accept = false;
             if (j0 + c0 + 31 > i) {
@@ -1151,72 +1158,81 @@ __global__ void __launch_bounds__(32 * SMALL_WARPS) k_small_tests(const __grid_c
             count += __popc(m);
             if (lane == 0) V.words[(size_t)i * V.nw + (j0 + c0) / 32] = m;
         }
+    if (lane == 0) {
+        if (live) V.cnt[(size_t)chunk * n + i] = (uint16_t)count;
+        count_s[w] = count;
     }
-    if (live && lane == 0) V.cnt[i] = count;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+#pragma unroll
+        for (int q = 0; q < SMALL_WARPS; ++q) t += count_s[q];
+        V.bsum[chunk * V.nrb + rb] = t;
+    }
 }
 
-// The list from the rows' words: each block sums the counts before its rows
-// and of all rows, then a warp per row writes the row's pairs and its walls.
-// The capacity rule is the grid build's (there the pairs beyond KSLOT per
-// particle also wait at the tail of the pair arrays).
+// The list from the rows' words: each block sums the pairs and walls before
+// its rows and all pairs, then a warp per row writes the row's pairs and its
+// walls, as far as the arrays reach.  The count follows the grid build's rule
+// (there the pairs beyond KSLOT per particle also wait at the tail of the pair
+// arrays): the first block counts those too.
 __global__ void __launch_bounds__(32 * SMALL_WARPS) k_small_list(const __grid_constant__ SmallView V)
 {
     pdl_wait();
     pdl_trigger();
     const int n = V.P.n, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int i0 = blockIdx.x * SMALL_WARPS;
-    // sums: pairs and walls before this block's rows, all pairs, all overflow; the flags
-    int s[5] = {0, 0, 0, 0, 0};
-    int64_t total = 0;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const int c = V.cnt[k], b = V.wbits[k], wn = (b & 1) + ((b >> 1) & 1);
-        if (k < i0) {
-            s[0] += c;
-            s[1] += wn;
+    const int rb = blockIdx.x, i0 = rb * SMALL_WARPS;
+    __shared__ int part[3][SMALL_WARPS];
+    auto block_sum = [&](int s[3]) {
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int v = (int)__reduce_add_sync(0xffffffffu, (unsigned)s[q]);
+            if (lane == 0) part[q][w] = v;
         }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            s[q] = 0;
+            for (int t = 0; t < SMALL_WARPS; ++t) s[q] += part[q][t];
+        }
+    };
+    // pairs and walls before this block's rows, all pairs
+    int s[3] = {0, 0, 0};
+    for (int k = threadIdx.x; k < V.nrb * V.nch; k += blockDim.x) {
+        const int c = V.bsum[k];
+        if (k % V.nrb < rb) s[0] += c;
         s[2] += c;
-        s[3] += wn + (c > KSLOT ? c - KSLOT : 0);
-        s[4] |= b & 0x80;
     }
-    __shared__ int part[5][SMALL_WARPS];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-        const int v = q < 4 ? (int)__reduce_add_sync(0xffffffffu, (unsigned)s[q])
-                            : (int)__reduce_or_sync(0xffffffffu, (unsigned)s[q]);
-        if (lane == 0) part[q][w] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-        s[q] = 0;
-        for (int t = 0; t < SMALL_WARPS; ++t) s[q] = q < 4 ? s[q] + part[q][t] : s[q] | part[q][t];
-    }
-    // (s[3] counts all walls and the overflow: what the list needs beyond the pairs)
-    total = (int64_t)s[2] + s[3];
+    for (int k = threadIdx.x; k < i0; k += blockDim.x) s[1] += __popc(V.wbits[k] & 3);
+    block_sum(s);
     const int pairs = s[2];
-    if (blockIdx.x == 0) {
-        // the walls alone, for the count
-        int walls = 0;
-        for (int k = threadIdx.x; k < n; k += blockDim.x) walls += (V.wbits[k] & 1) + ((V.wbits[k] >> 1) & 1);
-        walls = (int)__reduce_add_sync(0xffffffffu, (unsigned)walls);
-        __syncthreads();
-        if (lane == 0) part[0][w] = walls;
-        __syncthreads();
+    if (rb == 0) {
+        // all walls, the pairs beyond KSLOT per row, the flags
+        int t[3] = {0, 0, 0};
+        for (int k = threadIdx.x; k < n; k += blockDim.x) {
+            t[0] += __popc(V.wbits[k] & 3);
+            t[2] += V.wbits[k] >> 7;
+            int c = 0;
+            for (int q = 0; q < V.nch; ++q) c += V.cnt[(size_t)q * n + k];
+            if (c > KSLOT) t[1] += c - KSLOT;
+        }
+        block_sum(t);
         if (threadIdx.x == 0) {
-            walls = 0;
-            for (int t = 0; t < SMALL_WARPS; ++t) walls += part[0][t];
-            *V.d_count = total > V.cap ? (int32_t)total : pairs + walls;
-            if (V.flags_out) *V.flags_out = s[4] ? 1 : 0;
+            const int total = pairs + t[0];
+            const int64_t need = (int64_t)total + t[1];
+            *V.d_count = need > V.cap ? (int32_t)need : total;
+            if (V.flags_out) *V.flags_out = t[2] ? 1 : 0;
         }
     }
-    if (total > V.cap) return;
     const int i = i0 + w;
     if (i >= n) return;
-    int at = s[0], wat = pairs + s[1];
-    for (int k = i0; k < i; ++k) {
-        at += V.cnt[k];
-        wat += (V.wbits[k] & 1) + ((V.wbits[k] >> 1) & 1);
-    }
+    // this row's offsets: the rows of the block before it
+    int before = 0;
+    for (int e = lane; e < w * V.nch; e += 32) before += V.cnt[(size_t)(e / w) * n + i0 + e % w];
+    int at = s[0] + (int)__reduce_add_sync(0xffffffffu, (unsigned)before);
+    int wat = pairs + s[1];
+    for (int k = i0; k < i; ++k) wat += __popc(V.wbits[k] & 3);
     const uint32_t *row = V.words + (size_t)i * V.nw;
     for (int q0 = 0; q0 < V.nw; q0 += 32) {
         uint32_t m = q0 + lane < V.nw ? row[q0 + lane] : 0u;
@@ -1228,18 +1244,19 @@ __global__ void __launch_bounds__(32 * SMALL_WARPS) k_small_list(const __grid_co
             if (lane >= o) x += u;
         }
         int k = at + x - c;
-        while (m) {
+        for (; m && k < V.cap; ++k) {
             V.pair_i[k] = i;
             V.pair_j[k] = 32 * (q0 + lane) + __ffs(m) - 1;
             m &= m - 1;
-            ++k;
         }
         at += __shfl_sync(0xffffffffu, x, 31);
     }
     if (lane < 2 && (V.wbits[i] >> lane & 1)) {
         const int k = wat + (lane == 1 ? (V.wbits[i] & 1) : 0);
-        V.pair_i[k] = i;
-        V.pair_j[k] = -1 - lane;
+        if (k < V.cap) {
+            V.pair_i[k] = i;
+            V.pair_j[k] = -1 - lane;
+        }
     }
 }
 
@@ -1357,10 +1374,27 @@ Layout layout(void *base, int64_t N, int64_t ncell, bool ens = false)
     return L;
 }
 
-// the small build's workspace: words, counts, walls
+// the small build's workspace: words, counts per row and chunk and per block, walls
+struct SmallLayout {
+    int64_t nw, nrb, nch;
+    size_t words, cnt, bsum, wbits;
+};
+SmallLayout small_layout(int64_t n)
+{
+    SmallLayout L;
+    L.nw = (n + 31) / 32;
+    L.nrb = (n + SMALL_WARPS - 1) / SMALL_WARPS;
+    L.nch = (n + SMALL_CHUNK - 1) / SMALL_CHUNK;
+    L.words = align256((size_t)(n * L.nw * 4));
+    L.cnt = align256((size_t)(n * L.nch * 2));
+    L.bsum = align256((size_t)(L.nrb * L.nch * 4));
+    L.wbits = align256((size_t)n);
+    return L;
+}
 size_t small_bytes(int64_t n)
 {
-    return align256((size_t)n * ((n + 31) / 32) * 4) + align256((size_t)n * 4) + align256((size_t)n);
+    const SmallLayout L = small_layout(n);
+    return L.words + L.cnt + L.bsum + L.wbits;
 }
 
 int build_small(lub_ctx *ctx, void *scratch, const Grid &G, const PView &P, const DView &D, const lub_params &prm,
@@ -1375,25 +1409,26 @@ int build_small(lub_ctx *ctx, void *scratch, const Grid &G, const PView &P, cons
     V.margin = G.margin;
     V.rmax_bound = rmax;
     V.cutoff_d = prm.list_cutoff;
-    V.nw = (P.n + 31) / 32;
+    const SmallLayout L = small_layout(P.n);
+    V.nw = (int32_t)L.nw;
+    V.nrb = (int32_t)L.nrb;
+    V.nch = (int32_t)L.nch;
     char *b = (char *)scratch;
     V.words = (uint32_t *)b;
-    b += align256((size_t)P.n * V.nw * 4);
-    V.cnt = (int32_t *)b;
-    b += align256((size_t)P.n * 4);
-    V.wbits = (uint8_t *)b;
+    V.cnt = (uint16_t *)(b + L.words);
+    V.bsum = (int32_t *)(b + L.words + L.cnt);
+    V.wbits = (uint8_t *)(b + L.words + L.cnt + L.bsum);
     V.pair_i = pi;
     V.pair_j = pj;
     V.d_count = d_count;
     V.flags_out = flags_out;
     V.cap = cap;
-    const int grid = (P.n + SMALL_WARPS - 1) / SMALL_WARPS;
     lub_trace_mark(ctx, LUB_TRACE_SWEEP, st);
-    cudaError_t e = launch_pdl(k_small_tests, grid, 32 * SMALL_WARPS, 0, st, V);
+    cudaError_t e = launch_pdl(k_small_tests, V.nrb * V.nch, 32 * SMALL_WARPS, 0, st, V);
     lub_trace_mark(ctx, LUB_TRACE_SWEEP, st);
     int rc = lub_check_cuda(ctx, e, "small tests launch");
     if (rc) return rc;
-    e = launch_pdl(k_small_list, grid, 32 * SMALL_WARPS, 0, st, V);
+    e = launch_pdl(k_small_list, V.nrb, 32 * SMALL_WARPS, 0, st, V);
     return lub_check_cuda(ctx, e, "small list launch");
 }
 

@@ -38,7 +38,7 @@ def scattered(n, seed, periodic, walls, spread=1.0):
     return p, dict(L=(L, L, L), periodic=periodic, walls=[(0.0, 1), (L, -1)][:walls])
 
 
-@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 255, 256, 257, 1025, 4095, 4096, 4097])
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 255, 256, 257, 1025, 1535, 1536, 1537, 4097])
 @pytest.mark.parametrize("periodic,walls", [((True, True, True), 0), ((True, True, False), 2),
                                             ((False, False, False), 1)])
 def test_lists_match_the_oracle(n, periodic, walls):
