@@ -1350,6 +1350,8 @@ __global__ void __launch_bounds__(256) k_carry_ranges(const int32_t *__restrict_
                                                       const int32_t *__restrict__ q_count, int32_t qcap, int32_t n,
                                                       int2 *__restrict__ rng)
 {
+    pdl_wait();
+    pdl_trigger();
     __shared__ int seg_s;
     const int mq = pair_count(q_count, qcap);
     if (threadIdx.x == 0) seg_s = wall_segment(qj, mq);
@@ -1371,6 +1373,8 @@ __global__ void __launch_bounds__(256) k_carry_normals(const int32_t *__restrict
                                                        const int32_t *__restrict__ d_count, int32_t cap,
                                                        double *__restrict__ n)
 {
+    pdl_wait();
+    pdl_trigger();
     __shared__ int seg_s;
     const int mq = pair_count(q_count, qcap);
     if (threadIdx.x == 0) seg_s = wall_segment(qj, mq);
@@ -1427,12 +1431,15 @@ int launch_carry_normals(lub_ctx *ctx, int32_t n_particles, const int32_t *qi, c
     int rc = lub_ensure_scratch(ctx, bytes);
     if (rc) return rc;
     int2 *rng = (int2 *)ctx->scratch;
-    if ((rc = lub_check_cuda(ctx, cudaMemsetAsync(rng, 0, bytes, st), "memset ranges"))) return rc;
+    if ((rc = zero_async(ctx, ctx->num_sms, rng, bytes, st))) return rc;
+    cudaError_t e = cudaSuccess;
     if (qcap > 0)
-        k_carry_ranges<<<grid_for(qcap, 256, ctx->num_sms, 16), 256, 0, st>>>(qi, qj, q_count, qcap, n_particles, rng);
-    k_carry_normals<<<grid_for(cap, 256, ctx->num_sms, 16), 256, 0, st>>>(qi, qj, qn, q_count, qcap, rng, n_particles,
-                                                                          pi, pj, d_count, cap, n);
-    return lub_check_cuda(ctx, cudaGetLastError(), "carry launch");
+        e = launch_pdl(k_carry_ranges, grid_for(qcap, 256, ctx->num_sms, 16), 256, 0, st, qi, qj, q_count, qcap,
+                       n_particles, rng);
+    if (e == cudaSuccess)
+        e = launch_pdl(k_carry_normals, grid_for(cap, 256, ctx->num_sms, 16), 256, 0, st, qi, qj, qn, q_count, qcap,
+                       (const int2 *)rng, n_particles, pi, pj, d_count, cap, n);
+    return lub_check_cuda(ctx, e, "carry launch");
 }
 
 int launch_correct(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E, const lub_params &prm,
