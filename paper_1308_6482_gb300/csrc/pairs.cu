@@ -20,10 +20,11 @@
 //   3. the test of the candidates the sweep's FP32 tests left inside their
 //      margin, in float-float, then in FP64 inside the float-float margin
 //      (k_pairs_undecided), stored as the sweep stores pairs;
-//   4. one scan over [particle-pair counts | wall-pair counts] gives every
-//      offset (wall pairs land after all particle pairs);
-//   5. compaction: each particle sorts its partners (canonical (i, j) order)
-//      and writes them, and its wall pairs, at its offsets.
+//   4. the list: the offsets by a scan over the particles' pair and wall
+//      counts inside the same kernel (single pass, decoupled look-back; wall
+//      pairs land after all particle pairs, whose total the sweep has counted),
+//      each particle sorting its partners (canonical (i, j) order) and writing
+//      them, and its wall pairs, at its offsets.
 // The pair arrays must hold the pairs plus the overflow entries; the count
 // reports their sum when it does not fit (a capacity error, as for the pairs).
 // The tests run in FP32 on cell-relative coordinates with a safety margin; a
@@ -38,6 +39,7 @@
 
 #include "ff.cuh"
 #include "lub_internal.cuh"
+#include "scan_tile.cuh"
 
 namespace {
 
@@ -226,9 +228,9 @@ __device__ __forceinline__ void cells_fill(const BuildView &V)
     int32_t *__restrict__ cnt = V.cnt;
     unsigned long long *__restrict__ zero = V.scan_state;
     const int64_t nzero = V.z2;
-    // the sweep's counts (2N + 1) and the state of the scan after it start at zero
+    // the sweep's counts and the state of the list's scan after it start at zero
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < 2 * (int64_t)P.n + 1; k += stride) cnt[k] = 0;
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P.n; k += stride) cnt[k] = 0;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nzero; k += stride) zero[k] = 0ull;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.n; i += gridDim.x * blockDim.x) {
         const int b = ENS ? batch_of(E, i) : 0;
@@ -492,13 +494,14 @@ struct SweepWarp {
     int qt[64];       // queued: candidate slot t
     uint8_t qo[64];   // queued: lane of the particle
     int2 und[kWarpUnd];  // candidates inside the FP32 margin (smaller, larger index)
-    int nund, pad;       // how many there were
+    int nund;            // how many there were
+    int nacc;            // accepted pairs
 };
 static_assert(sizeof(SweepWarp) % 16 == 0, "warp blocks stay 16-byte aligned");
 
 // One thread per slot s (cell order); the thread also tests its particle's
-// walls.  cnt: [0, N) pair counts per particle (of the smaller index of each
-// pair), [N, 2N) wall-pair counts; slots [KSLOT][N] (slot-major, so that the
+// walls.  cnt: pair counts per particle (of the smaller index of each
+// pair); totals[4], [5]: all pairs and wall pairs; slots [KSLOT][N] (slot-major, so that the
 // compaction's reads of the first few slots of consecutive particles are
 // coalesced and touch only the slots in use); wall bits per particle;
 // overflow entry o at pair_i/pair_j[cap - 1 - o].
@@ -586,9 +589,10 @@ __device__ __forceinline__ void sweep_groups(const BuildView &V)
         const Grid &G = grid_ref<ENS>(G0, EG, bo);
         const int r = pair_decide(G.cutoff, wm.y, wm.x, W.own1[o], d.w, b1, d.x, d.y, d.z);
         // inside the margin the test in float-float and FP64 decides, at the end
-        if (r == kAccept)
+        if (r == kAccept) {
+            atomicAdd(&W.nacc, 1);
             store_candidate(ii, jj, N, cnt, slots, ovf_n, cap, pair_i, pair_j);
-        else if (r == kUndecided) {
+        } else if (r == kUndecided) {
             const int u = atomicAdd(&W.nund, 1);
             if (u < kWarpUnd)
                 W.und[u] = make_int2(min(ii, jj), max(ii, jj));
@@ -596,9 +600,9 @@ __device__ __forceinline__ void sweep_groups(const BuildView &V)
                 defer_candidate(ii, jj, V);
         }
     };
-    if (lane == 0) W.nund = 0;
+    if (lane == 0) W.nund = W.nacc = 0;
     __syncwarp();
-    int b = 0, cc = 0, colkey = -1, pidx = -1;
+    int b = 0, cc = 0, colkey = -1, pidx = -1, walls = 0;
     float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
     if (valid) {
         b = ENS ? sbat[s] : 0;
@@ -635,9 +639,13 @@ __device__ __forceinline__ void sweep_groups(const BuildView &V)
                     ++wf;
                 }
             }
-            cnt[N + i] = wf;
             wbits[i] = (uint8_t)bits;
+            walls = wf;
         }
+    }
+    if (row_first == 0) {  // (the same for the whole block)
+        walls = (int)__reduce_add_sync(FULL, (unsigned)walls);
+        if (lane == 0 && walls) atomicAdd(V.totals + 5, walls);
     }
     const int cx = cc & 1023;
     float4 *const cg = &W.cand[g * (SC + 1)];
@@ -830,9 +838,13 @@ __device__ __forceinline__ void sweep_groups(const BuildView &V)
         const int b = ENS ? batch_of(E, e.x) : 0;
         const DView &D = dom_ref<ENS>(D0, E, b);
         const int dec = pair_decide_ff(P, D, e.x, e.y, cutoff_d);
-        if (dec == kAccept || (dec == kUndecided && pair_test_fp64(P, D, e.x, e.y, cutoff_d)))
+        if (dec == kAccept || (dec == kUndecided && pair_test_fp64(P, D, e.x, e.y, cutoff_d))) {
+            atomicAdd(&W.nacc, 1);
             store_candidate(e.x, e.y, N, cnt, slots, ovf_n, cap, pair_i, pair_j);
+        }
     }
+    __syncwarp();
+    if (lane == 0 && W.nacc) atomicAdd(V.totals + 4, W.nacc);
 }
 
 // 64 registers: four blocks of 256 or eight of 128 per SM (the shared memory
@@ -880,6 +892,7 @@ __global__ void __launch_bounds__(256) k_pairs_undecided(const __grid_constant__
         bool keep = false;  // accepted beyond the slots
         if (dec == kAccept || (dec == kUndecided && pair_test_fp64(V.P, D, lo, hi, V.cutoff_d))) {
             const int q = atomicAdd(V.cnt + lo, 1);
+            atomicAdd(V.totals + 4, 1);
             if (q < KSLOT)
                 V.slots[(size_t)q * N + lo] = hi;
             else
@@ -892,64 +905,185 @@ __global__ void __launch_bounds__(256) k_pairs_undecided(const __grid_constant__
     }
 }
 
-// Canonical order: each particle's partners, sorted, then its wall pairs, at
-// the offsets of the scan (off = the scanned counts, off[2N] = the total).
-// The count is the total, or total + overflow entries when they do not fit.
-__device__ __forceinline__ void pairs_compact(const BuildView &V)
+// The list's scan state: a ticket, then one word per tile of 256 G particles:
+// flag (bits 62, 63) | walls (31 bits) | pairs (31 bits) of the tile, or of all
+// tiles up to it.
+constexpr unsigned long long EM_AGG = 1ull << 62, EM_PREFIX = 2ull << 62, EM_VALUE = (1ull << 62) - 1;
+constexpr int64_t kEmitLarge = 262144;  // from here on a warp takes 4 x 32 particles (fewer tiles to look back over)
+inline int64_t emit_tiles(int64_t n)
 {
+    const int64_t t = n >= kEmitLarge ? 1024 : 256;
+    return (n + t - 1) / t;
+}
+
+// The sums of all tiles before `tile`, by one warp: its own total published
+// first, then a look back over 32 tiles at a time to the nearest published
+// prefix (decoupled look-back, Merrill & Garland 2016; tiles are taken by
+// ticket, so a tile only waits on running blocks), then its own prefix.
+// Bounded: on timeout sets bit 2 of the flags and carries on.
+__device__ __forceinline__ unsigned long long emit_prefix(unsigned long long *state, int tile, unsigned long long own,
+                                                          int32_t *flags, int32_t *flags_out)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned long long excl = 0;
+    if (tile > 0) {
+        if (lane == 0) atomicExch(state + tile, EM_AGG | own);
+        long spins = 0;
+        int top = tile - 1;
+        while (true) {
+            const int p = top - lane;
+            const unsigned long long w = p >= 0 ? scan_tile::load_state(state + p) : EM_PREFIX;
+            const unsigned pre = __ballot_sync(0xffffffffu, (w & EM_PREFIX) != 0);
+            const unsigned none = __ballot_sync(0xffffffffu, (w >> 62) == 0);
+            const int stop = pre ? __ffs(pre) - 1 : 32;
+            const unsigned upto = stop == 32 ? 0xffffffffu : ((2u << stop) - 1u);
+            if (none & upto) {
+                if (++spins > scan_tile::kSpinLimit) {
+                    if (lane == 0) {
+                        atomicOr(flags, 4);
+                        if (flags_out) {
+                            atomicOr(flags_out, 4);
+                            atomicOr(flags_out + 1, 4);
+                        }
+                    }
+                    break;
+                }
+                continue;
+            }
+            unsigned long long x = lane <= stop ? w & EM_VALUE : 0ull;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            excl += x;
+            if (stop < 32) break;
+            top -= 32;
+        }
+    }
+    if (lane == 0) atomicExch(state + tile, EM_PREFIX | ((excl + own) & EM_VALUE));
+    return excl;
+}
+
+// The list, in canonical order: each particle's partners, sorted, then (after
+// all particle pairs) the wall pairs.  The count is the total, or total +
+// overflow entries when they do not fit; both totals come from the sweep, so
+// every block knows them at once.  The scan and the write share one kernel
+// (a scan kernel before it cost a launch and another pass over the counts,
+// some 2 to 5 us: the step at 32,768 particles 53.2 -> 51.3 us, at 1,048,576
+// 829 -> 824).
+template <int G>
+__global__ void __launch_bounds__(256) k_pairs_emit(const __grid_constant__ BuildView V)
+{
+    pdl_wait();
+    pdl_trigger();
     const int32_t n = V.P.n;
-    const int32_t *__restrict__ off = V.cnt;
+    const int32_t *__restrict__ cnt = V.cnt;
     const int32_t *__restrict__ slots = V.slots;
     const uint8_t *__restrict__ wbits = V.wbits;
-    const int32_t *__restrict__ ovf_n = V.totals + 2;
     const int32_t cap = V.cap;
     int32_t *__restrict__ pair_i = V.pair_i;
     int32_t *__restrict__ pair_j = V.pair_j;
-    int32_t *__restrict__ d_count = V.d_count;
-    const int32_t *__restrict__ flags = V.flags;
-    int32_t *__restrict__ flags_out = V.flags_out;
-    const int total = off[2 * n];
-    const int novf = *ovf_n;
-    const int64_t need = (int64_t)total + novf;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *d_count = need > cap ? (int32_t)(need < (int64_t)INT32_MAX ? need : (int64_t)INT32_MAX) : total;
-        if (flags_out) {
-            *flags_out = *flags;  // this build's flags, for the host-count path
-            if (*flags & 4) atomicOr(flags_out + 1, 4);  // a timed-out wait, for lub_sync_status
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    __shared__ int tile_s;
+    __shared__ int2 warp_s[8];
+    __shared__ unsigned long long prefix_s;
+    if (threadIdx.x == 0) tile_s = (int)atomicAdd(V.scan_state, 1ull);
+    const int all_pairs = V.totals[4], novf = V.totals[2];
+    const int64_t total = (int64_t)all_pairs + V.totals[5], need = total + novf;
+    __syncthreads();
+    const int tile = tile_s;
+    if (tile == 0 && threadIdx.x == 0) {
+        *V.d_count = need > cap ? (int32_t)(need < (int64_t)INT32_MAX ? need : (int64_t)INT32_MAX) : (int32_t)total;
+        // this build's flags, for the host-count path (before this tile
+        // publishes, so before any look-back can time out)
+        if (V.flags_out) {
+            *V.flags_out = *V.flags;
+            if (*V.flags & 4) atomicOr(V.flags_out + 1, 4);  // a timed-out wait, for lub_sync_status
+            __threadfence();
         }
     }
     if (need > cap) return;
-    // each warp's pairs are one run of the output (its particles are
-    // consecutive): staged in shared memory and stored as whole runs, unless
-    // a particle of the warp has more pairs than slots (then every lane
-    // stores its own)
+    // the counts of the warp's particles and their places within the warp
+    const int p0 = (tile * 8 + w) * 32 * G;
+    int m[G], rel[G], bits[G], wrel[G];
+    int tp = 0, tw = 0;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        const int i = p0 + 32 * g + lane;
+        m[g] = i < n ? cnt[i] : 0;
+        bits[g] = i < n ? wbits[i] & 3 : 0;
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        int x = m[g];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        rel[g] = tp + x - m[g];
+        tp += __shfl_sync(0xffffffffu, x, 31);
+        const unsigned b0 = __ballot_sync(0xffffffffu, bits[g] & 1), b1 = __ballot_sync(0xffffffffu, bits[g] & 2);
+        wrel[g] = tw + __popc(b0 & below) + __popc(b1 & below);
+        tw += __popc(b0) + __popc(b1);
+    }
+    if (lane == 0) warp_s[w] = make_int2(tp, tw);
+    __syncthreads();
+    int bp = 0, bw = 0, op = 0, ow = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int2 v = warp_s[q];
+        if (q < w) {
+            op += v.x;
+            ow += v.y;
+        }
+        bp += v.x;
+        bw += v.y;
+    }
+    if (w == 0) {
+        const unsigned long long ex = emit_prefix(V.scan_state + 1, tile,
+                                                  (unsigned long long)bp | (unsigned long long)bw << 31, V.flags,
+                                                  V.flags_out);
+        if (lane == 0) prefix_s = ex;
+    }
+    __syncthreads();
+    const int pp = (int)(prefix_s & 0x7fffffffull) + op, pw = (int)(prefix_s >> 31 & 0x7fffffffull) + ow;
+    // each group of 32 particles' pairs are one run of the output: staged in
+    // shared memory and stored as whole runs, unless a particle has more
+    // pairs than slots (then every lane stores its own)
     __shared__ int2 stage[8][32 * KSLOT];
-    int2 *const sg = stage[threadIdx.x >> 5];
-    const int lane = threadIdx.x & 31;
-    // warp-uniform loop bound: every lane of a warp takes part in the
-    // warp's reductions and its staged stores
-    const int n_up = (n + 31) & ~31;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_up; i += gridDim.x * blockDim.x) {
+    int2 *const sg = stage[w];
+#pragma unroll 1
+    for (int g = 0; g < G; ++g) {
+        const int i = p0 + 32 * g + lane;
         const bool live = i < n;
-        const int b = live ? off[i] : 0, m = live ? off[i + 1] - b : 0;
-        // the unrolled slot loads and pair stores stop at the warp's largest
-        // count (mostly 4..8 of the 16), so the loads and stores beyond it
-        // are skipped, not issued with every lane predicated off
-        const int mw = __reduce_max_sync(0xffffffffu, m < KSLOT ? m : KSLOT);
-        if (!__any_sync(0xffffffffu, m > KSLOT)) {
-            // sort in registers: compare-exchange passes (m is small, mostly 0..4)
+        // (selected, not indexed: the arrays stay in registers)
+        int mi = 0, ri = 0, bi = 0, wi = 0;
+#pragma unroll
+        for (int q = 0; q < G; ++q)
+            if (q == g) {
+                mi = m[q];
+                ri = rel[q];
+                bi = bits[q];
+                wi = wrel[q];
+            }
+        const int b = pp + ri;
+        // the slot loads and the sort's passes stop at the warp's largest
+        // count (mostly 4..8 of the 16)
+        const int mw = __reduce_max_sync(0xffffffffu, mi < KSLOT ? mi : KSLOT);
+        if (!__any_sync(0xffffffffu, mi > KSLOT)) {
+            // sort in registers: compare-exchange passes (mi is small, mostly 0..4)
             int v[KSLOT];
 #pragma unroll
             for (int q = 0; q < KSLOT; ++q) v[q] = INT32_MAX;
 #pragma unroll
             for (int q = 0; q < KSLOT; ++q) {
                 if (q >= mw) break;
-                if (q < m) v[q] = slots[(size_t)q * n + i];
+                if (q < mi) v[q] = slots[(size_t)q * n + i];
             }
-            if (m > 1) {
+            if (mi > 1) {
 #pragma unroll
                 for (int q = 1; q < KSLOT; ++q) {
-                    if (q >= m) break;
+                    if (q >= mi) break;
 #pragma unroll
                     for (int r = q; r > 0; --r) {
                         const int x = v[r - 1], y = v[r];
@@ -958,45 +1092,44 @@ __device__ __forceinline__ void pairs_compact(const BuildView &V)
                     }
                 }
             }
-            // lane 0 is live whenever any lane is (i grows with the lane)
-            const int b0 = __shfl_sync(0xffffffffu, b, 0);
-            const int tw = (int)__reduce_max_sync(0xffffffffu, (unsigned)(live ? b + m - b0 : 0));
+            const int r0 = __shfl_sync(0xffffffffu, ri, 0);
+            const int tot = __shfl_sync(0xffffffffu, ri + mi, 31) - r0;
 #pragma unroll
             for (int q = 0; q < KSLOT; ++q) {
                 if (q >= mw) break;
-                if (q < m) sg[b - b0 + q] = make_int2(i, v[q]);
+                if (q < mi) sg[ri - r0 + q] = make_int2(i, v[q]);
             }
             __syncwarp();
-            for (int t = lane; t < tw; t += 32) {
+            for (int t = lane; t < tot; t += 32) {
                 const int2 e = sg[t];
-                pair_i[b0 + t] = e.x;
-                pair_j[b0 + t] = e.y;
+                pair_i[pp + r0 + t] = e.x;
+                pair_j[pp + r0 + t] = e.y;
             }
             __syncwarp();
         } else if (live) {
             // the slots, then (beyond them) this particle's entries at the
             // tail and among the candidates the FP64 test accepted, then
             // sort in place
-            const int ms = m < KSLOT ? m : KSLOT;
+            const int ms = mi < KSLOT ? mi : KSLOT;
             for (int q = 0; q < ms; ++q) {
                 pair_i[b + q] = i;
                 pair_j[b + q] = slots[(size_t)q * n + i];
             }
             int c = ms;
-            for (int o = 0; o < novf && c < m; ++o)
+            for (int o = 0; o < novf && c < mi; ++o)
                 if (pair_i[cap - 1 - o] == i) {
                     pair_j[b + c] = pair_j[cap - 1 - o];
                     pair_i[b + c] = i;
                     ++c;
                 }
             const int nu = min(V.totals[3], V.und_cap);
-            for (int u = 0; u < nu && c < m; ++u)
+            for (int u = 0; u < nu && c < mi; ++u)
                 if (V.und[u].x == i) {
                     pair_j[b + c] = V.und[u].y;
                     pair_i[b + c] = i;
                     ++c;
                 }
-            for (int a = b + 1; a < b + m; ++a) {
+            for (int a = b + 1; a < b + mi; ++a) {
                 const int x = pair_j[a];
                 int q = a - 1;
                 while (q >= b && pair_j[q] > x) {
@@ -1006,24 +1139,14 @@ __device__ __forceinline__ void pairs_compact(const BuildView &V)
                 pair_j[q + 1] = x;
             }
         }
-        if (!live) continue;
-        const int wb = off[n + i];
-        const int bits = wbits[i];
-        int c = 0;
-        for (int w = 0; w < 2; ++w)
-            if (bits & (1 << w)) {
-                pair_i[wb + c] = i;
-                pair_j[wb + c] = -1 - w;
-                ++c;
+        int k = all_pairs + pw + wi;
+        for (int q = 0; q < 2; ++q)
+            if (bi & (1 << q)) {
+                pair_i[k] = i;
+                pair_j[k] = -1 - q;
+                ++k;
             }
     }
-}
-
-__global__ void __launch_bounds__(256) k_pairs_compact(const __grid_constant__ BuildView V)
-{
-    pdl_wait();
-    pdl_trigger();
-    pairs_compact(V);
 }
 
 // ---------------------------------------------------------------------------
@@ -1334,15 +1457,17 @@ struct Layout {
 
 Layout layout(void *base, int64_t N, int64_t ncell, bool ens = false)
 {
-    const size_t b_cell = align256((ncell + 1) * 4), b_n = align256((N + 1) * 4), b_n2 = align256((2 * N + 1) * 4);
+    const size_t b_cell = align256((ncell + 1) * 4), b_n = align256((N + 1) * 4), b_cnt = align256((N + 1) * 4);
     const size_t b_slots = align256((size_t)N * KSLOT * 4), b_bits = align256((size_t)N + 1);
-    const size_t b_rec = align256(N * 16),
-                 b_tmp = align256(scan_tmp_bytes(ncell + 1 > 2 * N + 1 ? ncell + 1 : 2 * N + 1));
+    // the cell scan's state, then the list's
+    const size_t b_scan = scan_tmp_bytes(ncell + 1), b_emit = (size_t)(emit_tiles(N) + 1) * 8;
+    const size_t b_rec = align256(N * 16), b_tmp = align256(b_scan > b_emit ? b_scan : b_emit);
     Layout L;
     char *s = (char *)base;
     L.flags = (int32_t *)s;
     s += 256;
-    L.totals = (int32_t *)s;  // [0] all pairs, [1] cells, [2] tail entries, [3] candidates left to FP64
+    L.totals = (int32_t *)s;  // [1] cells, [2] tail entries, [3] candidates left over,
+                              // [4] pairs, [5] wall pairs
     s += 256;
     L.cell_cnt = (int32_t *)s;
     s += b_cell;
@@ -1357,7 +1482,7 @@ Layout layout(void *base, int64_t N, int64_t ncell, bool ens = false)
     L.sbat = (int32_t *)s;  // suspension of each slot (ensemble mode only)
     if (ens) s += b_n;
     L.cnt = (int32_t *)s;
-    s += b_n2;
+    s += b_cnt;
     L.slots = (int32_t *)s;
     L.rel = (float4 *)s;  // shares the slots' storage: read by the cells fill, before the sweep fills the slots
     s += b_slots;
@@ -1473,7 +1598,7 @@ int build_core(lub_ctx *ctx, int num_sms, void *scratch, const Grid &G, const PV
     V.rec1 = L.rec1;
     V.scan_state = (unsigned long long *)L.tmp;
     V.z1 = scan_state_words(G.ncell + 1);
-    V.z2 = scan_state_words(2 * N + 1);
+    V.z2 = emit_tiles(N) + 1;
     V.cutoff_d = prm.list_cutoff;
     V.pair_i = pi;
     V.pair_j = pj;
@@ -1508,10 +1633,8 @@ int build_core(lub_ctx *ctx, int num_sms, void *scratch, const Grid &G, const PV
     if ((rc = lub_check_cuda(ctx, e, "sweep launch"))) return rc;
     e = launch_pdl(k_pairs_undecided<ENS>, num_sms, 256, 0, st, V);
     if ((rc = lub_check_cuda(ctx, e, "undecided pairs launch"))) return rc;
-    // one scan over [particle pairs | wall pairs] (+1 entry: the end of the last run)
-    if ((rc = scan_exclusive(ctx, L.cnt, 2 * N + 1, L.totals + 0, L.tmp, L.tmp_bytes, st, L.flags, true))) return rc;
-    e = launch_pdl(k_pairs_compact, grid_for(N, 256, num_sms, 32), 256, 0, st, V);
-    return lub_check_cuda(ctx, e, "pairs compact launch");
+    e = launch_pdl(N >= kEmitLarge ? k_pairs_emit<4> : k_pairs_emit<1>, (int)emit_tiles(N), 256, 0, st, V);
+    return lub_check_cuda(ctx, e, "pairs list launch");
 }
 
 }  // namespace
