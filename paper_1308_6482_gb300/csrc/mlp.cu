@@ -72,9 +72,35 @@ __device__ __forceinline__ float2 gelu_both(float x)
 // forward product along its rows (lane's columns lane + 32 j) and the backward
 // one along its columns (4 lane ..): the row stride of 132 floats keeps both,
 // and the activations' rows, free of bank conflicts.  Measured: forward,
-// backward and Adam on 8,192 samples in 44 us, against 1,559 us for one launch
+// backward and Adam on 8,192 samples in 37 us (44 with scalar multiply-adds
+// and the weights and targets fetched one by one), against 1,559 us for one launch
 // per layer and direction (32 x 32 tiles, each weight gradient summed over
 // the whole batch by a single block per tile).
+// Two FP32 multiply-adds in one instruction (each lane rounded as by itself).
+// It does not raise the FP32 rate, but it halves the issue slots, which the
+// shared-memory loads share.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_pack(float a, float b)
+{
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 f2_get(f2 a)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c)
+{
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// four consecutive floats (16-byte aligned) as two pairs
+__device__ __forceinline__ ulonglong2 f2_load4(const float *p) { return *reinterpret_cast<const ulonglong2 *>(p); }
+
 constexpr int TLD = 132;  // row stride of W2 and the activations (floats)
 
 template <int RW>
@@ -85,6 +111,7 @@ struct TrainSmem {
     float W1t[NI * NH];                        // [k][n]
     float W3[NO * NH];
     float x[8 * RW * NI];
+    float tg[8 * RW * NO], wg[8 * RW * NO];    // targets and loss weights
     float dy[8 * RW * NO];
     float b1[NH], b2[NH], b3[NO];
 };
@@ -102,8 +129,21 @@ __global__ void __launch_bounds__(256, 1) k_mlp_train(const float *__restrict__ 
     const float *W1 = params, *b1 = W1 + NH * NI, *W2 = b1 + NH, *b2 = W2 + NH * NH, *W3 = b2 + NH, *b3 = W3 + NO * NH;
     pdl_wait();
     pdl_trigger();
-    for (int e = tid; e < NH * NH; e += 256) S.W2[(e >> 7) * TLD + (e & 127)] = W2[e];
+    static_assert(R * NO <= 256, "one target per thread");
+    // (W2 starts 6,656 bytes into the parameters: as aligned as they are)
+    if (((uintptr_t)W2 & 15u) == 0) {
+#pragma unroll
+        for (int t = 0; t < NH * NH / 1024; ++t) {
+            const int e = 4 * (tid + 256 * t);
+            *reinterpret_cast<float4 *>(&S.W2[(e >> 7) * TLD + (e & 127)]) = *reinterpret_cast<const float4 *>(W2 + e);
+        }
+    } else {
+#pragma unroll 16
+        for (int e = tid; e < NH * NH; e += 256) S.W2[(e >> 7) * TLD + (e & 127)] = W2[e];
+    }
+#pragma unroll
     for (int e = tid; e < NH * NI; e += 256) S.W1t[(e % NI) * NH + e / NI] = W1[e];
+#pragma unroll
     for (int e = tid; e < NO * NH; e += 256) S.W3[e] = W3[e];
     if (tid < NH) {
         S.b1[tid] = b1[tid];
@@ -114,17 +154,24 @@ __global__ void __launch_bounds__(256, 1) k_mlp_train(const float *__restrict__ 
     // dW2 rows {4 tn + a, 64 + 4 tn + a} x columns {4 tk + b, 64 + 4 tk + b};
     // dW3 rows 2 hf, 2 hf + 1 and dW1 columns 6 hf .. of row (column) cn
     const int tn = tid >> 4, tk = tid & 15, cn = tid & 127, hf = tid >> 7;
-    float g2a[8][8], g3a[2] = {0.f, 0.f}, g1a[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, gba = 0.f, gb3 = 0.f;
+    f2 g2a[8][4];  // (pairs of columns)
+    float g3a[2] = {0.f, 0.f}, g1a[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, gba = 0.f, gb3 = 0.f;
 #pragma unroll
     for (int a = 0; a < 8; ++a)
 #pragma unroll
-        for (int b = 0; b < 8; ++b) g2a[a][b] = 0.f;
+        for (int b = 0; b < 4; ++b) g2a[a][b] = 0ull;
     const float inv_m = 1.0f / (float)M;
     for (int base = blockIdx.x * R; base < M; base += gridDim.x * R) {
         __syncthreads();  // the weights are staged; the tile before is used up
         for (int e = tid; e < R * NI; e += 256) {
             const int64_t at = (int64_t)base * NI + e;
             S.x[e] = at < (int64_t)M * NI ? x[at] : 0.f;
+        }
+        if (tid < R * NO) {
+            const int64_t at = (int64_t)base * NO + tid;
+            const bool in = at < (int64_t)M * NO;
+            S.tg[tid] = in ? tgt[at] : 0.f;
+            S.wg[tid] = in ? (wgt ? wgt[at] : 1.f) : 0.f;
         }
         __syncthreads();
         // layer 1: z1 = x W1^T + b1, columns lane + 32 j
@@ -158,34 +205,30 @@ __global__ void __launch_bounds__(256, 1) k_mlp_train(const float *__restrict__ 
         __syncwarp();
         // layer 2: z2 = h1 W2^T + b2, columns lane + 32 j
         {
-            float acc[RW][4];
+            // (the sums over even and odd k side by side)
+            f2 acc[RW][4];
 #pragma unroll
             for (int q = 0; q < RW; ++q)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[q][j] = S.b2[lane + 32 * j];
+                for (int j = 0; j < 4; ++j) acc[q][j] = f2_pack(S.b2[lane + 32 * j], 0.f);
 #pragma unroll 2
             for (int k = 0; k < NH; k += 4) {
-                float4 wv[4];
+                ulonglong2 wv[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    wv[j] = *reinterpret_cast<const float4 *>(&S.W2[(lane + 32 * j) * TLD + k]);
+                for (int j = 0; j < 4; ++j) wv[j] = f2_load4(&S.W2[(lane + 32 * j) * TLD + k]);
 #pragma unroll
                 for (int q = 0; q < RW; ++q) {
-                    const float4 a = *reinterpret_cast<const float4 *>(&S.h1[(r0 + q) * TLD + k]);
+                    const ulonglong2 a = f2_load4(&S.h1[(r0 + q) * TLD + k]);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        acc[q][j] = fmaf(a.x, wv[j].x, acc[q][j]);
-                        acc[q][j] = fmaf(a.y, wv[j].y, acc[q][j]);
-                        acc[q][j] = fmaf(a.z, wv[j].z, acc[q][j]);
-                        acc[q][j] = fmaf(a.w, wv[j].w, acc[q][j]);
-                    }
+                    for (int j = 0; j < 4; ++j) acc[q][j] = f2_fma(a.y, wv[j].y, f2_fma(a.x, wv[j].x, acc[q][j]));
                 }
             }
 #pragma unroll
             for (int q = 0; q < RW; ++q)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float2 g = gelu_both(acc[q][j]);
+                    const float2 z = f2_get(acc[q][j]);
+                    const float2 g = gelu_both(z.x + z.y);
                     S.h2[(r0 + q) * TLD + lane + 32 * j] = g.x;
                     S.d2[(r0 + q) * TLD + lane + 32 * j] = g.y;
                 }
@@ -213,9 +256,9 @@ __global__ void __launch_bounds__(256, 1) k_mlp_train(const float *__restrict__ 
                     float l = 0.f;
 #pragma unroll
                     for (int o = 0; o < NO; ++o) {
-                        float r = y[o] + S.b3[o] - tgt[(size_t)m * NO + o];
+                        float r = y[o] + S.b3[o] - S.tg[(r0 + q) * NO + o];
                         if (o & 1) r = wrap_pi_f(r);
-                        const float wg = wgt ? wgt[(size_t)m * NO + o] : 1.f;
+                        const float wg = S.wg[(r0 + q) * NO + o];
                         l += 0.5f * wg * r * r;
                         dyv[o] = wg * r * inv_m;
                     }
@@ -235,36 +278,35 @@ __global__ void __launch_bounds__(256, 1) k_mlp_train(const float *__restrict__ 
         __syncwarp();
         // d1 = (d2 W2) gelu'(z1): lane's columns 4 lane .., in place of g1
         {
-            float4 acc[RW];
+            f2 acc[RW][2];
 #pragma unroll
-            for (int q = 0; q < RW; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int q = 0; q < RW; ++q) acc[q][0] = acc[q][1] = 0ull;
 #pragma unroll 2
             for (int n = 0; n < NH; n += 4) {
-                float4 wv[4];
+                ulonglong2 wv[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    wv[j] = *reinterpret_cast<const float4 *>(&S.W2[(n + j) * TLD + 4 * lane]);
+                for (int j = 0; j < 4; ++j) wv[j] = f2_load4(&S.W2[(n + j) * TLD + 4 * lane]);
 #pragma unroll
                 for (int q = 0; q < RW; ++q) {
                     const float4 a = *reinterpret_cast<const float4 *>(&S.d2[(r0 + q) * TLD + n]);
                     const float av[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        acc[q].x = fmaf(av[j], wv[j].x, acc[q].x);
-                        acc[q].y = fmaf(av[j], wv[j].y, acc[q].y);
-                        acc[q].z = fmaf(av[j], wv[j].z, acc[q].z);
-                        acc[q].w = fmaf(av[j], wv[j].w, acc[q].w);
+                        const f2 aa = f2_pack(av[j], av[j]);
+                        acc[q][0] = f2_fma(aa, wv[j].x, acc[q][0]);
+                        acc[q][1] = f2_fma(aa, wv[j].y, acc[q][1]);
                     }
                 }
             }
 #pragma unroll
             for (int q = 0; q < RW; ++q) {
                 float4 *gp = reinterpret_cast<float4 *>(&S.g1[(r0 + q) * TLD + 4 * lane]);
+                const float2 u = f2_get(acc[q][0]), v = f2_get(acc[q][1]);
                 float4 g = *gp;
-                g.x *= acc[q].x;
-                g.y *= acc[q].y;
-                g.z *= acc[q].z;
-                g.w *= acc[q].w;
+                g.x *= u.x;
+                g.y *= u.y;
+                g.z *= v.x;
+                g.w *= v.y;
                 *gp = g;
             }
         }
@@ -274,14 +316,15 @@ __global__ void __launch_bounds__(256, 1) k_mlp_train(const float *__restrict__ 
         for (int m = 0; m < R; ++m) {
             const float4 p0 = *reinterpret_cast<const float4 *>(&S.d2[m * TLD + 4 * tn]);
             const float4 p1 = *reinterpret_cast<const float4 *>(&S.d2[m * TLD + 64 + 4 * tn]);
-            const float4 q0 = *reinterpret_cast<const float4 *>(&S.h1[m * TLD + 4 * tk]);
-            const float4 q1 = *reinterpret_cast<const float4 *>(&S.h1[m * TLD + 64 + 4 * tk]);
+            const ulonglong2 q0 = f2_load4(&S.h1[m * TLD + 4 * tk]), q1 = f2_load4(&S.h1[m * TLD + 64 + 4 * tk]);
             const float pv[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
-            const float qv[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+            const f2 qv[4] = {q0.x, q0.y, q1.x, q1.y};
 #pragma unroll
-            for (int a = 0; a < 8; ++a)
+            for (int a = 0; a < 8; ++a) {
+                const f2 pp = f2_pack(pv[a], pv[a]);
 #pragma unroll
-                for (int b = 0; b < 8; ++b) g2a[a][b] = fmaf(pv[a], qv[b], g2a[a][b]);
+                for (int b = 0; b < 4; ++b) g2a[a][b] = f2_fma(pp, qv[b], g2a[a][b]);
+            }
         }
 #pragma unroll 4
         for (int m = 0; m < R; ++m) {
@@ -306,8 +349,12 @@ __global__ void __launch_bounds__(256, 1) k_mlp_train(const float *__restrict__ 
 #pragma unroll
     for (int a = 0; a < 8; ++a)
 #pragma unroll
-        for (int b = 0; b < 8; ++b)
-            oW2[(4 * tn + (a & 3) + 64 * (a >> 2)) * NH + 4 * tk + (b & 3) + 64 * (b >> 2)] = g2a[a][b];
+        for (int b = 0; b < 4; ++b) {
+            const float2 v = f2_get(g2a[a][b]);
+            float *const o = &oW2[(4 * tn + (a & 3) + 64 * (a >> 2)) * NH + 4 * tk + 2 * (b & 1) + 64 * (b >> 1)];
+            o[0] = v.x;
+            o[1] = v.y;
+        }
     oW3[(2 * hf) * NH + cn] = g3a[0];
     oW3[(2 * hf + 1) * NH + cn] = g3a[1];
 #pragma unroll
