@@ -559,9 +559,10 @@ __device__ __forceinline__ void tc_hidden_epilogue(uint32_t trow, int c0, const 
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// the network's start normal for each pair of a tile (used by closest.cu)
+// the network's start normal for each pair of a tile (used by closest.cu),
+// or (PQ) its outputs
 // ---------------------------------------------------------------------------
-template <bool ENS>
+template <bool ENS, bool PQ>
 __global__ void __launch_bounds__(32 * INF_WARPS, 2) k_mlp_start(PView P, const __grid_constant__ DView D0, Ens E, const int32_t *__restrict__ pi,
                                                                 const int32_t *__restrict__ pj,
                                                                 const int32_t *__restrict__ d_count, int32_t cap,
@@ -580,9 +581,15 @@ __global__ void __launch_bounds__(32 * INF_WARPS, 2) k_mlp_start(PView P, const 
     for (int base = (blockIdx.x * INF_WARPS + w) * 32; base < count; base += gridDim.x * INF_WARPS * 32) {
         const int k = base + lane;
         float f[NI];
-        PairIn in = pair_inputs<ENS>(P, D0, E, pi, pj, k, count, S.mean, S.istd, f);
-        const float4 y = warp_mlp(S, S.x[w], S.y[w], f, lane);
-        pair_outputs(P, in, y, k, count, C, n0, pq);
+        if (PQ) {
+            PairIn in = pair_inputs<ENS>(P, D0, E, pi, pj, k, count, S.mean, S.istd, f);
+            const float4 y = warp_mlp(S, S.x[w], S.y[w], f, lane);
+            pair_outputs(P, in, y, k, count, C, n0, pq);
+        } else {
+            const bool ok = start_inputs<ENS>(P, D0, E, pi, pj, k, count, S.mean, S.istd, f, &S.geo[w][lane]);
+            const float4 y = warp_mlp(S, S.x[w], S.y[w], f, lane);
+            start_output(ok, y, k, count, C, &S.geo[w][lane], n0);
+        }
     }
 }
 
@@ -740,17 +747,19 @@ int launch_mlp_start_t(lub_ctx *ctx, const PView &P, const DView &D, const Ens &
         return lub_check_cuda(ctx, cudaGetLastError(), "k_mlp_start_tc launch");
     }
     const size_t smem = mlp_start_smem();
-    if (!(ctx->mlp_smem_set & (1 << ENS))) {
+    const auto kernel = pq ? k_mlp_start<ENS, true> : k_mlp_start<ENS, false>;
+    const int bit = (pq ? 16 : 1) << ENS;
+    if (!(ctx->mlp_smem_set & bit)) {
         int rc = lub_check_cuda(
-            ctx, cudaFuncSetAttribute(k_mlp_start<ENS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+            ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
             "shared memory attribute");
         if (rc) return rc;
-        ctx->mlp_smem_set |= 1 << ENS;
+        ctx->mlp_smem_set |= bit;
     }
     const int64_t tiles = ((int64_t)cap + 32 * INF_WARPS - 1) / (32 * INF_WARPS);
     const int grid = (int)(tiles < 2 * ctx->num_sms ? tiles : 2 * ctx->num_sms);
     return lub_check_cuda(ctx,
-                          launch_pdl(k_mlp_start<ENS>, grid, 32 * INF_WARPS, smem, st, P, D, E, pi, pj, d_count, cap,
+                          launch_pdl(kernel, grid, 32 * INF_WARPS, smem, st, P, D, E, pi, pj, d_count, cap,
                                      *(const MlpDevice *)ctx->mlp, n0, pq),
                           "k_mlp_start launch");
 }

@@ -146,6 +146,7 @@ struct InfSmem {
     float mean[NI], istd[NI];
     __nv_bfloat16 x[INF_WARPS][32 * XS];
     float4 y[INF_WARPS][32];
+    float geo[INF_WARPS][13 * 32];  // the start kernel's geometry while the network runs
 };
 
 // the 4 network outputs of the calling lane's pair (features f, standardised,
@@ -347,6 +348,131 @@ __device__ __forceinline__ void pair_outputs(const PView &P, const PairIn &in, c
         n0[C + k] = widen_bits(s0.y);
         n0[2 * C + k] = widen_bits(s0.z);
     }
+}
+
+// ---------------------------------------------------------------------------
+// the start normals alone (k_mlp_start without pq)
+// ---------------------------------------------------------------------------
+// The same features and the same normals at the predicted points, written
+// with the symmetry axes alone: the body frame turned about i's axis until d
+// lies in its x-z half-plane has the axes e1 (d's part normal to o_i), o_i x e1
+// and o_i, and a surface point's azimuth is measured from the support point's,
+// so no rotation matrix is formed and no azimuth; reciprocals, roots and
+// logarithms by the hardware's approximations (a few ulp, against the BF16
+// the features are rounded to).  1M pairs from this start in mixed precision
+// 307 -> 262 us (lub_mlp_features and lub_mlp_predict keep the exact forms: their
+// values are results).  The pair's geometry waits in shared memory while the
+// network runs.
+constexpr int GEO = 13;  // per lane: d / |d|, o_i, o_j, R_par,i, R_perp,i, R_par,j, R_perp,j
+
+__device__ __forceinline__ float log_approx(float x)
+{
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return 0.693147180559945309417f * r;
+}
+
+template <bool ENS>
+__device__ __forceinline__ bool start_inputs(const PView &P, const DView &D0, const Ens &E,
+                                             const int32_t *__restrict__ pi, const int32_t *__restrict__ pj, int k,
+                                             int count, const float *mean, const float *istd, float f[NI], float *geo)
+{
+    bool ok = false;
+    if (k < count) {
+        const int i = pi[k], j = pj[k];
+        bool alien;
+        const DView &D = pair_domain<ENS>(D0, E, i, j, &alien);
+        ok = !alien && i >= 0 && i < P.n && j >= 0 && j < P.n && i != j;
+        if (ok) {
+            const float rpi = __ldg(P.rpar + i), rqi = __ldg(P.rperp + i), rpj = __ldg(P.rpar + j),
+                        rqj = __ldg(P.rperp + j);
+            ok = shape_ok(rpi, rqi) && shape_ok(rpj, rqj);
+            const V3<float> d = separation_f(P, D, i, j);
+            const V3<float> oi = quat_axis<float>(__ldg(P.qw + i), __ldg(P.qx + i), __ldg(P.qy + i), __ldg(P.qz + i)),
+                            oj = quat_axis<float>(__ldg(P.qw + j), __ldg(P.qx + j), __ldg(P.qy + j), __ldg(P.qz + j));
+            const float dd = dot(d, d), idl = rsqrtf(dd), dl = dd * idl;
+            const V3<float> e = scl(idl, d);
+            const float ci = dot(oi, e), cj = dot(oj, e);
+            const V3<float> q = axpy(-ci, oi, e);
+            const float s2 = dot(q, q);
+            const bool off = s2 > 1e-14f;  // off i's axis (on it any direction normal to it serves)
+            const float is = off ? rsqrtf(s2) : 0.f, sn = s2 * is;
+            const V3<float> e1 = off ? scl(is, q)
+                                     : (fabsf(oi.x) < 0.6f ? normalized(axpy(-oi.x, oi, mk<float>(1.f, 0.f, 0.f)))
+                                                           : normalized(axpy(-oi.y, oi, mk<float>(0.f, 1.f, 0.f))));
+            const V3<float> e2 = cross(oi, e1);
+            const float iri = rcp_fast(rqi), irj = rcp_fast(rqj);
+            const float a2i = rqi * rqi, a2j = rqj * rqj;
+            const float wi = sqrt_fast(a2i + (rpi * rpi - a2i) * ci * ci), wj = sqrt_fast(a2j + (rpj * rpj - a2j) * cj * cj);
+            f[0] = dl * sn * iri;
+            f[1] = dl * ci * iri;
+            f[2] = dot(oj, e1);
+            f[3] = dot(oj, e2);
+            f[4] = dot(oj, oi);
+            f[5] = log_approx(rpi);
+            f[6] = log_approx(rqi);
+            f[7] = log_approx(rpj);
+            f[8] = log_approx(rqj);
+            const float g = (dl - wi - wj) * rcp_fast(fminf(fminf(rpi, rqi), fminf(rpj, rqj)));
+            f[9] = copysignf(log_approx(fabsf(g) + sqrt_fast(fmaf(g, g, 1.f))), g);
+            f[10] = log_approx(wi * iri);
+            f[11] = log_approx(wj * irj);
+            float sum = 0.f;
+#pragma unroll
+            for (int a = 0; a < NI; ++a) {
+                f[a] = (f[a] - mean[a]) * istd[a];
+                sum += f[a];
+            }
+            if (!isfinite(sum)) ok = false;
+            const float v[GEO] = {e.x, e.y, e.z, oi.x, oi.y, oi.z, oj.x, oj.y, oj.z, rpi, rqi, rpj, rqj};
+#pragma unroll
+            for (int a = 0; a < GEO; ++a) geo[a * 32] = v[a];
+        }
+    }
+    if (!ok)
+#pragma unroll
+        for (int a = 0; a < NI; ++a) f[a] = 0.f;
+    return ok;
+}
+
+// the unit outward normal at the point whose parameters are those of the
+// support point along the unit e, shifted by (dp, dq): see shifted_normal
+__device__ __forceinline__ V3<float> shifted_normal_axis(const V3<float> &o, float rpar, float rperp,
+                                                         const V3<float> &e, float dp, float dq)
+{
+    const float c = dot(o, e);
+    const V3<float> q = axpy(-c, o, e);
+    const float s2 = dot(q, q);
+    const bool off = s2 > 1e-14f;
+    const float is = off ? rsqrtf(s2) : 0.f, sn = s2 * is;
+    const V3<float> u = off ? scl(is, q) : mk<float>(0.f, 0.f, 0.f), w = cross(o, u);
+    const float cp0u = rperp * sn, sp0u = rpar * c, ih = rsqrtf(cp0u * cp0u + sp0u * sp0u);
+    const float cp0 = cp0u * ih, sp0 = sp0u * ih;
+    float sdp, cdp, sdq, cdq;
+    __sincosf(dp, &sdp, &cdp);
+    __sincosf(dq, &sdq, &cdq);
+    const float cp = cp0 * cdp - sp0 * sdp, sp = sp0 * cdp + cp0 * sdp;
+    return normalized(axpy(rpar * cp, axpy(cdq, u, scl(sdq, w)), scl(rperp * sp, o)));
+}
+
+// Newton's start normal of pair k from the network's outputs y
+__device__ __forceinline__ void start_output(bool ok, const float4 y, int k, int count, size_t C, const float *geo,
+                                             double *__restrict__ n0)
+{
+    if (k >= count) return;
+    V3<float> s0 = mk<float>(0.f, 0.f, 0.f);
+    if (ok) {
+        const V3<float> e = mk<float>(geo[0], geo[32], geo[64]), oi = mk<float>(geo[96], geo[128], geo[160]),
+                        oj = mk<float>(geo[192], geo[224], geo[256]);
+        const V3<float> ni = shifted_normal_axis(oi, geo[288], geo[320], e, y.x, y.y);
+        const V3<float> nj = shifted_normal_axis(oj, geo[352], geo[384], scl(-1.0f, e), y.z, y.w);
+        const V3<float> s = sub(ni, nj);
+        const float l2 = dot(s, s);
+        if (l2 > 1e-12f && isfinite(l2)) s0 = scl(rsqrtf(l2), s);
+    }
+    n0[k] = widen_bits(s0.x);
+    n0[C + k] = widen_bits(s0.y);
+    n0[2 * C + k] = widen_bits(s0.z);
 }
 
 // the weights, biases and feature scaling of the installed network into a
