@@ -180,10 +180,14 @@ def _ptr(t):
     """Device (or host) pointer of a tensor / numpy array / int / None."""
     if t is None:
         return None
+    # tensors first and without a look-up beforehand: a step of a small
+    # suspension converts some twenty of them, as long as its kernels run
+    try:
+        return t.data_ptr()
+    except AttributeError:
+        pass
     if isinstance(t, int):
         return t
-    if hasattr(t, "data_ptr"):
-        return t.data_ptr()
     if isinstance(t, np.ndarray):
         return t.ctypes.data
     raise TypeError(type(t))
@@ -195,16 +199,16 @@ def _dom(domain):
 
 
 def _stream(stream):
+    if isinstance(stream, int):
+        return stream
     if stream is None:
         import torch
         return torch.cuda.current_stream().cuda_stream
-    if isinstance(stream, int):
-        return stream
     return stream.cuda_stream
 
 
 def _check(ctx, rc):
-    if rc != LUB_OK:
+    if rc:  # not LUB_OK
         msg = load_library().lub_last_error(ctx).decode()
         raise LubError(rc, msg)
     return rc
@@ -237,10 +241,11 @@ def lub_last_error(ctx):
 
 def lub_pairs_build(ctx, particles, domain, params, pair_i, pair_j, capacity, d_count, h_count=None,
                     stream=None, check=True):
-    hc = ctypes.c_int32(0)
+    hc = ctypes.c_int32(0) if h_count else None
     rc = load_library().lub_pairs_build(ctx, ctypes.byref(particles), _dom(domain), ctypes.byref(params),
                                         _ptr(pair_i), _ptr(pair_j), int(capacity), _ptr(d_count),
-                                        ctypes.byref(hc) if h_count else None, _stream(stream))
+                                        ctypes.byref(hc) if h_count else None,
+                                        _stream(stream))
     if check and rc not in (LUB_OK, LUB_ERR_CAPACITY):
         _check(ctx, rc)
     return rc, (hc.value if h_count else None)
@@ -655,11 +660,10 @@ class Pipeline:
         per_pair=False skips the per-pair outputs other than the normals,
         pair_forces=False only the per-pair forces and lever arms (FT,
         lever): the per-particle sums are the step's result either way."""
-        o = (lambda t: t) if per_pair else (lambda t: None)
-        f = (lambda t: t) if (per_pair and pair_forces) else (lambda t: None)
+        gap, status, iters = (self.gap, self.status, self.iters) if per_pair else (None, None, None)
+        FT, lever = (self.FT, self.lever) if per_pair and pair_forces else (None, None)
         lub_correct(self.ctx.h, self.P.c, self.D, self.prm, self.pair_i, self.pair_j, self.d_count, self.cap, self.nrm,
-                    o(self.gap), o(self.status), o(self.iters), f(self.FT), f(self.lever), self.force, self.torque, 0,
-                    stream)
+                    gap, status, iters, FT, lever, self.force, self.torque, 0, stream)
 
     def resistance_apply(self, per_pair=True, stream=None):
         """Resistance and the atomic scatter in one pass (lub_resistance_apply)."""
@@ -684,6 +688,8 @@ class Pipeline:
         if deterministic:
             form = "calls"
         temporal = self.prm.warm_start == LUB_WARM_PREVIOUS
+        if not temporal:  # (keep_previous takes the stream itself)
+            stream = _stream(stream)  # once for the step's calls
         if build:
             self.build_pairs(sync_count=sync_count, grow=sync_count, stream=stream)
         if temporal and getattr(self, "prev_cap", None) == self.cap:
