@@ -178,14 +178,21 @@ constexpr int kNoEntry = 0x7fffffff;
 // Largest capacity of a pair list that lub_correct takes in one pass
 // (k_fused_mixed) in mixed precision.  One pass saves two launches, the
 // records' second read and the normals' and gaps' way through memory, some
-// 15 us in all; two kernels of 64 and 72 registers keep more warps in flight
-// than one of 96, which is worth 13 us per million pairs.  Measured: 60.4 ->
-// 55.8 us (step, 65k pairs), 238 -> 231 us (0.6M pairs, ensemble), 828 -> 893
-// us (4.4M pairs): level near 1.2 million pairs, and capacities are usually a
+// 15 us in all; but its 64 registers spill where those of the two kernels (64
+// and 72) do not, which costs some 12 us per million pairs.  Measured: 60.4 ->
+// 55.8 us (step, 65k pairs), 238 -> 231 us (0.6M pairs, ensemble), 820 -> 864
+// us (4.4M pairs): level near 1.3 million pairs, and capacities are usually a
 // third above the count.
 constexpr int kFusedMax = 1600000;
-// blocks of 128 threads per SM that the one-pass kernel's registers allow for
-constexpr int kFusedBlocks = 5;
+// The one-pass kernel's blocks of 128 threads per SM: with few pairs (capacity
+// up to kFusedFew) 4, its registers unlimited, since the list then fills the
+// GPU about once and each warp's own chain is what counts; otherwise 8 (64
+// registers, some spilled), for the warps in flight.  Measured at 4, 5, 6, 7,
+// 8: step at 32,768 particles (65k pairs) 49.4, 51.3, 51.3, 51.5, - us; at
+// 131,072 (0.56M pairs, temporal start) 170, 167, 164, 162, 162; ensemble of
+// 262,144 particles 223, 216, 213, 211, 208.
+constexpr int kFusedFew = 160000;
+constexpr int kFusedBlocks = 8;
 
 // The FP32 stage's finish for a particle pair, in float-float on the FP32
 // pipe (GB300 runs FP64 at 1/74 of the FP32 rate): the gap at the FP32 Newton
@@ -1032,8 +1039,10 @@ __device__ __forceinline__ void force_and_scatter(const PView &P, const RParams 
     scatter_warp<T>(ok ? i : -1, ok ? j : -1, (size_t)P.n, ci, cj, force, torque);
 }
 
+// (128 registers: 16 warps per SM keep the FP64 pipe busier than 12 with 160,
+// 294 -> 257 us a step of 20,011 spheroids; 20 warps spill, 271)
 template <bool ENS>
-__global__ void __launch_bounds__(128) k_fused_fp64(PView P, const __grid_constant__ DView D0, Ens E, RParams R,
+__global__ void __launch_bounds__(128, 4) k_fused_fp64(PView P, const __grid_constant__ DView D0, Ens E, RParams R,
                                                     const int32_t *__restrict__ pi, const int32_t *__restrict__ pj,
                                                     const int32_t *__restrict__ d_count, int32_t cap,
                                                     double *__restrict__ nout, double *__restrict__ gap,
@@ -1066,8 +1075,8 @@ __global__ void __launch_bounds__(128) k_fused_fp64(PView P, const __grid_consta
 // whose FP32 Newton did not converge are gathered in shared memory and solved
 // in FP64 by its first lanes before the block goes on, so that a few such
 // pairs cost one FP64 solve per block and not one per warp.
-template <bool ENS>
-__global__ void __launch_bounds__(128, kFusedBlocks) k_fused_mixed(
+template <bool ENS, int BLOCKS>
+__global__ void __launch_bounds__(128, BLOCKS) k_fused_mixed(
     PView P, const __grid_constant__ DView D0, Ens E, const __grid_constant__ RParams R,
     const int32_t *__restrict__ pi, const int32_t *__restrict__ pj, const int32_t *__restrict__ d_count, int32_t cap,
     double *__restrict__ nout, double *__restrict__ gap, uint8_t *__restrict__ status, uint8_t *__restrict__ iters,
@@ -1302,7 +1311,8 @@ int launch_correct_t(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E,
             const RParams R = make_rparams(prm);
             const Shape2 sh = tuned_shape(ctx, LUB_TUNE_CLOSEST_MIXED, cap);
             lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
-            (void)launch_pdl(k_fused_mixed<ENS>, sh.grid, sh.block, 0, st, P, D, E, R, pi, pj, d_count, cap, n, gap,
+            (void)launch_pdl(cap <= kFusedFew ? k_fused_mixed<ENS, 4> : k_fused_mixed<ENS, kFusedBlocks>, sh.grid,
+                             sh.block, 0, st, P, D, E, R, pi, pj, d_count, cap, n, gap,
                              status, iters, (float *)FT, (float *)lever, prm.max_newton, (float)prm.newton_tol,
                              warm, (float *)force, (float *)torque, (const float2 *)pff);
             lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);

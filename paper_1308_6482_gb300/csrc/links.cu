@@ -296,7 +296,7 @@ __device__ __noinline__ int measure_links(LinkWarp &W, int queued, double pre)
 }
 
 template <bool ENS>
-__global__ void __launch_bounds__(128, 4) k_links(PView P, const __grid_constant__ DView D0, Ens E,
+__global__ void __launch_bounds__(128, 5) k_links(PView P, const __grid_constant__ DView D0, Ens E,
                                                const int32_t *__restrict__ pi, const int32_t *__restrict__ pj,
                                                const int32_t *__restrict__ d_count, int32_t cap, double mu,
                                                double qbar, double *__restrict__ force, double *__restrict__ torque,
