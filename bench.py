@@ -314,19 +314,19 @@ def run_multi(lub, torch, np, pl, P, stream, G, replays, step0):
 
 def kernels_in_step(form=None, precision="mixed"):
     # lub_pairs_build: zeroing of its counters, cells count, scan, cells fill,
-    # sweep, FP64 test of the candidates within the sweep's margin, scan,
-    # compaction = 8.  lub_correct (the fused form), mixed:
-    # particle table (which also clears the sums and the work list), FP32
-    # stage, work-list FP64 solves, resistance with scatter = 4; FP64: zeroing
-    # and the one pass = 2.  The merged form (lub_closest_points, then
+    # sweep, test of the margin candidates it leaves over, list = 7 (more than
+    # 1,536 particles).  lub_correct (the fused form), mixed, long lists or the
+    # gated learned start: particle table (which also clears the sums and the
+    # work list), FP32 stage, work-list FP64 solves, resistance with scatter =
+    # 4; FP64: zeroing and the one pass = 2.  The merged form (lub_closest_points, then
     # lub_resistance_apply), mixed: 3 + 3 (zeroing and a second particle
     # table); FP64: 1 + 2.
     form = form or STEP_FORM
     if form == "fused":
-        return 8 + (4 if precision == "mixed" else 2)
+        return 7 + (4 if precision == "mixed" else 2)
     if precision == "mixed":
-        return 8 + 3 + 3
-    return 8 + 1 + 2
+        return 7 + 3 + 3
+    return 7 + 1 + 2
 
 
 def rooflines(kernel_ms, call_ms, npairs, n, mean_it, pk, traffic):
@@ -336,7 +336,7 @@ def rooflines(kernel_ms, call_ms, npairs, n, mean_it, pk, traffic):
     b = n * PAIRS_BYTES_PER_PARTICLE + npairs * PAIRS_BYTES_PER_PAIR
     ach = b / (call_ms["pairs_build"] * 1e-3) / 1e9
     out["pairs_build"] = {
-        "kernel": "lub_pairs_build (8 kernels; k_pairs_sweep %.0f%% of the call)"
+        "kernel": "lub_pairs_build (7 kernels; k_pairs_sweep %.0f%% of the call)"
                   % (100 * kernel_ms["sweep"] / call_ms["pairs_build"]),
         "bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": ach / pk["hbm_gbs"],
         "traffic": traffic.get("pairs_build"), "algorithmic_bytes": b, "ms": call_ms["pairs_build"],
@@ -713,7 +713,7 @@ def suspension_32k(args, lub, torch, np, dev, stream, flush, ws, rank, pk):
             "comparison_link_model": {"ms_per_call": link_ms, "pairs_per_s": npairs / (link_ms * 1e-3),
                                       "links_per_pair": float(nl_host.mean()),
                                       "note": "Eq. methods:dlub on a unit lattice, D3Q19 links, q_bar = 0.6, FP64 "
-                                              "per link, the step's pair list, one warp per pair"},
+                                              "per link, the step's pair list, eight pairs per warp"},
             "substepping": {"ms_per_lb_step": lb_ms, "substeps": 10, "pairs": pairs_s,
                             "pair_corrections_per_s": 10 * pairs_s / (lb_ms * 1e-3),
                             "note": "h_c=0.01, eps_c=100, dt=0.1, density 1, external force N(0,0.01^2)"},

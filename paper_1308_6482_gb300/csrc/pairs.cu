@@ -17,9 +17,10 @@
 //      two indices in one of that particle's KSLOT slots (atomic slot index); the
 //      rare pairs beyond KSLOT go to an overflow list kept at the tail of the
 //      caller's pair arrays; each thread also tests its particle's plane walls;
-//   3. the test of the candidates the sweep's FP32 tests left inside their
-//      margin, in float-float, then in FP64 inside the float-float margin
-//      (k_pairs_undecided), stored as the sweep stores pairs;
+//   3. the candidates the sweep's FP32 tests left inside their margin, tested
+//      in float-float, then in FP64 inside the float-float margin, and stored
+//      as the sweep stores pairs: by their own warp at the end of its sweep,
+//      or, beyond the kWarpUnd a warp keeps, by k_pairs_undecided;
 //   4. the list: the offsets by a scan over the particles' pair and wall
 //      counts inside the same kernel (single pass, decoupled look-back; wall
 //      pairs land after all particle pairs, whose total the sweep has counted),
@@ -27,6 +28,8 @@
 //      them, and its wall pairs, at its offsets.
 // The pair arrays must hold the pairs plus the overflow entries; the count
 // reports their sum when it does not fit (a capacity error, as for the pairs).
+// Up to kSmallMax particles all pairs are tested instead (k_small_tests,
+// k_small_list).
 // The tests run in FP32 on cell-relative coordinates with a safety margin; a
 // test inside the margin is decided again in FP64 from the original double
 // positions, so every decision is the double-precision one.
@@ -502,7 +505,7 @@ static_assert(sizeof(SweepWarp) % 16 == 0, "warp blocks stay 16-byte aligned");
 // One thread per slot s (cell order); the thread also tests its particle's
 // walls.  cnt: pair counts per particle (of the smaller index of each
 // pair); totals[4], [5]: all pairs and wall pairs; slots [KSLOT][N] (slot-major, so that the
-// compaction's reads of the first few slots of consecutive particles are
+// list kernel's reads of the first few slots of consecutive particles are
 // coalesced and touch only the slots in use); wall bits per particle;
 // overflow entry o at pair_i/pair_j[cap - 1 - o].
 //
@@ -862,9 +865,9 @@ __global__ void __launch_bounds__(256, 4) k_pairs_sweep(const __grid_constant__ 
 // in und, then the tagged entries of the pair arrays' tail (entries untagged
 // there are pairs beyond their particle's slots).  An accepted candidate
 // takes the next slot of its smaller index as the sweep's pairs do; beyond
-// the slots it stays where it is, as a pair the compaction collects (an und
+// the slots it stays where it is, as a pair the list kernel collects (an und
 // entry, or the tail entry untagged).  Every other entry becomes -1, which
-// the compaction never matches.  Nothing is appended here, so the tail's
+// the list kernel never matches.  Nothing is appended here, so the tail's
 // length stays as the sweep left it.
 template <bool ENS>
 __global__ void __launch_bounds__(256) k_pairs_undecided(const __grid_constant__ BuildView V)

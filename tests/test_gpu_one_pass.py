@@ -58,3 +58,28 @@ def test_walls_and_invalid_pairs():
     assert np.abs(one["h"] - sep["h"]).max() <= 1e-9
     scale = np.abs(sep["force"]).max()
     assert np.abs(one["force"] - sep["force"]).max() <= 1e-4 * scale
+
+
+@pytest.mark.parametrize("tol", [1e-4, 1e-12])
+@pytest.mark.parametrize("capacity", [160000, 160001, 1600000, 1600001])
+def test_forms_at_their_capacities(capacity, tol):
+    """The one-pass kernel's two register budgets and the separate kernels for
+    long lists are chosen by the pair arrays' capacity: the same list through
+    each, next to the smallest capacity's results."""
+    import torch
+
+    import paper_1308_6482_gb300 as lub
+    parts, dom, pi, pj = gen.pair_stream(1000, seed=77, kind="aspect", gap_range=(1e-4, 1.0))
+    res = []
+    for cap in (1000, capacity):
+        pl = lub.Pipeline(parts, dom, lub.default_params(newton_tol=tol), capacity=cap)
+        pl.set_pairs(pi, pj)
+        pl.correct()
+        torch.cuda.synchronize()
+        res.append(pl.results())
+    a, b = res
+    compare(parts, dom, b, oracle_ref(parts, dom, pi, pj), "mixed", pi, pj)
+    np.testing.assert_array_equal(a["status"], b["status"])
+    np.testing.assert_array_equal(a["iters"], b["iters"])
+    assert np.abs(a["h"] - b["h"]).max() <= 1e-11 * 30.0
+    assert np.abs(a["n"] - b["n"]).max() <= 1e-11
