@@ -36,8 +36,9 @@
 // Measuring across pairs fills the lanes (a pair has some 35 links, so one
 // batch of 32 per pair would be followed by a nearly empty one), and the
 // set-up of one body per lane replaces one by all lanes for every pair.
-// Measured: 65k pairs of a mixed suspension 1.35 ms, against 4.03 ms for one
-// pair per warp with the set-up by all lanes and a measure per pair.
+// Measured: 65k pairs of a mixed suspension 1.175 ms (FP64 pipe 81 % busy),
+// against 4.03 ms for one pair per warp with the set-up by all lanes and a
+// measure per pair, and 1.335 with the measure on the box's own axes.
 #include "lub_internal.cuh"
 
 namespace {
@@ -173,30 +174,51 @@ __device__ __forceinline__ double small_int(int m)
     return abs(m) < (1 << 24) ? widen_bits((float)m) : (double)m;
 }
 
-// c x for c = -1, 0 or 1 on the integer pipe
-__device__ __forceinline__ double times_sign(int c, double x)
+// c x for c = -1 or 1, and for c = -1, 0 or 1, on the integer pipe
+__device__ __forceinline__ double with_sign(int c, double x)
 {
-    const int hi = __double2hiint(x) ^ (c & 0x80000000), lo = __double2loint(x);
-    return c ? __hiloint2double(hi, lo) : 0.0;
+    return __hiloint2double(__double2hiint(x) ^ (c & 0x80000000), __double2loint(x));
+}
+__device__ __forceinline__ double times_sign(int c, double x) { return c ? with_sign(c, x) : 0.0; }
+
+// The measure works on axes turned cyclically, (p, q, k), so that the lattice
+// vector is (cp, cq, 0) with cp = -1 or 1: its products with vectors are then
+// one addition each instead of two, and its cross products one instead of
+// three.  The bodies' components come from shared memory at the turned
+// indices, so the turn costs address arithmetic only.
+struct LinkAxes {
+    int p, q, k, cp, cq;
+};
+__device__ __forceinline__ LinkAxes link_axes(int r)
+{
+    LinkAxes x;
+    x.p = r < 6 ? r >> 1 : r < 10 ? 0 : r < 14 ? 2 : 1;
+    x.q = x.p == 2 ? 0 : x.p + 1;
+    x.k = x.p == 0 ? 2 : x.p - 1;
+    x.cp = d3q19(r, x.p);
+    x.cq = d3q19(r, x.q);
+    return x;
 }
 
-// The line x0 + t c (c: a lattice vector, |c|^2 = cc) and body b: t of the
+// The line x0 + t c (c: a lattice vector in turned axes) and body b: t of the
 // smaller or larger crossing of its surface, from x0 - r = u; false where it
-// misses.  uxc: u x c.  H: twice the mean curvature at the crossing (radii of
+// misses.  uxc: the third component of u x c (the others are -cq u_k and
+// cp u_k).  H: twice the mean curvature at the crossing (radii of
 // curvature of Eq. lub:curvature-radii): with z the crossing's height along
 // the axis and sin^2 p = z^2 / R_par^2, cos^2 p = 1 - sin^2 p on the surface,
 // s1^2 = R_perp^2 sin^2 p + R_par^2 cos^2 p, 1/S1 = R_par R_perp / s1^3 and
-// 1/S2 = R_par / (R_perp s1).
+// 1/S2 = R_par / (R_perp s1).  (Signs and zeros are tested on the integer
+// pipe: a comparison costs as much as a multiply-add.)
 template <bool LARGER>
-__device__ __forceinline__ bool cross_surface(const Body &b, const double u[3], const int c[3], double &t, double &H,
-                                              double uxc[3])
+__device__ __forceinline__ bool cross_surface(const Body &b, const double u[3], const LinkAxes &c, double &t, double &H,
+                                              double &uxc)
 {
-    const double o0 = b.o[0], o1 = b.o[1], o2 = b.o[2];
-    const double ou = o0 * u[0] + o1 * u[1] + o2 * u[2];
+    const double op = b.o[c.p], oq = b.o[c.q], ok = b.o[c.k];
+    const double ou = op * u[0] + oq * u[1] + ok * u[2];
     const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const double oc = times_sign(c[0], o0) + times_sign(c[1], o1) + times_sign(c[2], o2);
-    const double uc = times_sign(c[0], u[0]) + times_sign(c[1], u[1]) + times_sign(c[2], u[2]);
-    const int diag = (c[0] != 0) + (c[1] != 0) + (c[2] != 0) == 2;
+    const double oc = with_sign(c.cp, op) + times_sign(c.cq, oq);
+    const double uc = with_sign(c.cp, u[0]) + times_sign(c.cq, u[1]);
+    const int diag = c.cq != 0;
     const double ia2 = b.ia2, dc = b.dc;
     // |c|^2 / R_perp^2 by the exponent
     const double ccia2 = __hiloint2double(__double2hiint(ia2) + (diag << 20), __double2loint(ia2));
@@ -205,15 +227,13 @@ __device__ __forceinline__ bool cross_surface(const Body &b, const double u[3], 
     const double B = fma(dou, oc, uc * ia2);  // half the linear coefficient
     const double C = fma(dou, ou, fma(uu, ia2, -1.0));
     const double disc = fma(B, B, -A * C);
-    if (!(disc >= 0.0)) return false;
-    const double sq = disc > 0.0 ? disc * rsqrt64(disc) : 0.0;
+    if ((unsigned)__double2hiint(disc) >= 0x7ff00000u) return false;  // negative (never -0) or not finite
+    const double sq = __double2hiint(disc) | __double2loint(disc) ? disc * rsqrt64(disc) : 0.0;
     t = ((LARGER ? sq : -sq) - B) * rcp64(A);
     const double z = fma(t, oc, ou);
     const double is1 = rsqrt64(fma(b.kk * z, z, b.c2));
     H = is1 * fma(b.rr * is1, is1, b.rq);
-    uxc[0] = times_sign(c[2], u[1]) - times_sign(c[1], u[2]);
-    uxc[1] = times_sign(c[0], u[2]) - times_sign(c[2], u[0]);
-    uxc[2] = times_sign(c[1], u[0]) - times_sign(c[0], u[1]);
+    uxc = times_sign(c.cq, u[0]) - with_sign(c.cp, u[1]);
     return true;
 }
 
@@ -221,57 +241,67 @@ __device__ __forceinline__ bool cross_surface(const Body &b, const double u[3], 
 // and torques to the pairs' sums and moves the rest of the queue to the front;
 // returns what is left.  Out of line: called from two places, and the scan's
 // loops then stay small (inlined, the warps waited for instructions).
-__device__ __noinline__ int measure_links(LinkWarp &W, int queued, double pre)
+__device__ __noinline__ int measure_links(LinkWarp &W, int queued, double2 pre)
 {
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
     __syncwarp();
     const int n = queued < 32 ? queued : 32;
-    const LinkEntry en = W.queue[lane];
+    // (an entry past the queue's end is read but not used)
+    const int tag = W.queue[lane].tag;
+    const LinkAxes c = link_axes(lane < n ? tag & 255 : 0);
+    const int m[3] = {W.queue[lane].m[c.p], W.queue[lane].m[c.q], W.queue[lane].m[c.k]};
     const LinkEntry nx = W.queue[32 + lane];
     __syncwarp();
     if (lane < queued - 32) W.queue[lane] = nx;
-    double F[3] = {0, 0, 0}, Ti[3] = {0, 0, 0}, Tj[3] = {0, 0, 0};
-    const int pr = lane < n ? en.tag >> 16 : 0;
+    double Fp = 0.0, Fq = 0.0, Ti[3] = {0, 0, 0}, Tj[3] = {0, 0, 0};  // in turned axes (F has no third)
+    const int pr = lane < n ? tag >> 16 : 0;
     if (lane < n) {
         const Body &bi = W.body[2 * pr], &bj = W.body[2 * pr + 1];
-        const int r = en.tag & 255, kind = (en.tag >> 8) & 255;
-        const int c[3] = {d3q19(r, 0), d3q19(r, 1), d3q19(r, 2)};
+        const int r = tag & 255, kind = (tag >> 8) & 255;
+        const int ax[3] = {c.p, c.q, c.k}, cs[3] = {c.cp, c.cq, 0};
         double ui[3], uj[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const double x0 = small_int(bi.nint[a] + en.m[a] - kind * c[a]);
-            ui[a] = x0 - bi.r[a];
-            uj[a] = x0 - bj.r[a];
+            const double x0 = small_int(bi.nint[ax[a]] + m[a] - kind * cs[a]);
+            ui[a] = x0 - bi.r[ax[a]];
+            uj[a] = x0 - bj.r[ax[a]];
         }
-        double ti, tj, Hi, Hj, xi[3], xj[3];
+        double ti, tj, Hi, Hj, xi, xj;
         const bool mi = cross_surface<false>(bi, ui, c, ti, Hi, xi);
         const bool mj = cross_surface<true>(bj, uj, c, tj, Hj, xj);
-        const double tau = ti - tj;  // h* / c_r
-        if (mi && mj && tau > 0.0 && tau < 1.0) {
+        const double tau = ti - tj;  // h* / c_r; 0 < tau < 1:
+        const int th = __double2hiint(tau);
+        if (mi && mj && (unsigned)th < 0x3ff00000u && (th | __double2loint(tau))) {
             // c.(v_i + w_i x a_i - v_j - w_j x a_j), with c.(w x a) = w.(a x c) = w.(u x c)
-            const double cv = times_sign(c[0], bi.v[0] - bj.v[0]) + times_sign(c[1], bi.v[1] - bj.v[1]) +
-                              times_sign(c[2], bi.v[2] - bj.v[2]) + bi.w[0] * xi[0] + bi.w[1] * xi[1] +
-                              bi.w[2] * xi[2] - bj.w[0] * xj[0] - bj.w[1] * xj[1] - bj.w[2] * xj[2];
+            const double cv = with_sign(c.cp, bi.v[c.p] - bj.v[c.p]) + times_sign(c.cq, bi.v[c.q] - bj.v[c.q]) +
+                              ui[2] * (with_sign(c.cp, bi.w[c.q]) - times_sign(c.cq, bi.w[c.p])) + bi.w[c.k] * xi -
+                              uj[2] * (with_sign(c.cp, bj.w[c.q]) - times_sign(c.cq, bj.w[c.p])) - bj.w[c.k] * xj;
             // df = -3 qbar mu / (2 c_r^2 lambda) (c/c_r) (c/c_r . dv) (1/h*^2 - 1/c_r^2),
-            // lambda = (H_i + H_j) / 4, h* = tau c_r
+            // lambda = (H_i + H_j) / 4, h* = tau c_r, c_r^6 = 8 on the diagonals
             const double t2 = tau * tau;
-            double s = 2.0 * pre * cv * (1.0 - t2) * rcp64((Hi + Hj) * t2);
-            if (r >= 6) s *= 0.125;  // c_r^6 = 8
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                F[a] = times_sign(c[a], s);
-                Ti[a] = s * xi[a];
-                Tj[a] = -s * xj[a];
-            }
+            const double s = (r >= 6 ? pre.y : pre.x) * cv * (1.0 - t2) * rcp64((Hi + Hj) * t2);
+            Fp = with_sign(c.cp, s);
+            Fq = times_sign(c.cq, s);
+            const double sui = s * ui[2], suj = s * uj[2];
+            Ti[0] = -times_sign(c.cq, sui);
+            Ti[1] = with_sign(c.cp, sui);
+            Ti[2] = s * xi;
+            Tj[0] = times_sign(c.cq, suj);
+            Tj[1] = -with_sign(c.cp, suj);
+            Tj[2] = -s * xj;
             atomicAdd(&W.nl[pr], 1);
         }
     }
+    {
+        const double F[3] = {Fp, Fq, 0.0};
+        const int ax[3] = {c.p, c.q, c.k};
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        W.res[a][lane] = F[a];
-        W.res[3 + a][lane] = Ti[a];
-        W.res[6 + a][lane] = Tj[a];
+        for (int a = 0; a < 3; ++a) {
+            W.res[ax[a]][lane] = F[a];
+            W.res[3 + ax[a]][lane] = Ti[a];
+            W.res[6 + ax[a]][lane] = Tj[a];
+        }
     }
     __syncwarp();
     const int part = lane / 9, comp = lane - 9 * part;
@@ -311,7 +341,8 @@ __global__ void __launch_bounds__(128, 5) k_links(PView P, const __grid_constant
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu, below = (1u << lane) - 1u;
     const int nwarp = (gridDim.x * blockDim.x) >> 5;
-    const double pre = -3.0 * qbar * mu;
+    // factors of a link along an axis, and of a diagonal (c_r^6 = 8)
+    const double2 pre = make_double2(-6.0 * qbar * mu, -6.0 * qbar * mu * 0.125);
     for (int64_t k0 = (int64_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * LB; k0 < count;
          k0 += (int64_t)nwarp * LB) {
         const int np = (int)(count - k0 < LB ? count - k0 : LB);

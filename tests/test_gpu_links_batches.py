@@ -1,4 +1,4 @@
-"""The link kernel at the edges of its batches (16 pairs per warp) and site
+"""The link kernel at the edges of its batches (8 pairs per warp) and site
 boxes of very different sizes, against the oracle's brute force."""
 import numpy as np
 import pytest
@@ -9,9 +9,9 @@ from test_gpu_links import check, lub, run  # noqa: F401  (lub: the module's fix
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("count", [1, 15, 16, 17, 63, 65])
+@pytest.mark.parametrize("count", [1, 7, 8, 9, 15, 16, 17, 63, 65])
 def test_batches_of_pairs_with_walls_and_invalid_pairs(lub, count):
-    # a warp takes 16 pairs; wall pairs, bad indices and self pairs among them give zeros
+    # a warp takes 8 pairs, a block 32; wall pairs, bad indices and self pairs among them give zeros
     parts, dom, pi, pj = gen.pair_stream(count, seed=90 + count, kind="mixed", gap_range=(0.02, 1.5))
     pi, pj = pi.copy(), pj.copy()
     bad = np.arange(count) % 5 == 3
