@@ -465,9 +465,10 @@ struct TcSmem {
     unsigned long long mbar_w, mbar_mma;
     uint32_t tmem;
     int stop;
-    // padding: above 76 KB a third CTA never fits an SM, so two CTAs x 256
-    // columns never exceed the SM's 512 TMEM columns (allocation never waits)
-    unsigned char pad[4096];
+    // the pairs' geometry while the network runs.  With it the block takes above
+    // 76 KB, so a third CTA never fits an SM and two CTAs x 256 columns never
+    // exceed the SM's 512 TMEM columns (allocation never waits)
+    float geo[TC_ROWS / 32][GEO * 32];
 };
 static_assert(sizeof(TcSmem) > 228 * 1024 / 3, "at most two CTAs per SM");
 
@@ -593,7 +594,7 @@ __global__ void __launch_bounds__(32 * INF_WARPS, 2) k_mlp_start(PView P, const 
     }
 }
 
-template <bool ENS>
+template <bool ENS, bool PQ>
 __global__ void __launch_bounds__(TC_THREADS) k_mlp_start_tc(PView P, const __grid_constant__ DView D0, Ens E,
                                                           const int32_t *__restrict__ pi,
                                                           const int32_t *__restrict__ pj,
@@ -636,6 +637,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_mlp_start_tc(PView P, const __gr
 #else
     constexpr bool skip_mma = false;
 #endif
+    float *const geo = &S.geo[warp & 3][tid & 31];  // (a row's first thread only)
     const uint32_t sX = smem_u32(S.X), sH = smem_u32(S.H);
     const uint32_t sW1 = smem_u32(S.w.W1), sW2 = smem_u32(S.w.W2), sW3 = smem_u32(S.w.W3);
     const int count = pair_count(d_count, cap);
@@ -648,7 +650,10 @@ __global__ void __launch_bounds__(TC_THREADS) k_mlp_start_tc(PView P, const __gr
         float f[NI];
         PairIn in{-1, -1, &D0, false};
         if (half == 0) {
-            in = pair_inputs<ENS>(P, D0, E, pi, pj, k, count, S.w.mean, S.w.istd, f);
+            if (PQ)
+                in = pair_inputs<ENS>(P, D0, E, pi, pj, k, count, S.w.mean, S.w.istd, f);
+            else
+                in.ok = start_inputs<ENS>(P, D0, E, pi, pj, k, count, S.w.mean, S.w.istd, f, geo);
             uint4 lo, hi;
             lo.x = pack_bf16(f[0], f[1]);
             lo.y = pack_bf16(f[2], f[3]);
@@ -710,7 +715,10 @@ __global__ void __launch_bounds__(TC_THREADS) k_mlp_start_tc(PView P, const __gr
         tmem_ld32(trow, v);  // all warps: the load is warp-collective
         if (half == 0) {
             const float4 y = make_float4(v[0] + S.w.b3[0], v[1] + S.w.b3[1], v[2] + S.w.b3[2], v[3] + S.w.b3[3]);
-            pair_outputs(P, in, y, k, count, C, n0, pq);
+            if (PQ)
+                pair_outputs(P, in, y, k, count, C, n0, pq);
+            else
+                start_output(in.ok, y, k, count, C, geo, n0);
         }
         tc_fence_before();
     }
@@ -731,19 +739,20 @@ int launch_mlp_start_t(lub_ctx *ctx, const PView &P, const DView &D, const Ens &
 {
     if (ctx->mlp_engine == LUB_MLP_TCGEN05) {
         const size_t smem = sizeof(TcSmem);
-        if (!(ctx->mlp_smem_set & (4 << ENS))) {
-            int rc = lub_check_cuda(ctx,
-                                    cudaFuncSetAttribute(k_mlp_start_tc<ENS>,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                                    "shared memory attribute");
+        const auto kernel = pq ? k_mlp_start_tc<ENS, true> : k_mlp_start_tc<ENS, false>;
+        const int bit = (pq ? 64 : 4) << ENS;
+        if (!(ctx->mlp_smem_set & bit)) {
+            int rc = lub_check_cuda(
+                ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                "shared memory attribute");
             if (rc) return rc;
-            ctx->mlp_smem_set |= 4 << ENS;
+            ctx->mlp_smem_set |= bit;
         }
         const MlpDevice &M = *(const MlpDevice *)ctx->mlp;
         const int tiles = (cap + TC_ROWS - 1) / TC_ROWS;
         const int grid = tiles < 2 * ctx->num_sms ? (tiles > 0 ? tiles : 1) : 2 * ctx->num_sms;
-        k_mlp_start_tc<ENS><<<grid, TC_THREADS, smem, st>>>(P, D, E, pi, pj, d_count, cap,
-                                                         (const TcImage *)M.tc_image, n0, pq, ctx->d_flags + 1);
+        kernel<<<grid, TC_THREADS, smem, st>>>(P, D, E, pi, pj, d_count, cap, (const TcImage *)M.tc_image, n0, pq,
+                                               ctx->d_flags + 1);
         return lub_check_cuda(ctx, cudaGetLastError(), "k_mlp_start_tc launch");
     }
     const size_t smem = mlp_start_smem();

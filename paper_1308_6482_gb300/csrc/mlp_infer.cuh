@@ -46,7 +46,8 @@ __device__ __forceinline__ V3<float> separation_f(const PView &P, const DView &D
 __device__ __forceinline__ void pair_features(const PView &P, const DView &D, int i, int j, const float *mean,
                                               const float *istd, float f[NI])
 {
-    const V3<float> d = separation_f(P, D, i, j);
+    const V3<double> dd = min_image(D, sub(load_pos(P, j), load_pos(P, i)));
+    const V3<float> d = cvt<float>(dd);
     float qa[4] = {P.qw[i], P.qx[i], P.qy[i], P.qz[i]};
     const float na = rsqrtf(qa[0] * qa[0] + qa[1] * qa[1] + qa[2] * qa[2] + qa[3] * qa[3]);
     for (int a = 0; a < 4; ++a) qa[a] *= na;
@@ -336,7 +337,7 @@ __device__ __forceinline__ void pair_outputs(const PView &P, const PairIn &in, c
         V3<float> s0 = mk<float>(0, 0, 0);
         if (in.ok) {
             // corrections to the parameters of the line-of-centres start
-            const V3<float> d = separation_f(P, *in.D, in.i, in.j);
+            const V3<float> d = cvt<float>(min_image(*in.D, sub(load_pos(P, in.j), load_pos(P, in.i))));
             const V3<float> e = normalized(d);
             const V3<float> ni = shifted_normal(P, in.i, rot_of(P, in.i), e, y.x, y.y);
             const V3<float> nj = shifted_normal(P, in.j, rot_of(P, in.j), scl(-1.0f, e), y.z, y.w);
@@ -351,7 +352,7 @@ __device__ __forceinline__ void pair_outputs(const PView &P, const PairIn &in, c
 }
 
 // ---------------------------------------------------------------------------
-// the start normals alone (k_mlp_start without pq)
+// the start normals alone (k_mlp_start and k_mlp_start_tc without pq)
 // ---------------------------------------------------------------------------
 // The same features and the same normals at the predicted points, written
 // with the symmetry axes alone: the body frame turned about i's axis until d
@@ -360,8 +361,10 @@ __device__ __forceinline__ void pair_outputs(const PView &P, const PairIn &in, c
 // so no rotation matrix is formed and no azimuth; reciprocals, roots and
 // logarithms by the hardware's approximations (a few ulp, against the BF16
 // the features are rounded to).  1M pairs from this start in mixed precision
-// 307 -> 262 us (lub_mlp_features and lub_mlp_predict keep the exact forms: their
-// values are results).  The pair's geometry waits in shared memory while the
+// 307 -> 262 us, on the tcgen05 engine 385 -> 311 (lub_mlp_features and
+// lub_mlp_predict keep the exact forms: their values are results, and their
+// FP64 separations, which run beside the scalar work, are the faster ones
+// there: predict on 1M pairs 193 us with float-float separations, 173 with FP64).  The pair's geometry waits in shared memory while the
 // network runs.
 constexpr int GEO = 13;  // per lane: d / |d|, o_i, o_j, R_par,i, R_perp,i, R_par,j, R_perp,j
 
