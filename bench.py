@@ -63,11 +63,11 @@ PAIRS_BYTES_PER_PAIR = 8.0       # (i, j) written
 # (one ncu capture of dram__bytes_read.sum + dram__bytes_write.sum per kernel
 # over `bench.py --only large --steps 3`, the last of its three steps)
 TRAFFIC = {
-    "large": {"sources": "f33b023ddd56a8f2",
-              "bytes": {"pairs_build": 274182656, "k_closest_mixed": 372022272, "k_resistance_apply": 496749056}},
+    "large": {"sources": "bf020ae8dc23c2d3",
+              "bytes": {"pairs_build": 251237632, "k_closest_mixed": 371877632, "k_resistance_apply": 522065408}},
 }
 TRAFFIC_SOURCES = ("closest.cu", "pair_force.cuh", "resistance.cu", "pairs.cu", "ff.cuh", "lub_internal.cuh",
-                   "mlp_infer.cuh", "scan.cu", "scan_tile.cuh", "apply.cu")
+                   "scan.cu", "scan_tile.cuh", "apply.cu")
 # the form of the timed step: lub_pairs_build, then lub_correct (closest
 # points, resistance and scatter in one call)
 STEP_FORM = "fused"
