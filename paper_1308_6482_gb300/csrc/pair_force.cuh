@@ -98,11 +98,15 @@ __device__ __forceinline__ float log1p_t(float x) { return log1pf(x); }
 // with m in [sqrt(1/2), sqrt(2)), log m = 2 atanh(s), s = (m - 1)/(m + 1)
 // (Abramowitz & Stegun 4.1.27), |s| < 0.1716, as its Taylor series to s^23
 // (the next term is below 2^-60 of the first).  For k = 0 m - 1 is x itself,
-// so the result keeps its relative accuracy as x goes to 0.
+// so the result keeps its relative accuracy as x goes to 0.  x = -1 gives
+// -infinity (a gap below 2^-53 of the cut-off comes to that), below it and
+// NaN give NaN, as log1p does.
 __device__ __forceinline__ double log1p_t(double x)
 {
     const double a = 1.0 + x;
     const int hi = __double2hiint(a);
+    if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u)  // zero, negative, infinite or NaN
+        return (hi | __double2loint(a)) == 0 ? -(double)INFINITY : hi > 0 ? a : (double)NAN;
     // k: the exponent of a / sqrt(1/2) rounded down
     const int k = (hi - 0x3fe6a09e) >> 20;
     const double m = __hiloint2double(hi - (k << 20), __double2loint(a));

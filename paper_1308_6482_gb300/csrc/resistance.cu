@@ -195,3 +195,27 @@ int launch_resistance(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E
     lub_trace_mark(ctx, LUB_TRACE_RESISTANCE, st);
     return lub_check_cuda(ctx, cudaGetLastError(), "k_resistance launch");
 }
+
+#ifdef LUB_TESTING
+// Test build only (no counterpart in the product library): y = the scalar
+// function fn of x, on the device.
+__global__ void k_test_math(int fn, const double *__restrict__ x, double *__restrict__ y, int n)
+{
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const double v = x[k];
+        y[k] = fn == 0   ? log1p_t(v)
+               : fn == 1 ? rcp64(v)
+               : fn == 2 ? rsqrt64(v)
+               : fn == 3 ? widen_bits((float)v)
+               : fn == 4 ? (double)round_bits(v)
+                         : (double)narrow_bits(v);
+    }
+}
+
+extern "C" int lub_test_math(int32_t fn, const double *x, double *y, int32_t n, void *stream)
+{
+    if (fn < 0 || fn > 5 || n < 1 || !x || !y) return LUB_ERR_ARG;
+    k_test_math<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream>>>(fn, x, y, n);
+    return cudaGetLastError() == cudaSuccess ? LUB_OK : LUB_ERR_CUDA;
+}
+#endif
