@@ -224,13 +224,17 @@ __device__ __forceinline__ V3<T> axpy(T s, const V3<T> &a, const V3<T> &b)  // s
 // FP64 warp instruction per 19 clocks and SM, and the conversions use that
 // pipe too (17 clocks), so one costs as much as some seventy integer
 // instructions.
-// The double of a float, exactly (float subnormals give zero).
+// The double of a float, exactly.
 __device__ __forceinline__ double widen_bits(float f)
 {
     const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
     unsigned hi = (m >> 3) + (m < 0x7f800000u ? 0x38000000u : 0x70000000u);
     unsigned lo = b << 29;
-    if (m < 0x00800000u) hi = lo = 0u;
+    if (m < 0x00800000u) {  // zero, or subnormal: as a normal float 2^24 times as large
+        const unsigned g = __float_as_uint(__fmul_rn(__uint_as_float(m), 0x1p24f));
+        hi = g ? (g >> 3) + 0x38000000u - (24u << 20) : 0u;
+        lo = g << 29;
+    }
     return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo);
 }
 
@@ -260,14 +264,15 @@ __device__ __forceinline__ float narrow_bits(double d)
 }
 
 // Double-precision reciprocal and reciprocal square root: an FP32 seed from
-// the argument's mantissa (its exponent handled by integer operations, so the
-// whole double range is covered and nothing is converted) and one third-order
-// step.  With the residual e = 1 - a x (1 - a y^2), of order 2^-22 (the seed
-// and its truncated argument), 1/(1 - e) = 1 + e + e^2 + ... and (1 - e)^(-1/2)
-// = 1 + e/2 + 3 e^2/8 + ... leave an error of order e^3 = 2^-66, below double
-// rounding, in 3 and 5 FP64 operations (two Newton-Raphson steps with
-// converted seeds took 6 and 9).  A zero argument gives infinity or a huge
-// value, a negative square root NaN.
+// the argument's mantissa (its exponent handled by integer operations, so that
+// nothing is converted) and one third-order step, for |a| from 2^-1022 up to
+// 2^1022 (reciprocal) and every positive normal a (root).  With the residual
+// e = 1 - a x (1 - a y^2), of order 2^-22 (the seed and its truncated
+// argument), 1/(1 - e) = 1 + e + e^2 + ... and (1 - e)^(-1/2) = 1 + e/2 +
+// 3 e^2/8 + ... leave an error of order e^3 = 2^-66, below double rounding, in
+// 3 and 5 FP64 operations (two Newton-Raphson steps with converted seeds took
+// 6 and 9).  The reciprocal of zero is infinite, the root's
+// of zero some 1e154; a negative root gives NaN.
 __device__ __forceinline__ double rcp64(double a)
 {
     const int hi = __double2hiint(a), k = (hi >> 20 & 0x7ff) - 1023;
