@@ -90,17 +90,25 @@ __device__ __forceinline__ void body_at(Body &b, const PView &P, int k, const V3
     b.kk = (Rperp * Rperp - Rpar * Rpar) * ic2;
     b.rr = Rpar * Rperp;
     b.rq = Rpar * rcp64(Rperp);
-    const float a2 = rperp * rperp, e = rpar * rpar - a2;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const double fl = floor(rv[a]);
-        const float of = (float)ov[a];
         b.r[a] = rv[a];
         b.o[a] = ov[a];
         b.nint[a] = (int)fl;
         b.f[a] = (float)(rv[a] - fl);
-        b.of[a] = of;
-        b.half[a] = sqrtf(fmaxf(a2 + e * of * of, 0.f));
+        b.of[a] = (float)ov[a];
+    }
+    // the half extent sqrt(R_perp^2 (1 - o_a^2) + R_par^2 o_a^2) as a sum of
+    // positive terms (1 - o_a^2 from the other two components, |o| = 1 to
+    // 2^-23), which is good to some 2^-22 of itself for any shape: as
+    // R_perp^2 + (R_par^2 - R_perp^2) o_a^2 it cancels for a disc whose axis is
+    // close to a, and a site just inside a thin one (R_perp / R_par above some
+    // 200 at R_perp = 100) would be missed; 1e-6 outward for the rounding
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float u = b.of[a], v = b.of[a == 2 ? 0 : a + 1], w = b.of[a == 0 ? 2 : a - 1];
+        b.half[a] = 1.000001f * sqrtf(rperp * rperp * (v * v + w * w) + rpar * rpar * (u * u));
     }
     b.ia2f = (float)ia2;
     b.dcf = (float)(ic2 - ia2);
@@ -373,7 +381,7 @@ __global__ void __launch_bounds__(128, 5) k_links(PView P, const __grid_constant
             if (!((valid >> (2 * q)) & 1u)) continue;
             const Body &bi = W.body[2 * q], &bj = W.body[2 * q + 1];
             // the box of sites as offsets m from i's anchor (the same site is
-            // m + dij from j's); 1e-3 outward for the FP32 half extents
+            // m + dij from j's); 1e-3 outward for the FP32 sums
             int lo[3], nn[3], dij[3];
             int nsites = 1;
 #pragma unroll
