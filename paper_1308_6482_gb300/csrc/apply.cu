@@ -7,12 +7,21 @@
 //                  come sorted by i) are combined first with a segmented
 //                  warp reduction, so i-side atomics drop to one per run.
 //   deterministic  incidence lists (counting sort by particle, entries
-//                  sorted by pair index and side), eight lanes per particle
-//                  summing in that fixed order: bitwise reproducible.
+//                  sorted by pair index and side), eight lanes or one lane
+//                  per particle summing in that fixed order: bitwise
+//                  reproducible.
 #include "pair_force.cuh"
 
 namespace {
 
+// v, or -v where side is 1, off the FP64 pipe
+__device__ __forceinline__ float side_sign(float v, int side) { return side ? -v : v; }
+__device__ __forceinline__ double side_sign(double v, int side)
+{
+    return __hiloint2double(__double2hiint(v) ^ (side << 31), __double2loint(v));
+}
+
+// (six multiply-adds in all: in FP64 mode the FP64 pipe bounds the sums)
 template <typename T>
 __device__ __forceinline__ void pair_contrib(const T *__restrict__ FT, const T *__restrict__ lever, size_t C,
                                              int k, int side, T out[6])
@@ -21,10 +30,12 @@ __device__ __forceinline__ void pair_contrib(const T *__restrict__ FT, const T *
     const V3<T> Tq = mk<T>(FT[3 * C + k], FT[4 * C + k], FT[5 * C + k]);
     const V3<T> l = side ? mk<T>(lever[3 * C + k], lever[4 * C + k], lever[5 * C + k])
                          : mk<T>(lever[k], lever[C + k], lever[2 * C + k]);
-    const V3<T> t = add(Tq, cross(l, F));
-    const T sg = side ? T(-1) : T(1);
-    out[0] = sg * F.x; out[1] = sg * F.y; out[2] = sg * F.z;
-    out[3] = sg * t.x; out[4] = sg * t.y; out[5] = sg * t.z;
+    out[0] = side_sign(F.x, side);
+    out[1] = side_sign(F.y, side);
+    out[2] = side_sign(F.z, side);
+    out[3] = side_sign(fma(l.y, F.z, fma(-l.z, F.y, Tq.x)), side);
+    out[4] = side_sign(fma(l.z, F.x, fma(-l.x, F.z, Tq.y)), side);
+    out[5] = side_sign(fma(l.x, F.y, fma(-l.y, F.x, Tq.z)), side);
 }
 
 template <typename T>
@@ -97,18 +108,86 @@ __global__ void k_inc_fill(const int32_t *__restrict__ pi, const int32_t *__rest
 
 // The sums, eight lanes per particle: the lanes sort the particle's entries
 // (pair index, side) by rank, fetch the contributions of eight entries at a
-// time (twelve scattered loads each, the bound: one lane per particle had
+// time (nine scattered loads each, the bound: one lane per particle had
 // them one entry after the other, 37 us at 100,003 particles and 340k pairs
 // against 13) and six lanes add one component each in the sorted order, as a
 // single lane would.  A particle of more than kRankMax entries is sorted in
 // place by one lane.
 constexpr int kGroup = 8, kRankMax = 32;
 
+// One lane per particle, sorting in place, is the better form where there are
+// enough particles to fill the GPU and too few entries for eight lanes: below
+// 1.5 a particle from kLaneFrom particles on, below 3.5 from kLaneMore on.  The
+// number of entries is known on the device only, so the kernel has both forms.
+// Whole call in mixed precision, eight lanes and one: 200,000 particles with
+// 0.8 entries each 24.5 and 18.8 us, with 2.4 each 30.9 and 33.3; 262,144 with
+// 1.6 each 33.9 and 30.1, with 4.8 each 57.5 and 67.5; 400,000 with 2.2 each
+// 50.9 and 48.4, with 3.2 each 61.7 and 63.7, but 81.6 and 63.4 in arrays of 16
+// pairs a particle (random order, components 26 MB apart).
+constexpr int kLaneFrom = 131072, kLaneMore = 250000;
+__device__ __forceinline__ bool one_lane(int n, int entries)
+{
+    return n >= kLaneFrom && 2 * (int64_t)entries < (n >= kLaneMore ? 7 : 3) * (int64_t)n;
+}
+
+// a particle's entries [b, e), sorted in place by the calling lane
+__device__ __forceinline__ void sort_entries(int32_t *inc, int b, int e)
+{
+    for (int a = b + 1; a < e; ++a) {
+        const int v = inc[a];
+        int c = a - 1;
+        while (c >= b && inc[c] > v) {
+            inc[c + 1] = inc[c];
+            --c;
+        }
+        inc[c + 1] = v;
+    }
+}
+
+// a component of a particle's sum
 template <typename T>
-__global__ void __launch_bounds__(256) k_inc_sum(const int32_t *__restrict__ start, const int32_t *__restrict__ total,
+__device__ __forceinline__ void store_sum(T *force, T *torque, size_t N, int p, int comp, T v, int accumulate)
+{
+    T *const dst = comp < 3 ? force + comp * N + p : torque + (comp - 3) * N + p;
+    *dst = accumulate ? *dst + v : v;
+}
+
+// the sums by one lane per particle
+template <typename T>
+__device__ __forceinline__ void sum_by_lane(const int32_t *__restrict__ start, int entries, int32_t *__restrict__ inc,
+                                            int n, const T *__restrict__ FT, const T *__restrict__ lever, int32_t cap,
+                                            T *__restrict__ force, T *__restrict__ torque, int accumulate,
+                                            int blocks)
+{
+    const size_t C = (size_t)cap, N = (size_t)n;
+    if ((int)blockIdx.x >= blocks) return;
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += blocks * blockDim.x) {
+        const int b = max(0, min(start[p], 2 * cap));
+        const int e = max(b, min((p + 1 < n) ? start[p + 1] : entries, 2 * cap));
+        sort_entries(inc, b, e);
+        T acc[6] = {0, 0, 0, 0, 0, 0};
+        for (int a = b; a < e; ++a) {
+            const int v = inc[a];
+            if (v < 0 || (v >> 1) >= cap) continue;  // never filled (after a timed-out scan)
+            T c6[6];
+            pair_contrib<T>(FT, lever, C, v >> 1, v & 1, c6);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) acc[q] += c6[q];
+        }
+#pragma unroll
+        for (int q = 0; q < 6; ++q) store_sum(force, torque, N, p, q, acc[q], accumulate);
+    }
+}
+
+// resident blocks of 256 threads per SM: the registers' limit
+template <typename T>
+constexpr int sum_blocks() { return sizeof(T) == 4 ? 8 : 5; }
+
+template <typename T>
+__global__ void __launch_bounds__(256, sum_blocks<T>()) k_inc_sum(const int32_t *__restrict__ start, const int32_t *__restrict__ total,
                                                  int32_t *__restrict__ inc, int n, const T *__restrict__ FT,
                                                  const T *__restrict__ lever, int32_t cap, T *__restrict__ force,
-                                                 T *__restrict__ torque, int accumulate)
+                                                 T *__restrict__ torque, int accumulate, int wave)
 {
     pdl_wait();
     pdl_trigger();
@@ -116,6 +195,11 @@ __global__ void __launch_bounds__(256) k_inc_sum(const int32_t *__restrict__ sta
     __shared__ int key_s[NGRP][kRankMax + 1], sorted_s[NGRP][kRankMax + 1];
     __shared__ T c_s[NGRP][kGroup * 6 + 1];
     const size_t C = (size_t)cap, N = (size_t)n;
+    if (one_lane(n, *total)) {  // (the same for every block)
+        sum_by_lane<T>(start, *total, inc, n, FT, lever, cap, force, torque, accumulate,
+                       min((int)gridDim.x, wave));
+        return;
+    }
     const int sub = threadIdx.x % kGroup, g = threadIdx.x / kGroup;
     int *const key = key_s[g], *const sorted = sorted_s[g];
     T *const cs = c_s[g];
@@ -132,16 +216,7 @@ __global__ void __launch_bounds__(256) k_inc_sum(const int32_t *__restrict__ sta
         if (!many)
             for (int q = sub; q < m; q += kGroup) key[q] = inc[b + q];
         else if (sub == 0)
-            // insertion sort of this particle's entries
-            for (int a = b + 1; a < e; ++a) {
-                const int v = inc[a];
-                int c = a - 1;
-                while (c >= b && inc[c] > v) {
-                    inc[c + 1] = inc[c];
-                    --c;
-                }
-                inc[c + 1] = v;
-            }
+            sort_entries(inc, b, e);
         __syncwarp();
         if (!many)
             for (int q = sub; q < m; q += kGroup) {
@@ -168,11 +243,27 @@ __global__ void __launch_bounds__(256) k_inc_sum(const int32_t *__restrict__ sta
                 for (int t = 0; t < kGroup && q0 + t < m; ++t) acc += cs[t * 6 + sub];
             __syncwarp();
         }
-        if (p < n && sub < 6) {
-            T *const dst = sub < 3 ? force + sub * N + p : torque + (sub - 3) * N + p;
-            *dst = accumulate ? *dst + acc : acc;
-        }
+        if (p < n && sub < 6) store_sum(force, torque, N, p, sub, acc, accumulate);
     }
+}
+
+template <typename T>
+void launch_sum(int num_sms, cudaStream_t st, const int32_t *start, const int32_t *total, int32_t *inc, int n,
+                const T *FT, const T *lever, int32_t cap, T *force, T *torque, int accumulate)
+{
+    constexpr int block = 256;
+    const int grid = grid_for((int64_t)n * kGroup, block, num_sms, n >= kLaneFrom ? 16 : 32);
+    const int wave = sum_blocks<T>() * num_sms;
+    // A grid of less than one wave, but more than two blocks an SM, and the form
+    // by one lane take a plain launch: with a programmatic one the blocks fill
+    // those SMs first that the kernel before leaves first, eight to an SM, while
+    // others stay empty (20,000 particles with 8 entries each: 22.4 us for the
+    // call against 17.4, in FP64 27.2 and 21.0)
+    if (n >= kLaneFrom || (grid > 2 * num_sms && grid < wave))
+        k_inc_sum<T><<<grid, block, 0, st>>>(start, total, inc, n, FT, lever, cap, force, torque, accumulate, wave);
+    else
+        (void)launch_pdl(k_inc_sum<T>, grid, block, 0, st, start, total, inc, n, FT, lever, cap, force, torque,
+                         accumulate, wave);
 }
 
 inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -225,13 +316,11 @@ int launch_apply(lub_ctx *ctx, const int32_t *pi, const int32_t *pj, const int32
     if (rc) return rc;
     (void)launch_pdl(k_inc_fill, gp, block, 0, st, pi, pj, d_count, cap, n, (const int32_t *)cnt, (const int2 *)place,
                      inc);
-    const int gn = grid_for((int64_t)n * kGroup, block, ctx->num_sms, 32);
     if (precision == LUB_MIXED)
-        (void)launch_pdl(k_inc_sum<float>, gn, block, 0, st, (const int32_t *)cnt, (const int32_t *)tot, inc, n,
-                         (const float *)FT, (const float *)lever, cap, (float *)force, (float *)torque, accumulate);
+        launch_sum<float>(ctx->num_sms, st, cnt, tot, inc, n, (const float *)FT, (const float *)lever, cap,
+                          (float *)force, (float *)torque, accumulate);
     else
-        (void)launch_pdl(k_inc_sum<double>, gn, block, 0, st, (const int32_t *)cnt, (const int32_t *)tot, inc, n,
-                         (const double *)FT, (const double *)lever, cap, (double *)force, (double *)torque,
-                         accumulate);
+        launch_sum<double>(ctx->num_sms, st, cnt, tot, inc, n, (const double *)FT, (const double *)lever, cap,
+                           (double *)force, (double *)torque, accumulate);
     return lub_check_cuda(ctx, cudaGetLastError(), "deterministic apply launch");
 }
