@@ -14,7 +14,9 @@
 // act at the two intersection points, torques about the centres; walls give
 // nothing.
 //
-// A warp takes 8 pairs at a time.  What bounds the work is the FP64 pipe (two
+// A warp takes up to 8 pairs at a time (as few as give every resident warp some:
+// below some 24,000 pairs the list does not fill the GPU and a warp's own chain
+// is what counts).  What bounds the work is the FP64 pipe (two
 // lanes per clock and SM: one warp instruction costs as much as some 70 on
 // the other pipes), so every FP64 operation runs with all lanes busy, and
 // what need not be FP64 is not:
@@ -38,12 +40,14 @@
 // set-up of one body per lane replaces one by all lanes for every pair.
 // Measured: 65k pairs of a mixed suspension 1.175 ms (FP64 pipe 81 % busy),
 // against 4.03 ms for one pair per warp with the set-up by all lanes and a
-// measure per pair, and 1.335 with the measure on the box's own axes.
+// measure per pair, and 1.335 with the measure on the box's own axes; 103 pairs
+// 49 us (103 and, with batches of 8 whatever the list's length, 201).
 #include "lub_internal.cuh"
 
 namespace {
 
-constexpr int LB = 8;             // pairs per warp and batch (two bodies each: one per lane)
+constexpr int LB = 8;             // most pairs per warp and batch (two bodies each: one per lane)
+constexpr int LBLOCKS = 5;        // resident blocks (of four warps) per SM
 constexpr int LQ = 64;            // queued links and gathered sites per warp: at most 31 waiting plus 32 new
 
 // A particle at its (image) centre r: what the tests and the measure need.
@@ -334,11 +338,11 @@ __device__ __noinline__ int measure_links(LinkWarp &W, int queued, double2 pre)
 }
 
 template <bool ENS>
-__global__ void __launch_bounds__(128, 5) k_links(PView P, const __grid_constant__ DView D0, Ens E,
+__global__ void __launch_bounds__(128, LBLOCKS) k_links(PView P, const __grid_constant__ DView D0, Ens E,
                                                const int32_t *__restrict__ pi, const int32_t *__restrict__ pj,
                                                const int32_t *__restrict__ d_count, int32_t cap, double mu,
                                                double qbar, double *__restrict__ force, double *__restrict__ torque,
-                                               int32_t *__restrict__ nlinks)
+                                               int32_t *__restrict__ nlinks, int resident)
 {
     pdl_wait();
     pdl_trigger();
@@ -349,11 +353,16 @@ __global__ void __launch_bounds__(128, 5) k_links(PView P, const __grid_constant
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu, below = (1u << lane) - 1u;
     const int nwarp = (gridDim.x * blockDim.x) >> 5;
+    // pairs per batch: enough that every resident warp has one.  Measured with
+    // 1, 2, 4 and 8 (us): 100 pairs 57, 75, 108, 195; 2,000 92, 90, 131, 221;
+    // 6,000 161, 156, 181, 255; 20,000 474, 417, 408, 416; 60,000 1321, 1107,
+    // 1003, 1047
+    const int per = min(LB, max(1, (count + resident - 1) / resident));
     // factors of a link along an axis, and of a diagonal (c_r^6 = 8)
     const double2 pre = make_double2(-6.0 * qbar * mu, -6.0 * qbar * mu * 0.125);
-    for (int64_t k0 = (int64_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * LB; k0 < count;
-         k0 += (int64_t)nwarp * LB) {
-        const int np = (int)(count - k0 < LB ? count - k0 : LB);
+    for (int64_t k0 = (int64_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per; k0 < count;
+         k0 += (int64_t)nwarp * per) {
+        const int np = (int)(count - k0 < per ? count - k0 : per);
         // the bodies: lane 2 q takes i of pair q, lane 2 q + 1 takes j
         unsigned valid;
         {
@@ -516,21 +525,29 @@ int launch_links(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E, con
     if (cap == 0) return LUB_OK;
     const int block = 128;
     const size_t smem = (block / 32) * sizeof(LinkWarp);
-    static_assert(4 * sizeof(LinkWarp) <= 113 * 1024, "two blocks fit an SM");
+    static_assert(LBLOCKS * (4 * sizeof(LinkWarp) + 1024) <= 228 * 1024, "the resident blocks fit an SM's shared memory");
     const int warps = block / 32;
+    // a warp per batch of LB pairs, or (short lists, in batches of fewer) one wave of blocks
     int64_t grid = ((int64_t)cap + LB * warps - 1) / (LB * warps);
+    const int64_t wave = (int64_t)LBLOCKS * ctx->num_sms, each = ((int64_t)cap + warps - 1) / warps;
+    if (grid < wave) grid = each < wave ? each : wave;
     if (grid > 64 * (int64_t)ctx->num_sms) grid = 64 * (int64_t)ctx->num_sms;
+    const int resident = (int)wave * warps;
     int rc = lub_check_cuda(ctx,
                             cudaFuncSetAttribute(E.nb ? k_links<true> : k_links<false>,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                             "shared memory attribute");
     if (rc) return rc;
+    const auto kernel = E.nb ? k_links<true> : k_links<false>;
     cudaError_t e;
-    if (E.nb)
-        e = launch_pdl(k_links<true>, (int)grid, block, smem, st, P, D, E, pi, pj, d_count, cap, mu, qbar, force, torque,
-                       nlinks);
-    else
-        e = launch_pdl(k_links<false>, (int)grid, block, smem, st, P, D, E, pi, pj, d_count, cap, mu, qbar, force,
-                       torque, nlinks);
+    if (grid <= wave) {
+        // (a plain launch: its blocks are spread over all SMs, not packed on those
+        // that the kernel before leaves first)
+        kernel<<<(int)grid, block, smem, st>>>(P, D, E, pi, pj, d_count, cap, mu, qbar, force, torque, nlinks, resident);
+        e = cudaGetLastError();
+    } else {
+        e = launch_pdl(kernel, (int)grid, block, smem, st, P, D, E, pi, pj, d_count, cap, mu, qbar, force, torque,
+                       nlinks, resident);
+    }
     return lub_check_cuda(ctx, e, "k_links launch");
 }
