@@ -691,11 +691,11 @@ __device__ __forceinline__ V3<double> min_image_near(const DView &D, V3<double> 
     return min_image(D, d);
 }
 
-// LUB_FP64: the solve and gap of pair k (direct: by the FP64 iteration alone)
+// LUB_FP64: the solve and gap of pair k
 template <bool ENS>
 __device__ __forceinline__ void closest_fp64_one(const PView &P, const DView &D0, const Ens &E, int i, int j, int k,
                                                  const double *__restrict__ nin, size_t C, int warm, int maxit,
-                                                 V3<double> &n64, double &h, int &st, int &nit, bool direct = false)
+                                                 V3<double> &n64, double &h, int &st, int &nit)
 {
     st = 0;
     nit = 0;
@@ -736,7 +736,7 @@ __device__ __forceinline__ void closest_fp64_one(const PView &P, const DView &D0
                 const ff oj[3] = {ff_split_bits(sj.o.x), ff_split_bits(sj.o.y), ff_split_bits(sj.o.z)};
                 const ff n0[3] = {ff_split_bits(nn.x), ff_split_bits(nn.y), ff_split_bits(nn.z)};
                 ff nf[3];
-                bool done = !direct && solve_ff(df, oi, oj, rqi, rpi, rqj, rpj, n0, maxit, nf, nit);
+                bool done = solve_ff(df, oi, oj, rqi, rpi, rqj, rpj, n0, maxit, nf, nit);
                 if (done) done = finish_fp64(d, si, sj, nf, n64, h);
                 if (!done) {
                     const double scale = dl + (double)fmaxf(rpi, rqi) + (double)fmaxf(rpj, rqj);
@@ -927,15 +927,6 @@ __global__ void __launch_bounds__(32) k_closest_refine(PView P, const __grid_con
     }
 }
 
-// Lists of kDirectFrom to kDirectTo pairs from the cold start go to the FP64
-// iteration straight away.  There a warp has the FP64 pipe of its SM quarter to
-// itself, so the list takes as long as its slowest warp, and a warp with a pair
-// that solve_ff leaves (0.1 to 0.5 % of them) runs both solves, one after the
-// other: 50 to 69 us against 40 to 45 for the FP64 iteration alone (and 20 to 27
-// where no pair is left, the usual case of shorter lists); 20,000 pairs 64 to 71
-// and 57, 30,000 pairs 69 to 80 and 74.
-constexpr int kDirectFrom = 512, kDirectTo = 24576;
-
 template <bool ENS>
 __global__ void __launch_bounds__(128) k_closest_fp64(PView P, const __grid_constant__ DView D0, Ens E,
                                                       const int32_t *__restrict__ pi, const int32_t *__restrict__ pj,
@@ -948,13 +939,11 @@ __global__ void __launch_bounds__(128) k_closest_fp64(PView P, const __grid_cons
     pdl_trigger();
     const int count = pair_count(d_count, cap);
     const size_t C = (size_t)cap;
-    const bool direct = !warm && count >= kDirectFrom && count <= kDirectTo;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x) {
         V3<double> n64;
         double h;
         int st, nit;
-        closest_fp64_one<ENS>(P, D0, E, __ldg(pi + k), __ldg(pj + k), k, nout, C, warm, maxit, n64, h, st, nit,
-                              direct);
+        closest_fp64_one<ENS>(P, D0, E, __ldg(pi + k), __ldg(pj + k), k, nout, C, warm, maxit, n64, h, st, nit);
         store_pair(nout, gap, status, iters, C, k, n64, h, st, nit);
     }
 }
