@@ -874,6 +874,13 @@ __global__ void __launch_bounds__(256) k_pairs_undecided(const __grid_constant__
 {
     pdl_wait();
     pdl_trigger();
+    // this build's flags, for the host-count path: all that the kernels before
+    // have found (the list kernel after this one only adds its timed-out waits)
+    if (V.flags_out && blockIdx.x == 0 && threadIdx.x == 0) {
+        const int32_t f = *V.flags;
+        *V.flags_out = f;
+        if (f & 4) atomicOr(V.flags_out + 1, 4);  // a timed-out wait, for lub_sync_status
+    }
     const int N = V.P.n;
     const int nu = min(V.totals[3], V.und_cap);
     const int nt = V.totals[3] > V.und_cap ? min(V.totals[2], V.cap) : 0;
@@ -908,6 +915,11 @@ __global__ void __launch_bounds__(256) k_pairs_undecided(const __grid_constant__
     }
 }
 
+#ifdef LUB_TESTING
+// a test build's hook: the tile of the list kernel that never publishes (-1: none)
+__device__ int g_test_mute_list_tile = -1;
+#endif
+
 // The list's scan state: a ticket, then one word per tile of 256 G particles:
 // flag (bits 62, 63) | walls (31 bits) | pairs (31 bits) of the tile, or of all
 // tiles up to it.
@@ -923,14 +935,21 @@ inline int64_t emit_tiles(int64_t n)
 // first, then a look back over 32 tiles at a time to the nearest published
 // prefix (decoupled look-back, Merrill & Garland 2016; tiles are taken by
 // ticket, so a tile only waits on running blocks), then its own prefix.
-// Bounded: on timeout sets bit 2 of the flags and carries on.
+// Bounded: on timeout sets bit 2 of the flags (the caller's copy and the
+// context's record of timed-out waits, where there is one) and carries on: its
+// sums then lack some tiles, so its pairs land too early, but inside the list.
 __device__ __forceinline__ unsigned long long emit_prefix(unsigned long long *state, int tile, unsigned long long own,
-                                                          int32_t *flags, int32_t *flags_out)
+                                                          int32_t *flags_out)
 {
     const int lane = threadIdx.x & 31;
+#ifdef LUB_TESTING
+    const bool mute = tile == g_test_mute_list_tile;
+#else
+    constexpr bool mute = false;
+#endif
     unsigned long long excl = 0;
     if (tile > 0) {
-        if (lane == 0) atomicExch(state + tile, EM_AGG | own);
+        if (lane == 0 && !mute) atomicExch(state + tile, EM_AGG | own);
         long spins = 0;
         int top = tile - 1;
         while (true) {
@@ -942,12 +961,9 @@ __device__ __forceinline__ unsigned long long emit_prefix(unsigned long long *st
             const unsigned upto = stop == 32 ? 0xffffffffu : ((2u << stop) - 1u);
             if (none & upto) {
                 if (++spins > scan_tile::kSpinLimit) {
-                    if (lane == 0) {
-                        atomicOr(flags, 4);
-                        if (flags_out) {
-                            atomicOr(flags_out, 4);
-                            atomicOr(flags_out + 1, 4);
-                        }
+                    if (lane == 0 && flags_out) {
+                        atomicOr(flags_out, 4);
+                        atomicOr(flags_out + 1, 4);
                     }
                     break;
                 }
@@ -961,7 +977,7 @@ __device__ __forceinline__ unsigned long long emit_prefix(unsigned long long *st
             top -= 32;
         }
     }
-    if (lane == 0) atomicExch(state + tile, EM_PREFIX | ((excl + own) & EM_VALUE));
+    if (lane == 0 && !mute) atomicExch(state + tile, EM_PREFIX | ((excl + own) & EM_VALUE));
     return excl;
 }
 
@@ -996,13 +1012,6 @@ __global__ void __launch_bounds__(256) k_pairs_emit(const __grid_constant__ Buil
     const int tile = tile_s;
     if (tile == 0 && threadIdx.x == 0) {
         *V.d_count = need > cap ? (int32_t)(need < (int64_t)INT32_MAX ? need : (int64_t)INT32_MAX) : (int32_t)total;
-        // this build's flags, for the host-count path (before this tile
-        // publishes, so before any look-back can time out)
-        if (V.flags_out) {
-            *V.flags_out = *V.flags;
-            if (*V.flags & 4) atomicOr(V.flags_out + 1, 4);  // a timed-out wait, for lub_sync_status
-            __threadfence();
-        }
     }
     if (need > cap) return;
     // the counts of the warp's particles and their places within the warp
@@ -1044,7 +1053,7 @@ __global__ void __launch_bounds__(256) k_pairs_emit(const __grid_constant__ Buil
     }
     if (w == 0) {
         const unsigned long long ex = emit_prefix(V.scan_state + 1, tile,
-                                                  (unsigned long long)bp | (unsigned long long)bw << 31, V.flags,
+                                                  (unsigned long long)bp | (unsigned long long)bw << 31,
                                                   V.flags_out);
         if (lane == 0) prefix_s = ex;
     }
@@ -1729,3 +1738,12 @@ int launch_pairs_build_ens(lub_ctx *ctx, const PView &P, const Ens &E, const DVi
     return build_core<true>(ctx, ctx->num_sms, ctx->scratch, G, P, D, E, (const EnsGrid *)dev, prm, rmax, pi, pj, cap,
                             d_count, st, ctx->d_flags);
 }
+
+#ifdef LUB_TESTING
+// Test build only (no counterpart in the product library): the tile of the
+// list kernel that never publishes, as if its block never ran (-1: none).
+extern "C" int lub_test_mute_list_tile(int32_t tile)
+{
+    return cudaMemcpyToSymbol(g_test_mute_list_tile, &tile, sizeof(int)) == cudaSuccess ? LUB_OK : LUB_ERR_CUDA;
+}
+#endif
