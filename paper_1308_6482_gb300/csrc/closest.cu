@@ -31,6 +31,8 @@
 //     kernel, so only full warps of such pairs use the slow FP64 pipe.
 // LUB_FP64: the iterations in FP32 and float-float, the gap and the last step
 // in double (solve_ff, finish_fp64).
+#include <algorithm>
+
 #include "ff.cuh"
 #include "lub_mlp.cuh"
 #include "mlp_infer.cuh"
@@ -61,10 +63,14 @@ __device__ __forceinline__ V3<T> perp_unit(const V3<T> &n)
 // Newton ascent of g on the unit sphere from n (in/out), in precision T.
 // Step-size convergence: |s| < tol (radians), after which the last step is
 // applied.  Steps are clamped to 0.5 rad; a step that lowers g by more than
-// the rounding noise is halved (at most 12 times per solve).
-template <typename T>
+// the rounding noise is halved (at most 12 times per solve).  stop(): asked
+// twice in every iteration, ends the solve where its result is not wanted.
+struct NeverStop {
+    __device__ __forceinline__ bool operator()() const { return false; }
+};
+template <typename T, typename Stop = NeverStop>
 __device__ NewtonOut newton_sphere(const Shape<T> &si, const Shape<T> &sj, const V3<T> &d, V3<T> &n, int maxit,
-                                   T tol, T noise)
+                                   T tol, T noise, Stop stop = Stop())
 {
     n = normalized(n);  // g below assumes |n| = 1: a start off by 1e-7 would corrupt the first g
     V3<T> t1 = perp_unit(n);
@@ -73,6 +79,7 @@ __device__ NewtonOut newton_sphere(const Shape<T> &si, const Shape<T> &sj, const
     int halvings = 0;
     NewtonOut out{0, false};
     for (int it = 0; it < maxit; ++it) {
+        if (stop()) break;
         V3<T> t2 = cross(n, t1);
         T ci = dot(si.o, n), u1i = dot(si.o, t1), u2i = dot(si.o, t2);
         T cj = dot(sj.o, n), u1j = dot(sj.o, t1), u2j = dot(sj.o, t2);
@@ -89,6 +96,7 @@ __device__ NewtonOut newton_sphere(const Shape<T> &si, const Shape<T> &sj, const
             t1 = normalized(axpy(-dot(t1_acc, n), n, t1_acc));
             continue;
         }
+        if (stop()) break;
         n_acc = n;
         t1_acc = t1;
         t2_acc = t2;
@@ -663,17 +671,25 @@ __device__ __forceinline__ bool finish_fp64(const V3<double> &d, const Shape<dou
 }
 
 // the FP64 iteration itself, for the pairs that solve_ff leaves (out of line:
-// its registers are not the kernels')
+// its registers are not the kernels').  drop (if not null): bit `lane` set once
+// the result is not wanted any more.
 struct Fp64Solve {
     V3<double> n;
     double h;
     int iters, noconv;
 };
+struct StopOnBit {
+    const volatile unsigned *word;
+    int bit;
+    __device__ __forceinline__ bool operator()() const { return word && (*word >> bit & 1u); }
+};
 __device__ __noinline__ Fp64Solve solve_fp64(V3<double> d, Shape<double> si, Shape<double> sj, V3<double> n0,
-                                             double scale, int maxit)
+                                             double scale, int maxit, const volatile unsigned *drop)
 {
-    Fp64Solve r;
-    const NewtonOut o = newton_sphere<double>(si, sj, d, n0, maxit, kTolFp64, 1e-14 * scale);
+    Fp64Solve r = {};
+    const StopOnBit stop{drop, (int)(threadIdx.x & 31)};
+    const NewtonOut o = newton_sphere<double>(si, sj, d, n0, maxit, kTolFp64, 1e-14 * scale, stop);
+    if (stop()) return r;
     r.iters = o.iters;
     r.n = normalized(n0);
     r.h = dot(r.n, d) - support(si, r.n) - support(sj, r.n);
@@ -691,63 +707,86 @@ __device__ __forceinline__ V3<double> min_image_near(const DView &D, V3<double> 
     return min_image(D, d);
 }
 
-// LUB_FP64: the solve and gap of pair k
+// LUB_FP64: what pair k's solve works on
+struct Fp64Pair {
+    Shape<double> si, sj;
+    V3<double> d, start;
+    double scale;
+    float rpi, rqi, rpj, rqj;
+};
+
+// LUB_FP64: pair k up to its solve; false where there is nothing to solve
+// (invalid pairs, walls and spheres: n64, h and st are then final)
 template <bool ENS>
-__device__ __forceinline__ void closest_fp64_one(const PView &P, const DView &D0, const Ens &E, int i, int j, int k,
-                                                 const double *__restrict__ nin, size_t C, int warm, int maxit,
-                                                 V3<double> &n64, double &h, int &st, int &nit)
+__device__ __forceinline__ bool prepare_fp64(const PView &P, const DView &D0, const Ens &E, int i, int j, int k,
+                                             const double *__restrict__ nin, size_t C, int warm, Fp64Pair &a,
+                                             V3<double> &n64, double &h, int &st)
 {
     st = 0;
-    nit = 0;
     n64 = mk<double>(0, 0, 0);
     h = 0.0;
     bool alien;
     const DView &D = pair_domain<ENS>(D0, E, i, j, &alien);
     if (alien || pair_bad(P, D, i, j)) {
         st = LUB_ST_DEGENERATE;
-    } else if (j < 0) {
+        return false;
+    }
+    if (j < 0) {
         h = wall_gap(P, D, i, -1 - j, n64);
-    } else {
-        const V3<double> d = min_image_near(D, sub(load_pos(P, j), load_pos(P, i)));
-        const double dd = dot(d, d);
-        const double idl = rsqrt64(dd), dl = dd * idl;
-        if (!(dd > 0.0) || !isfinite(dd)) {
-            st = LUB_ST_DEGENERATE;
-        } else {
-            const float rpi = __ldg(P.rpar + i), rqi = __ldg(P.rperp + i);
-            const float rpj = __ldg(P.rpar + j), rqj = __ldg(P.rperp + j);
-            if (rpi == rqi && rpj == rqj) {
-                n64 = scl(idl, d);
-                h = dl - widen_bits(rpi) - widen_bits(rpj);
-            } else {
-                const Shape<double> si = load_shape<double>(P, i), sj = load_shape<double>(P, j);
-                V3<double> nn = scl(idl, d);
-                if (warm) {
-                    const V3<double> w0 = mk<double>(nin[k], nin[C + k], nin[2 * C + k]);
-                    const V3<float> wf = mk<float>(narrow_bits(w0.x), narrow_bits(w0.y), narrow_bits(w0.z));
-                    const float wl2 = dot(wf, wf);
-                    // a start on the far hemisphere falls back to the line of centres
-                    if (wl2 > 0.25f && wl2 < 4.0f && isfinite(wl2) && dot(w0, d) > 0.0) {
-                        nn = w0;
-                    }
-                }
-                const ff df[3] = {ff_split_bits(d.x), ff_split_bits(d.y), ff_split_bits(d.z)};
-                const ff oi[3] = {ff_split_bits(si.o.x), ff_split_bits(si.o.y), ff_split_bits(si.o.z)};
-                const ff oj[3] = {ff_split_bits(sj.o.x), ff_split_bits(sj.o.y), ff_split_bits(sj.o.z)};
-                const ff n0[3] = {ff_split_bits(nn.x), ff_split_bits(nn.y), ff_split_bits(nn.z)};
-                ff nf[3];
-                bool done = solve_ff(df, oi, oj, rqi, rpi, rqj, rpj, n0, maxit, nf, nit);
-                if (done) done = finish_fp64(d, si, sj, nf, n64, h);
-                if (!done) {
-                    const double scale = dl + (double)fmaxf(rpi, rqi) + (double)fmaxf(rpj, rqj);
-                    const Fp64Solve r = solve_fp64(d, si, sj, nn, scale, maxit);
-                    n64 = r.n;
-                    h = r.h;
-                    nit = r.iters;
-                    if (r.noconv) st |= LUB_ST_NOCONV;
-                }
-            }
-        }
+        return false;
+    }
+    a.d = min_image_near(D, sub(load_pos(P, j), load_pos(P, i)));
+    const double dd = dot(a.d, a.d);
+    const double idl = rsqrt64(dd), dl = dd * idl;
+    if (!(dd > 0.0) || !isfinite(dd)) {
+        st = LUB_ST_DEGENERATE;
+        return false;
+    }
+    a.rpi = __ldg(P.rpar + i), a.rqi = __ldg(P.rperp + i);
+    a.rpj = __ldg(P.rpar + j), a.rqj = __ldg(P.rperp + j);
+    if (a.rpi == a.rqi && a.rpj == a.rqj) {
+        n64 = scl(idl, a.d);
+        h = dl - widen_bits(a.rpi) - widen_bits(a.rpj);
+        return false;
+    }
+    a.si = load_shape<double>(P, i), a.sj = load_shape<double>(P, j);
+    a.start = scl(idl, a.d);
+    if (warm) {
+        const V3<double> w0 = mk<double>(nin[k], nin[C + k], nin[2 * C + k]);
+        const V3<float> wf = mk<float>(narrow_bits(w0.x), narrow_bits(w0.y), narrow_bits(w0.z));
+        const float wl2 = dot(wf, wf);
+        // a start on the far hemisphere falls back to the line of centres
+        if (wl2 > 0.25f && wl2 < 4.0f && isfinite(wl2) && dot(w0, a.d) > 0.0) a.start = w0;
+    }
+    a.scale = dl + (double)fmaxf(a.rpi, a.rqi) + (double)fmaxf(a.rpj, a.rqj);
+    return true;
+}
+
+// the solve in FP32 and float-float with its FP64 last step; false: left to solve_fp64
+__device__ __forceinline__ bool solve_mostly_ff(const Fp64Pair &a, int maxit, V3<double> &n64, double &h, int &nit)
+{
+    const ff df[3] = {ff_split_bits(a.d.x), ff_split_bits(a.d.y), ff_split_bits(a.d.z)};
+    const ff oi[3] = {ff_split_bits(a.si.o.x), ff_split_bits(a.si.o.y), ff_split_bits(a.si.o.z)};
+    const ff oj[3] = {ff_split_bits(a.sj.o.x), ff_split_bits(a.sj.o.y), ff_split_bits(a.sj.o.z)};
+    const ff n0[3] = {ff_split_bits(a.start.x), ff_split_bits(a.start.y), ff_split_bits(a.start.z)};
+    ff nf[3];
+    return solve_ff(df, oi, oj, a.rqi, a.rpi, a.rqj, a.rpj, n0, maxit, nf, nit) && finish_fp64(a.d, a.si, a.sj, nf, n64, h);
+}
+
+// LUB_FP64: the solve and gap of pair k
+template <bool ENS>
+__device__ __forceinline__ void closest_fp64_one(const PView &P, const DView &D0, const Ens &E, int i, int j, int k,
+                                                 const double *__restrict__ nin, size_t C, int warm, int maxit,
+                                                 V3<double> &n64, double &h, int &st, int &nit)
+{
+    Fp64Pair a;
+    nit = 0;
+    if (prepare_fp64<ENS>(P, D0, E, i, j, k, nin, C, warm, a, n64, h, st) && !solve_mostly_ff(a, maxit, n64, h, nit)) {
+        const Fp64Solve r = solve_fp64(a.d, a.si, a.sj, a.start, a.scale, maxit, nullptr);
+        n64 = r.n;
+        h = r.h;
+        nit = r.iters;
+        if (r.noconv) st |= LUB_ST_NOCONV;
     }
     if (!(st & LUB_ST_DEGENERATE) && h <= 0.0) st |= LUB_ST_OVERLAP;
 }
@@ -946,6 +985,77 @@ __global__ void __launch_bounds__(128) k_closest_fp64(PView P, const __grid_cons
         closest_fp64_one<ENS>(P, D0, E, __ldg(pi + k), __ldg(pj + k), k, nout, C, warm, maxit, n64, h, st, nit);
         store_pair(nout, gap, status, iters, C, k, n64, h, st, nit);
     }
+}
+
+// The same for short lists (arrays of up to kRaceCap pairs), with two warps per 32
+// pairs: the second warp runs the FP64 iteration from the start and drops the
+// pairs that the first has solved, so that those it leaves (0.1 to 0.5 % from the
+// cold start) have their FP64 solve half done.  A short list takes as long as its
+// slowest warp, and up to kRaceMax pairs its second warps run on quarters of SMs
+// that are idle otherwise.  The results are those of the other kernel, bit by bit
+// (a pair's result must not depend on the list it is in).  Measured, with one
+// solve after the other and with both at once: 1,000 cold pairs 50 to 59 us and
+// 34 to 46, 3,000 58 to 60 and 42 to 44, 6,000 60 to 70 and 45 to 48; with the
+// network's start 4,096 pairs 50 and 39.  Where no pair is left the second warp
+// costs some 3 us (100 pairs 23 to 26), so lists too short to have one, mostly, do
+// without, as do longer ones.
+constexpr int kRaceCold = 128, kRaceWarm = 512;
+constexpr int kRaceMax = 9728;  // two warps for every 32 pairs on 152 x 4 quarters
+constexpr int kRaceCap = 24576;
+
+template <bool ENS>
+__global__ void __launch_bounds__(64) k_closest_fp64_race(PView P, const __grid_constant__ DView D0, Ens E,
+                                                          const int32_t *__restrict__ pi,
+                                                          const int32_t *__restrict__ pj,
+                                                          const int32_t *__restrict__ d_count, int32_t cap,
+                                                          double *__restrict__ nout, double *__restrict__ gap,
+                                                          uint8_t *__restrict__ status, uint8_t *__restrict__ iters,
+                                                          int maxit, int warm)
+{
+    __shared__ unsigned solved_s;  // the lanes whose pair needs no FP64 iteration
+    __shared__ Fp64Solve res_s[32];
+    const int count = pair_count(d_count, cap);
+    const size_t C = (size_t)cap;
+    const bool race = count >= (warm ? kRaceWarm : kRaceCold) && count <= kRaceMax;  // (the same for every block)
+    const bool second = race && threadIdx.x >= 32;
+    const int lane = threadIdx.x & 31;
+    const int k = race ? blockIdx.x * 32 + lane : blockIdx.x * 64 + threadIdx.x;  // (the grid covers the list)
+    volatile unsigned *const solved = &solved_s;
+    if (race) {
+        if (threadIdx.x == 0) *solved = 0;
+        __syncthreads();
+    }
+    Fp64Pair a;
+    V3<double> n64;
+    double h;
+    int st, nit = 0;
+    bool left = false;  // needs the FP64 iteration
+    if (k < count) {
+        left = prepare_fp64<ENS>(P, D0, E, __ldg(pi + k), __ldg(pj + k), k, nout, C, warm, a, n64, h, st);
+        if (left && !second) left = !solve_mostly_ff(a, maxit, n64, h, nit);
+    }
+    if (race && !second) {
+        const unsigned m = __ballot_sync(0xffffffffu, !left);
+        if (lane == 0) *solved = m;
+    }
+    Fp64Solve r = {};
+    if (left && second == race) {
+        r = solve_fp64(a.d, a.si, a.sj, a.start, a.scale, maxit, race ? solved : nullptr);
+        if (race) res_s[lane] = r;
+    }
+    if (race) {
+        __syncthreads();
+        if (left && !second) r = res_s[lane];
+    }
+    if (second || k >= count) return;
+    if (left) {
+        n64 = r.n;
+        h = r.h;
+        nit = r.iters;
+        if (r.noconv) st |= LUB_ST_NOCONV;
+    }
+    if (!(st & LUB_ST_DEGENERATE) && h <= 0.0) st |= LUB_ST_OVERLAP;
+    store_pair(nout, gap, status, iters, C, k, n64, h, st, nit);
 }
 
 // LUB_WARM_MLP in mixed precision: the FP64 solves of the work list start
@@ -1276,8 +1386,13 @@ int launch_closest_t(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E,
     } else {
         const Shape2 sh = tuned_shape(ctx, LUB_TUNE_CLOSEST_FP64, cap);
         lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
-        (void)launch_pdl(k_closest_fp64<ENS>, sh.grid, sh.block, 0, st, P, D, E, pi, pj, d_count, cap, n, gap, status,
-                         iters, prm.max_newton, warm);
+        const int whole = (cap + 63) / 64, twice = (std::min(cap, kRaceMax) + 31) / 32;
+        if (cap <= kRaceCap)  // (a plain launch spreads the blocks over all SMs)
+            k_closest_fp64_race<ENS><<<std::max(whole, twice), 64, 0, st>>>(P, D, E, pi, pj, d_count, cap, n, gap,
+                                                                            status, iters, prm.max_newton, warm);
+        else
+            (void)launch_pdl(k_closest_fp64<ENS>, sh.grid, sh.block, 0, st, P, D, E, pi, pj, d_count, cap, n, gap,
+                             status, iters, prm.max_newton, warm);
         lub_trace_mark(ctx, LUB_TRACE_CLOSEST, st);
     }
     return lub_check_cuda(ctx, cudaGetLastError(), "k_closest launch");
