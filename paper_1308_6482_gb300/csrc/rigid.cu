@@ -81,10 +81,12 @@ __global__ void k_rigid_step(int n, double *__restrict__ x, double *__restrict__
         const V3<double> wm = inertia_apply(o, jpar, jperp, L);
         // q <- exp(dt wm / 2) q: with t the squared half angle, cos(sqrt t) and
         // sin(sqrt t) / sqrt t as series in t (the first term left out is
-        // below 2^-66 of the sum up to t = 0.04), beyond it by the functions
+        // below 2^-66 of the sum up to t = 0.04), beyond it by the functions; a
+        // rate that is not a number turns nothing (the orientation stays)
         const double hdt = 0.5 * dt;
         const double t = hdt * hdt * dot(wm, wm);
         double r0, sc;
+        V3<double> turn = wm;
         if (t <= 0.04) {
             r0 = fma(t, 1.0 / 479001600.0, -1.0 / 3628800.0);
             r0 = fma(t, r0, 1.0 / 40320.0);
@@ -98,13 +100,17 @@ __global__ void k_rigid_step(int n, double *__restrict__ x, double *__restrict__
             sc = fma(t, sc, 1.0 / 120.0);
             sc = fma(t, sc, -1.0 / 6.0);
             sc = fma(t, sc, 1.0);
-        } else {
+        } else if (t > 0.04) {
             const double h = sqrt(t);
             r0 = cos(h);
             sc = sin(h) / h;
+        } else {
+            r0 = 1.0;
+            sc = 0.0;
+            turn = mk<double>(0.0, 0.0, 0.0);
         }
         const double s = hdt * sc;
-        const double r1 = s * wm.x, r2 = s * wm.y, r3 = s * wm.z;
+        const double r1 = s * turn.x, r2 = s * turn.y, r3 = s * turn.z;
         const double n0 = r0 * q0 - r1 * q1 - r2 * q2 - r3 * q3;
         const double n1 = r0 * q1 + r1 * q0 + r2 * q3 - r3 * q2;
         const double n2 = r0 * q2 - r1 * q3 + r2 * q0 + r3 * q1;

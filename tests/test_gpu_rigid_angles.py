@@ -44,3 +44,27 @@ def test_half_angles_on_both_sides_of_the_series(prec, dt):
     size = np.linalg.norm(w.astype(np.float64), axis=1)
     for k in ("wx", "wy", "wz"):
         assert np.all(np.abs(got[k] - ref[k]) <= (2.0 ** -24 + 1e-12) * size * 3.0), k
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_rates_that_are_not_numbers_leave_the_orientation(prec):
+    import torch
+
+    import paper_1308_6482_gb300 as lub
+    parts, dom, _, _ = gen.pair_stream(20, seed=61, kind="aspect")
+    parts = {k: np.array(v) for k, v in parts.items()}
+    parts["wx"][3] = parts["wz"][4] = np.nan
+    pl = lub.Pipeline(parts, dom, gpu_params(prec), capacity=1024)
+    pl.force.zero_()
+    pl.torque.zero_()
+    n = pl.n
+    pl.torque[n + 7] = float("nan")   # the torque's y component on particle 7
+    pl.rigid_step(1.0, 0.1)
+    torch.cuda.synchronize()
+    got = {k: v.cpu().numpy() for k, v in pl.P.t.items()}
+    odd = np.array([3, 4, 7])
+    for k in ("qw", "qx", "qy", "qz"):
+        assert np.isfinite(got[k]).all()
+        np.testing.assert_allclose(got[k][odd], parts[k][odd], rtol=0, atol=2.0 ** -23)
+    for k in ("wx", "wy", "wz"):
+        assert np.isnan(got[k][odd]).all() and np.isfinite(np.delete(got[k], odd)).all()
