@@ -677,9 +677,10 @@ class Pipeline:
         """One correction step: the pair build, then the per-pair work in one
         of three forms: "calls" (closest points, resistance, apply), "merged"
         (closest points, then resistance + scatter in one pass) or "fused"
-        (one lub_correct call: in FP64 all three in one pass, in mixed
-        precision the merged kernels on one set of particle records;
-        fused=True is the same).  deterministic needs
+        (one lub_correct call: all three in one pass, or in mixed precision,
+        for pair arrays of more than 1.6 million and with the gated network,
+        the merged kernels on one set of particle records; fused=True is the
+        same).  deterministic needs
         "calls".  With warm_start = LUB_WARM_PREVIOUS the normals are carried
         over from the step before (keep_previous is called at the end of
         every step).  pair_forces=False: the fused form writes no per-pair

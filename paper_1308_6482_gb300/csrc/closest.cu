@@ -189,13 +189,17 @@ constexpr int kNoEntry = 0x7fffffff;
 // 15 us in all; but its 64 registers spill where those of the two kernels (64
 // and 72) do not, which costs some 12 us per million pairs.  Measured: 60.4 ->
 // 55.8 us (step, 65k pairs), 238 -> 231 us (0.6M pairs, ensemble), 820 -> 864
-// us (4.4M pairs): level near 1.3 million pairs, and capacities are usually a
-// third above the count.
+// us (4.4M pairs).  Both forms on the same lists, one pass and two kernels: 0.9M
+// pairs of a suspension 118 and 127 us (arrays for 1.6M), 1.2M 160 and 158, 1.4M
+// 184 and 179, 1.6M 199 and 198; fresh pairs level within 1 % from 1.1M to 1.6M.
+// (The count is known on the device only.  A list far shorter than its arrays
+// gains from the one pass too, so arrays beyond the line forgo it: 0.5M pairs 85
+// and 102 us in arrays on either side.)
 constexpr int kFusedMax = 1600000;
 // The one-pass kernel's blocks of 128 threads per SM: with few pairs (capacity
-// up to kFusedFew) 4, its registers unlimited, since the list then fills the
-// GPU about once and each warp's own chain is what counts; otherwise 8 (64
-// registers, some spilled), for the warps in flight.  Measured at 4, 5, 6, 7,
+// up to kFusedFew) 4, which leaves it 128 registers (it takes 109), since the
+// list then fills the GPU about once and each warp's own chain is what counts;
+// otherwise 8 (64 registers, some spilled), for the warps in flight.  Measured at 4, 5, 6, 7,
 // 8: step at 32,768 particles (65k pairs) 49.4, 51.3, 51.3, 51.5, - us; at
 // 131,072 (0.56M pairs, temporal start) 170, 167, 164, 162, 162; ensemble of
 // 262,144 particles 223, 216, 213, 211, 208.
@@ -665,7 +669,8 @@ __device__ __forceinline__ bool finish_fp64(const V3<double> &d, const Shape<dou
     const float s1 = (P22 * G1 - P12 * G2) * idet, s2 = (P11 * G2 - P12 * G1) * idet;
     const V3<float> st = axpy(s1, t1, scl(s2, t2));
     n64 = mk<double>(n.x + widen_bits(st.x), n.y + widen_bits(st.y), n.z + widen_bits(st.z));
-    n64 = scl(sc, n64);  // (the step is normal to n: |n64| = |n| to 1e-22)
+    // (|n64| = 1 to rounding: the step, below 1e-9, lies along FP32 tangents, normal to n to some 1e-7)
+    n64 = scl(sc, n64);
     const V3<float> df = mk<float>(narrow_bits(d.x), narrow_bits(d.y), narrow_bits(d.z));
     return s1 * s1 + s2 * s2 < 1e-18f && dot(nv, df) > 1e-3f * sqrtf(dot(df, df)) && isfinite(narrow_bits(h));
 }
@@ -1306,8 +1311,8 @@ int launch_particles_ff(lub_ctx *ctx, const PView &P, float2 *out, cudaStream_t 
 
 namespace {
 
-// The work list of the mixed mode in the context scratch: counters [entries,
-// unused, queue 0, queue 1] and cap entries; with nh and status_in (the
+// The work list of the mixed mode in the context scratch: its length (the first
+// of four words) and cap entries; with nh and status_in (the
 // fused pass), also the hand-over of normals and gaps in float-float (32
 // bytes a pair, store_nh) and a status array for callers that pass none;
 // with P, the per-call particle table (pff: 80 bytes per particle).
@@ -1411,11 +1416,10 @@ int launch_correct_t(lub_ctx *ctx, const PView &P, const DView &D, const Ens &E,
     }
     if (cap == 0) return LUB_OK;
     if (prm.precision == LUB_MIXED) {
-        // the kernels of lub_closest_points, then those of lub_resistance_apply
-        // on the same per-call particle records (built once; their kernel also
-        // clears the sums unless accumulate is set)
+        // on one set of per-call particle records (their kernel also clears the
+        // sums unless accumulate is set): one pass over the pairs, or the kernels
+        // of lub_closest_points and then those of lub_resistance_apply
         if (prm.warm_start != LUB_WARM_MLP && cap <= kFusedMax) {
-            // small lists: the records, then one pass over the pairs
             int warm = 0;
             if ((rc = start_normals(ctx, P, D, E, prm, pi, pj, d_count, cap, n, st, &warm))) return rc;
             if ((rc = lub_ensure_scratch(ctx, particles_ff_bytes(P.n)))) return rc;

@@ -13,10 +13,11 @@
 //             start (the support points of i along d^ and of j along -d^), so
 //             a zero output gives back the cold start n0 = d^ exactly and the
 //             network only learns a small, continuous correction;
-//   training  FP32 kernels: linear forward (optionally + GELU), a weighted
-//             squared error with the azimuth differences wrapped to (-pi, pi],
-//             backward through the layers, Adam.  Parameters packed [W1 | b1 | W2 | b2 | W3 | b3]
-//             with W row-major [out][in].
+//   training  in FP32: one kernel for forward, loss (a weighted squared error
+//             with the azimuth differences wrapped to (-pi, pi]) and backward,
+//             tile by tile with partial gradients per block, the partials' sum,
+//             Adam.  Parameters packed [W1 | b1 | W2 | b2 | W3 | b3] with W
+//             row-major [out][in].
 //   inference BF16 weights and activations on the tensor cores (mma.sync
 //             m16n8k16, FP32 accumulate), one warp per 32 pairs with the
 //             activations in registers; the predicted (p, q) give the outward
@@ -811,9 +812,12 @@ static int launch_train(lub_ctx *ctx, int nblk, const float *params, const float
 int launch_mlp_forward_backward(lub_ctx *ctx, const float *params, const float *x, const float *tgt,
                                 const float *wgt, int M, float *grads, float *work, float *loss_rows, cudaStream_t st)
 {
-    // rows per block: the fewest (in eights) that cover the batch in one wave
-    // of one block per SM, and whose partial gradients fit the caller's
-    // scratch; larger batches take tiles of 64 rows in turns
+    // rows per block: the fewest of 8, 16, 32, 48, 56, 64 that cover the batch in
+    // one wave of one block per SM, and whose partial gradients fit the caller's
+    // scratch; larger batches take tiles of 64 rows in turns.  The scratch grows
+    // with the batch, a block's partial takes that of 24.1 samples: so 8 or 16
+    // rows come about for batches of at most 8 and 16 samples, and 32 rows serve
+    // nearly all from 49 to 4,864 (21 to 25 us)
     const int sms = ctx ? ctx->num_sms : 152;
     const int64_t room = (int64_t)M * LUB_MLP_WORK_PER_SAMPLE / LUB_MLP_PARAMS;
     const int most = (int)(room < 1 ? 1 : (room < sms ? room : sms));
