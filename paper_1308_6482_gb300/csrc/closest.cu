@@ -676,23 +676,17 @@ __device__ __forceinline__ bool finish_fp64(const V3<double> &d, const Shape<dou
 }
 
 // the FP64 iteration itself, for the pairs that solve_ff leaves (out of line:
-// its registers are not the kernels').  drop (if not null): bit `lane` set once
-// the result is not wanted any more.
+// its registers are not the kernels')
 struct Fp64Solve {
     V3<double> n;
     double h;
     int iters, noconv;
 };
-struct StopOnBit {
-    const volatile unsigned *word;
-    int bit;
-    __device__ __forceinline__ bool operator()() const { return word && (*word >> bit & 1u); }
-};
-__device__ __noinline__ Fp64Solve solve_fp64(V3<double> d, Shape<double> si, Shape<double> sj, V3<double> n0,
-                                             double scale, int maxit, const volatile unsigned *drop)
+template <typename Stop>
+__device__ __forceinline__ Fp64Solve solve_fp64_body(V3<double> d, const Shape<double> &si, const Shape<double> &sj,
+                                                     V3<double> n0, double scale, int maxit, Stop stop)
 {
     Fp64Solve r = {};
-    const StopOnBit stop{drop, (int)(threadIdx.x & 31)};
     const NewtonOut o = newton_sphere<double>(si, sj, d, n0, maxit, kTolFp64, 1e-14 * scale, stop);
     if (stop()) return r;
     r.iters = o.iters;
@@ -700,6 +694,22 @@ __device__ __noinline__ Fp64Solve solve_fp64(V3<double> d, Shape<double> si, Sha
     r.h = dot(r.n, d) - support(si, r.n) - support(sj, r.n);
     r.noconv = !o.converged || !(dot(r.n, d) > 0.0) || !isfinite(r.h);
     return r;
+}
+__device__ __noinline__ Fp64Solve solve_fp64(V3<double> d, Shape<double> si, Shape<double> sj, V3<double> n0,
+                                             double scale, int maxit)
+{
+    return solve_fp64_body(d, si, sj, n0, scale, maxit, NeverStop());
+}
+// the same, ended once this lane's bit of `drop` is set (the result is not wanted any more)
+struct StopOnBit {
+    const volatile unsigned *word;
+    int bit;
+    __device__ __forceinline__ bool operator()() const { return *word >> bit & 1u; }
+};
+__device__ __noinline__ Fp64Solve solve_fp64_until(V3<double> d, Shape<double> si, Shape<double> sj, V3<double> n0,
+                                                   double scale, int maxit, const volatile unsigned *drop)
+{
+    return solve_fp64_body(d, si, sj, n0, scale, maxit, StopOnBit{drop, (int)(threadIdx.x & 31)});
 }
 
 // minimum image of r_j - r_i, skipping the FP64 image shift of an axis where
@@ -712,7 +722,10 @@ __device__ __forceinline__ V3<double> min_image_near(const DView &D, V3<double> 
     return min_image(D, d);
 }
 
-// LUB_FP64: what pair k's solve works on
+// The parts of closest_fp64_one for the kernel of short lists, which has a warp
+// of its own for the FP64 iteration (its other use stays in one piece: split up,
+// the one-pass kernel of 20,011 spheroids took 298 us instead of 258).
+// What pair k's solve works on:
 struct Fp64Pair {
     Shape<double> si, sj;
     V3<double> d, start;
@@ -720,8 +733,8 @@ struct Fp64Pair {
     float rpi, rqi, rpj, rqj;
 };
 
-// LUB_FP64: pair k up to its solve; false where there is nothing to solve
-// (invalid pairs, walls and spheres: n64, h and st are then final)
+// pair k up to its solve; false where there is nothing to solve (invalid pairs,
+// walls and spheres: n64, h and st are then final)
 template <bool ENS>
 __device__ __forceinline__ bool prepare_fp64(const PView &P, const DView &D0, const Ens &E, int i, int j, int k,
                                              const double *__restrict__ nin, size_t C, int warm, Fp64Pair &a,
@@ -784,14 +797,57 @@ __device__ __forceinline__ void closest_fp64_one(const PView &P, const DView &D0
                                                  const double *__restrict__ nin, size_t C, int warm, int maxit,
                                                  V3<double> &n64, double &h, int &st, int &nit)
 {
-    Fp64Pair a;
+    st = 0;
     nit = 0;
-    if (prepare_fp64<ENS>(P, D0, E, i, j, k, nin, C, warm, a, n64, h, st) && !solve_mostly_ff(a, maxit, n64, h, nit)) {
-        const Fp64Solve r = solve_fp64(a.d, a.si, a.sj, a.start, a.scale, maxit, nullptr);
-        n64 = r.n;
-        h = r.h;
-        nit = r.iters;
-        if (r.noconv) st |= LUB_ST_NOCONV;
+    n64 = mk<double>(0, 0, 0);
+    h = 0.0;
+    bool alien;
+    const DView &D = pair_domain<ENS>(D0, E, i, j, &alien);
+    if (alien || pair_bad(P, D, i, j)) {
+        st = LUB_ST_DEGENERATE;
+    } else if (j < 0) {
+        h = wall_gap(P, D, i, -1 - j, n64);
+    } else {
+        const V3<double> d = min_image_near(D, sub(load_pos(P, j), load_pos(P, i)));
+        const double dd = dot(d, d);
+        const double idl = rsqrt64(dd), dl = dd * idl;
+        if (!(dd > 0.0) || !isfinite(dd)) {
+            st = LUB_ST_DEGENERATE;
+        } else {
+            const float rpi = __ldg(P.rpar + i), rqi = __ldg(P.rperp + i);
+            const float rpj = __ldg(P.rpar + j), rqj = __ldg(P.rperp + j);
+            if (rpi == rqi && rpj == rqj) {
+                n64 = scl(idl, d);
+                h = dl - widen_bits(rpi) - widen_bits(rpj);
+            } else {
+                const Shape<double> si = load_shape<double>(P, i), sj = load_shape<double>(P, j);
+                V3<double> nn = scl(idl, d);
+                if (warm) {
+                    const V3<double> w0 = mk<double>(nin[k], nin[C + k], nin[2 * C + k]);
+                    const V3<float> wf = mk<float>(narrow_bits(w0.x), narrow_bits(w0.y), narrow_bits(w0.z));
+                    const float wl2 = dot(wf, wf);
+                    // a start on the far hemisphere falls back to the line of centres
+                    if (wl2 > 0.25f && wl2 < 4.0f && isfinite(wl2) && dot(w0, d) > 0.0) {
+                        nn = w0;
+                    }
+                }
+                const ff df[3] = {ff_split_bits(d.x), ff_split_bits(d.y), ff_split_bits(d.z)};
+                const ff oi[3] = {ff_split_bits(si.o.x), ff_split_bits(si.o.y), ff_split_bits(si.o.z)};
+                const ff oj[3] = {ff_split_bits(sj.o.x), ff_split_bits(sj.o.y), ff_split_bits(sj.o.z)};
+                const ff n0[3] = {ff_split_bits(nn.x), ff_split_bits(nn.y), ff_split_bits(nn.z)};
+                ff nf[3];
+                bool done = solve_ff(df, oi, oj, rqi, rpi, rqj, rpj, n0, maxit, nf, nit);
+                if (done) done = finish_fp64(d, si, sj, nf, n64, h);
+                if (!done) {
+                    const double scale = dl + (double)fmaxf(rpi, rqi) + (double)fmaxf(rpj, rqj);
+                    const Fp64Solve r = solve_fp64(d, si, sj, nn, scale, maxit);
+                    n64 = r.n;
+                    h = r.h;
+                    nit = r.iters;
+                    if (r.noconv) st |= LUB_ST_NOCONV;
+                }
+            }
+        }
     }
     if (!(st & LUB_ST_DEGENERATE) && h <= 0.0) st |= LUB_ST_OVERLAP;
 }
@@ -1045,8 +1101,10 @@ __global__ void __launch_bounds__(64) k_closest_fp64_race(PView P, const __grid_
     }
     Fp64Solve r = {};
     if (left && second == race) {
-        r = solve_fp64(a.d, a.si, a.sj, a.start, a.scale, maxit, race ? solved : nullptr);
-        if (race) res_s[lane] = r;
+        if (race)
+            res_s[lane] = solve_fp64_until(a.d, a.si, a.sj, a.start, a.scale, maxit, solved);
+        else
+            r = solve_fp64(a.d, a.si, a.sj, a.start, a.scale, maxit);
     }
     if (race) {
         __syncthreads();
