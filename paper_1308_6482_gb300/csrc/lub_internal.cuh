@@ -227,14 +227,12 @@ __device__ __forceinline__ V3<T> axpy(T s, const V3<T> &a, const V3<T> &b)  // s
 // The double of a float, exactly.
 __device__ __forceinline__ double widen_bits(float f)
 {
-    const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
-    unsigned hi = (m >> 3) + (m < 0x7f800000u ? 0x38000000u : 0x70000000u);
-    unsigned lo = b << 29;
-    if (m < 0x00800000u) {  // zero, or subnormal: as a normal float 2^24 times as large
-        const unsigned g = __float_as_uint(__fmul_rn(__uint_as_float(m), 0x1p24f));
-        hi = g ? (g >> 3) + 0x38000000u - (24u << 20) : 0u;
-        lo = g << 29;
-    }
+    const unsigned b = __float_as_uint(f);
+    const bool sub = (b & 0x7f800000u) == 0u;  // zero or subnormal: as a float 2^24 times as large
+    const unsigned m = __float_as_uint(sub ? __fmul_rn(f, 0x1p24f) : f) & 0x7fffffffu;
+    unsigned hi = (m >> 3) + (m < 0x7f800000u ? 0x38000000u : 0x70000000u) - (sub ? 24u << 20 : 0u);
+    unsigned lo = m << 29;
+    if (m == 0u) hi = 0u;
     return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo);
 }
 
