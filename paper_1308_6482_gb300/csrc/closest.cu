@@ -1059,8 +1059,8 @@ __global__ void __launch_bounds__(128) k_closest_fp64(PView P, const __grid_cons
 // 34 to 46, 3,000 58 to 60 and 42 to 44, 6,000 60 to 70 and 45 to 48; with the
 // network's start 4,096 pairs 50 and 39.  Where no pair is left the second warp
 // costs some 3 us (100 pairs 23 to 26), so lists too short to have one, mostly, do
-// without, as do longer ones.
-constexpr int kRaceCold = 128, kRaceWarm = 512;
+// without (fewer are left from the network's start), as do longer ones.
+constexpr int kRaceCold = 128, kRaceWarm = 2048;
 constexpr int kRaceMax = 9728;  // two warps for every 32 pairs on 152 x 4 quarters
 constexpr int kRaceCap = 24576;
 

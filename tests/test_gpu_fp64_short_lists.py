@@ -30,7 +30,7 @@ def test_the_same_pairs_in_short_and_long_lists(kind, maxit, warm):
         d /= np.maximum(np.linalg.norm(d, axis=1, keepdims=True), 1e-9)
         start = d + 0.1 * np.random.default_rng(3).normal(size=d.shape)
     runs = {m: solve(parts, dom, pi[:m], pj[:m], start[:m] if warm else None, max_newton=maxit)
-            for m in (SHORT + 1, SHORT, TWO + 1, TWO, 513, 512, 511, 128, 127, 33, 1)}
+            for m in (SHORT + 1, SHORT, TWO + 1, TWO, 2048, 2047, 513, 128, 127, 33, 1)}
     ref = runs[SHORT + 1]
     for m, r in runs.items():
         for f in ("n", "h", "iters", "status"):
