@@ -512,7 +512,8 @@ int lub_random_motion(lub_ctx *ctx, const lub_particles *p, uint64_t seed, int64
  * ------------------------------------------------------------------------- */
 #define LUB_TUNE_CLOSEST_MIXED 0   /* lub_closest_points, LUB_MIXED, FP32 stage; lub_correct's one pass */
 #define LUB_TUNE_CLOSEST_REFINE 1  /* lub_closest_points, LUB_MIXED, work list of FP64 solves */
-#define LUB_TUNE_CLOSEST_FP64 2    /* lub_closest_points, LUB_FP64 */
+#define LUB_TUNE_CLOSEST_FP64 2    /* lub_closest_points, LUB_FP64, arrays of more than 24,576 pairs; lub_correct in
+                                      LUB_FP64 */
 #define LUB_TUNE_RESISTANCE 3      /* lub_resistance, lub_resistance_apply (and so
                                       lub_correct's two-kernel form) */
 #define LUB_TUNE_APPLY 4           /* lub_apply, atomic form */

@@ -1062,7 +1062,6 @@ __global__ void __launch_bounds__(128) k_closest_fp64(PView P, const __grid_cons
 // without (fewer are left from the network's start), as do longer ones.
 constexpr int kRaceCold = 128, kRaceWarm = 2048;
 constexpr int kRaceMax = 9728;  // two warps for every 32 pairs on 152 x 4 quarters
-constexpr int kRaceCap = 24576;
 
 template <bool ENS>
 __global__ void __launch_bounds__(64) k_closest_fp64_race(PView P, const __grid_constant__ DView D0, Ens E,

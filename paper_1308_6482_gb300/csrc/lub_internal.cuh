@@ -547,6 +547,10 @@ constexpr TuneDefault kTuneDefaults[LUB_TUNE_COUNT] = {
     {256, 32, 256},  // LUB_TUNE_APPLY
     {128, 32, 256},  // LUB_TUNE_SWEEP (the autotuner's choice at 1M particles)
 };
+// arrays of up to this many pairs: lub_closest_points in LUB_FP64 takes the kernel
+// of short lists (closest.cu), whose shape is its own
+constexpr int kRaceCap = 24576;
+
 inline Shape2 tuned_shape(const lub_ctx *ctx, int id, int64_t work)
 {
     int block = kTuneDefaults[id].block, per_sm = kTuneDefaults[id].per_sm;

@@ -104,7 +104,13 @@ int lub_autotune(lub_ctx *ctx, const lub_particles *p, const lub_domain *dom, co
         const int id = ids[q];
         float best = 1e30f;
         int bb = 0, bp = 0;
-        for (int block : blocks_of(id)) {
+        // (short FP64 lists are solved by a kernel of fixed shape: the default, for lub_correct)
+        const bool fixed = id == LUB_TUNE_CLOSEST_FP64 && capacity <= kRaceCap;
+        if (fixed) {
+            bb = kTuneDefaults[id].block;
+            bp = kTuneDefaults[id].per_sm;
+        }
+        for (int block : fixed ? std::vector<int>() : blocks_of(id)) {
             for (int per_sm : kBlocksPerSm) {
                 if (block * per_sm > 32768) continue;  // 16 waves of resident threads: as good as any larger grid
                 // the sweep runs one thread per item: its grid follows from the block

@@ -38,3 +38,12 @@ def test_the_same_pairs_in_short_and_long_lists(kind, maxit, warm):
     ok = (odd[:513] != 5) & (odd[:513] != 11)
     r = {f: v[ok] for f, v in runs[513].items() if f in ("n", "h", "iters", "status")}
     check(parts, dom, pi[:513][ok], pj[:513][ok], r, start[:513][ok] if warm else None, maxit)
+
+
+@pytest.mark.parametrize("capacity", [SHORT, SHORT + 1])
+def test_the_autotuner_keeps_the_default_where_the_shape_is_fixed(capacity):
+    import paper_1308_6482_gb300 as lub
+    parts, dom = gen.config_mixed_suspension(N=1000, phi=0.25, seed=4)
+    pl = lub.Pipeline(parts, dom, lub.default_params(precision="fp64"), capacity=capacity)
+    shape = pl.autotune(reps=1)["closest_fp64"]
+    assert shape == (64, 256) if capacity <= SHORT else shape[0] in (64, 128)
